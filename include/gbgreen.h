@@ -12,13 +12,17 @@
  * the GPU to Green's-function outputs (local DOS, density-matrix and
  * energy-density elements on the sparsity pattern, local charge and energy).
  *
- * Solver: one seed Krylov space of A = S^{-1} H built by a conjugate
- * orthogonal CG (COCG) in the S-bilinear form, shared by every shift through
- * the collinear-residual recurrence.  S^{-1} is applied exactly by a
- * block-bidiagonal Cholesky factor of S where S's half-bandwidth is at most 63
- * (chains), else by an inner block-Jacobi-preconditioned iteration (CG, or
- * Chebyshev in the mixed path).  The paper defers the method's details to its
- * references; the recurrences used are the standard shifted COCG ones.
+ * Solver: one Krylov space of A = S^{-1} H per right-hand side, shared by
+ * every shift.  Its basis is real (H, S and e_j are) and comes from the
+ * three-term recurrence in the S inner product; each shift's solution is the
+ * Galerkin one, its residual a polynomial in the shift.  Calls that name a seed
+ * shift or ask for panels of one or two columns build the same space by a
+ * conjugate orthogonal CG (COCG) in the S-bilinear form with that seed.
+ * S^{-1} is applied exactly by a block-bidiagonal Cholesky factor of S where
+ * S's half-bandwidth is at most 63 (chains), else by an inner
+ * block-Jacobi-preconditioned iteration (CG, or Chebyshev in the mixed path).
+ * The paper defers the method's details to its references; the recurrences
+ * used are the standard ones.
  *
  * Conventions for every entry point:
  *   - Return value: GB_OK (0) or a negative gb_status; gb_last_error() gives a
@@ -189,7 +193,8 @@ typedef struct {
   double inner_tol;      /* iterative inner solve's relative residual; <= 0:
                             library default (FP64: 1e-14; mixed: 1e-7 per FP32
                             refinement level); unused by the exact factor solve */
-  int32_t panel;         /* RHS columns per panel (1..32); <= 0: auto            */
+  int32_t panel;         /* RHS columns per panel (1..32); <= 0: auto; 1 and 2:
+                            the seed recurrence                             */
   int32_t flags;         /* Inner solve S w = u.  Default: the exact
                             block-bidiagonal Cholesky solve where S's
                             half-bandwidth is <= 63 (FP64: one solve; mixed: two
@@ -210,7 +215,9 @@ typedef struct {
                             3000 iterations (col_status 4 | 32; for use with
                             the correction solves, which set it themselves);
                             other bits are ignored                           */
-  int32_t seed_shift;    /* index of the seed shift; < 0: middle of the grid     */
+  int32_t seed_shift;    /* index of the seed shift of the seed recurrence; < 0:
+                            the real recurrence, which has none (with panel 1
+                            or 2: the middle of the grid)                    */
   int32_t reserved;
 } gb_solve_params;
 
@@ -223,7 +230,7 @@ typedef struct {
   double* edm;        /* [P] packed like rho, with the weights c^E_k            */
   double* q;          /* [nrhs] local charge  sum_i rho_ij S_ij                  */
   double* e_loc;      /* [nrhs] local energy  sum_i rho_ij H_ij                  */
-  int32_t* iters;     /* [nrhs] seed iterations used                            */
+  int32_t* iters;     /* [nrhs] outer iterations used                           */
   uint8_t* converged; /* [K][nrhs] 1 if the pair met tol                        */
   double* resid;      /* [K][nrhs] recursive residual estimate at exit          */
   double* g_proj;     /* [K][P][2] optional: G_ij(z_k) (re, im) on the pattern  */

@@ -33,7 +33,7 @@ __device__ __forceinline__ double2 warp_sum(double2 v) {
 
 // r_m[R_j] for every column of the panel -> one history row (FP64).
 template <bool MIX>
-__device__ void gather_hist(const Args& a, const Smem& sm, const SeedT<MIX>* r, double2* row) {
+__device__ void gather_hist(const Args& a, const SeedSmem& sm, const SeedT<MIX>* r, double2* row) {
   if (a.full_hist) {  // every row of every column: row[cc * N4 + i]
     const int N4 = 4 * a.m.nb, W = a.W;
     for (int e = threadIdx.x; e < N4 * W; e += TPB) {
@@ -60,7 +60,7 @@ struct PanelSmemExtra {
 };
 
 template <bool MIX>
-__device__ void solve_panel(const Args& a, Smem& sm, PanelSmemExtra& sx, char* ws, char* dyn) {
+__device__ void solve_panel(const Args& a, SeedSmem& sm, PanelSmemExtra& sx, char* ws, char* dyn) {
   using V = SeedT<MIX>;
   const int W = a.W, K = a.K, nb = a.m.nb, tid = threadIdx.x, c = tid % W;
   const size_t NE = (size_t)4 * nb * W;
@@ -655,72 +655,6 @@ __device__ void solve_panel(const Args& a, Smem& sm, PanelSmemExtra& sx, char* w
     }
   }
   __syncthreads();
-}
-
-template <bool MIX>
-__global__ void __launch_bounds__(TPB, MIN_TEAMS_PER_SM) team_kernel(const __grid_constant__ Args a) {
-  __shared__ Smem sm;
-  __shared__ PanelSmemExtra sx;
-  extern __shared__ __align__(16) char dyn_smem[];
-  char* ws = a.team_ws + (size_t)blockIdx.x * a.team_bytes;
-  team_init(sm, dyn_smem);
-  if (a.full_hist) {  // verification: one panel per team, panel = team
-    if (threadIdx.x == 0) sm.panel = blockIdx.x;
-    __syncthreads();
-    if (sm.panel < a.npanels) solve_panel<MIX>(a, sm, sx, ws, dyn_smem);
-    return;
-  }
-  for (;;) {
-    if (threadIdx.x == 0) sm.panel = atomicAdd(a.panel_counter, 1);
-    __syncthreads();
-    if (sm.panel >= a.npanels) return;
-    solve_panel<MIX>(a, sm, sx, ws, dyn_smem);
-    __syncthreads();
-  }
-}
-
-// Batched form: many independent systems (each with its own matrix, shifts,
-// columns and outputs) in one persistent launch.  Work items are (system,
-// panel) pairs numbered through panel_prefix (the host orders the systems,
-// largest first); a team copies the item's system descriptor into shared
-// memory and runs the same panel solver.  The team workspace is laid out for
-// the largest system.
-template <bool MIX>
-__global__ void __launch_bounds__(TPB, MIN_TEAMS_PER_SM)
-    team_kernel_batched(const Args* __restrict__ sys, const int* __restrict__ panel_prefix, int nsys,
-                        int* __restrict__ counter, char* team_ws, size_t team_bytes) {
-  __shared__ Smem sm;
-  __shared__ PanelSmemExtra sx;
-  __shared__ Args sa;
-  __shared__ int s_sys;
-  extern __shared__ __align__(16) char dyn_smem[];
-  char* ws = team_ws + (size_t)blockIdx.x * team_bytes;
-  team_init(sm, dyn_smem);
-  const int total = panel_prefix[nsys];
-  for (;;) {
-    if (threadIdx.x == 0) {
-      const int item = atomicAdd(counter, 1);
-      int lo = 0;
-      if (item < total) {
-        int hi = nsys;  // panel_prefix[lo] <= item < panel_prefix[hi]
-        while (hi - lo > 1) {
-          const int mid = (lo + hi) >> 1;
-          if (panel_prefix[mid] <= item) lo = mid;
-          else hi = mid;
-        }
-      }
-      s_sys = item < total ? lo : -1;
-      sm.panel = item < total ? item - panel_prefix[lo] : 0;
-    }
-    __syncthreads();
-    if (s_sys < 0) return;
-    const unsigned* src = reinterpret_cast<const unsigned*>(sys + s_sys);
-    unsigned* dst = reinterpret_cast<unsigned*>(&sa);
-    for (int i = threadIdx.x; i < (int)(sizeof(Args) / sizeof(unsigned)); i += TPB) dst[i] = src[i];
-    __syncthreads();
-    solve_panel<MIX>(sa, sm, sx, ws, dyn_smem);
-    __syncthreads();
-  }
 }
 
 }  // namespace gbk

@@ -9,7 +9,7 @@
 #include <vector>
 
 #include "gb_internal.h"
-#include "panel.cuh"
+#include "team_kernels.cuh"
 
 namespace gb {
 
@@ -797,7 +797,71 @@ void set_inner_method(const gb_matrix* m, const gb_solve_params* p, double itol,
   a.inner_cheb = 1;
 }
 
+// Which recurrence solves the panels.  The real three-term recurrence
+// (panel_real.cuh) does, except where the caller names a seed shift or asks for
+// panels of one or two columns: those run the seed recurrence (panel.cuh).  The
+// FP64 correction of stagnating columns is built on it (one-column panels,
+// another seed each time), and narrow panels are how callers reproduce what it
+// corrects.
+bool real_recurrence(const gb_solve_params* p, int panel) { return p->seed_shift < 0 && panel != 1 && panel != 2; }
+
+// Team-workspace layout of panels of W pairs (real recurrence) or W complex
+// columns (seed recurrence).
+size_t layout_team(size_t N4, int W, int K, int KG, int maxit, int Mcap, bool want_g, bool real, gbk::Args& a) {
+  const size_t Kz = K, R = real ? 2 * (size_t)W : W, mx = maxit;
+  const size_t esz = real ? 8 : 16;  // a history entry: v is real, r complex
+  size_t off = 0;
+  auto take = [&](size_t bytes) {
+    const size_t o = off;
+    off = align256(off + bytes);
+    return o;
+  };
+  const size_t vec = N4 * W * 16;
+  a.o_r = take(vec);
+  a.o_rt = take(vec);
+  a.o_p = real ? 0 : take(vec);
+  a.o_sp = real ? 0 : take(vec);
+  a.o_u = take(vec);
+  a.o_w = take(vec);
+  a.o_g = take(vec);
+  a.o_d = take(vec);
+  a.o_q = take(vec);
+  a.o_x = take(vec);
+  a.o_hr = take((mx + 1) * (size_t)Mcap * esz);
+  a.o_ab = take(mx * R * (real ? 24 : 32));
+  a.o_L = real ? 0 : take((mx + 1) * R * sizeof(int));
+  a.o_t = take((mx + 1) * R * esz);
+  a.o_ck = take((mx / gbk::CK + 1) * R * Kz * 2 * 16);
+  a.o_pi = take(R * Kz * 2 * 16);
+  a.o_nk = take(R * Kz * sizeof(int));
+  a.o_res = take(R * Kz * sizeof(double));
+  a.o_buf = take((gbk::CK + 1) * R * Kz * 16);
+  a.o_cp = take((mx + 1) * R * KG * 2 * esz);
+  a.o_cf = take((mx + 1) * R * 2 * esz);
+  a.o_cg = want_g ? take((mx + 1) * R * Kz * 16) : 0;
+  return off;
+}
+
+const void* team_fn(bool fp64, bool real) {
+  if (real) return fp64 ? (const void*)gbk::team_kernel<false, true> : (const void*)gbk::team_kernel<true, true>;
+  return fp64 ? (const void*)gbk::team_kernel<false, false> : (const void*)gbk::team_kernel<true, false>;
+}
+const void* batched_fn(bool fp64, bool real) {
+  if (real)
+    return fp64 ? (const void*)gbk::team_kernel_batched<false, true> : (const void*)gbk::team_kernel_batched<true, true>;
+  return fp64 ? (const void*)gbk::team_kernel_batched<false, false> : (const void*)gbk::team_kernel_batched<true, false>;
+}
+gb_status launch_team(gbk::Args& a, bool fp64, bool real, int teams, size_t dyn, cudaStream_t s) {
+  const void* fn = team_fn(fp64, real);
+  GB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+  void* args[] = {&a};
+  GB_CUDA(cudaLaunchKernel(fn, dim3(teams), dim3(gbk::TPB), args, dyn, s));
+  return GB_OK;
+}
+
 struct Plan {
+  int C;  // right-hand sides per panel
+  bool real;
   int W, KG, npanels, teams, teams_per_sm, Mcap, inner_maxit, cg_smem;
   size_t dyn_smem;
   double itol;
@@ -806,7 +870,9 @@ struct Plan {
   gbk::Args a;
 };
 
-gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, Plan* pl, bool full_hist = false) {
+// full_hist: the plan of a verification run of a solve by the recurrence `real`
+gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, Plan* pl, bool full_hist = false,
+                    bool verified_real = false) {
   if (!m) return fail(GB_EINVAL, "matrix is NULL");
   if (!p) return fail(GB_EINVAL, "params is NULL");
   if (p->nshift < 1 || p->nshift > 256) return fail(GB_EINVAL, "nshift must be in [1, 256]");
@@ -844,42 +910,48 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
   // two staged factor tiles in dynamic shared memory instead
   const bool bchol = !(p->flags & (kFlagCG | kFlagCheb)) && m->dm.bf_bw > 0;
   const bool want_smem = (p->flags & kFlagSmem) != 0 && !bchol;
+  const bool f64 = p->prec == GB_FP64, real = full_hist ? verified_real : real_recurrence(p, p->panel);
+  auto width = [&](int cols) { return real ? std::max(1, cols / 2) : cols; };  // stored pairs or complex columns
   auto fits = [&](int w) { return want_smem && 3 * n4 * (size_t)w * cg_esz + gbk::kRedBytes <= smem_budget; };
   auto dyn_bytes = [&](int w) -> size_t {
     const unsigned cg = fits(w) ? (unsigned)(3 * n4 * (size_t)w * cg_esz) : 0u;
-    return gbk::dyn_layout(p->prec == GB_FP64, w, bchol, cg, m->dm.bf_bw).bytes;
+    return gbk::dyn_layout(f64, w, bchol, cg, m->dm.bf_bw).bytes;
   };
   auto occupancy = [&](size_t dyn) {
     int per_sm = 1;
-    const void* fn = p->prec == GB_FP64 ? (const void*)gbk::team_kernel<false> : (const void*)gbk::team_kernel<true>;
+    const void* fn = team_fn(f64, real);
     if (dyn > 0) cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
     const cudaError_t oe = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, gbk::TPB, dyn);
     return (oe != cudaSuccess || per_sm < 1) ? 1 : per_sm;
   };
-  int W = p->panel;
-  if (W <= 0) {
+  int C = p->panel;
+  if (C <= 0) {
     // one wave that fills >= 3/4 of the team slots beats 1.5 waves of half-size
-    // panels (measured on the 1900-orbital chain: W = 8, 238 panels on 304
-    // slots, ~20% faster than W = 4)
-    W = 1;
+    // panels (measured on the 1900-orbital chain: 8 columns, 238 panels on 304
+    // slots, ~20% faster than 4)
+    C = 1;
     for (int cand : {32, 16, 8, 4, 2}) {
-      const size_t dyn = dyn_bytes(cand);
+      const size_t dyn = dyn_bytes(width(cand));
       if (4LL * ((p->nrhs + cand - 1) / cand) >= 3LL * nsm * occupancy(dyn)) {
-        W = cand;
+        C = cand;
         break;
       }
     }
+    if (real && C == 1 && p->nrhs > 1) C = 2;  // a pair costs what one of its columns does
   }
-  if (W != 1 && W != 2 && W != 4 && W != 8 && W != 16 && W != 32)
+  if (C != 1 && C != 2 && C != 4 && C != 8 && C != 16 && C != 32)
     return fail(GB_EINVAL, "panel must be 1, 2, 4, 8, 16 or 32");
+  const int W = width(C);
+  pl->C = C;
+  pl->real = real;
   pl->W = W;
   pl->cg_smem = fits(W) ? 1 : 0;
   pl->dyn_smem = dyn_bytes(W);
   pl->teams_per_sm = occupancy(pl->dyn_smem);
   pl->KG = (p->nshift + 31) / 32;
-  pl->npanels = (p->nrhs + W - 1) / W;
+  pl->npanels = (p->nrhs + C - 1) / C;
   pl->teams = std::min(pl->npanels, nsm * pl->teams_per_sm);
-  pl->Mcap = full_hist ? W * 4 * (int)m->nb : W * m->max_row;
+  pl->Mcap = full_hist ? (real ? 2 * W : W) * 4 * (int)m->nb : C * m->max_row;
   pl->inner_maxit = 500;
   // Inner-solve accuracy: the seed recurrence treats w = S^{-1} H p as exact,
   // and each iteration's error enters the shifted residual gap, so the inner
@@ -892,40 +964,16 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
 
   set_inner_method(m, p, pl->itol, pl->a);
   pl->a.bc_bw_alloc = m->dm.bf_bw;
-  const size_t K = p->nshift, Wz = W, maxit = p->maxit, N4 = 4 * (size_t)m->nb;
+  const size_t K = p->nshift, N4 = 4 * (size_t)m->nb;
+  pl->team_bytes = layout_team(N4, W, (int)K, pl->KG, p->maxit, pl->Mcap, want_g, real, pl->a);
+  pl->a.C = C;
+
   size_t off = 0;
   auto take = [&](size_t bytes) {
     const size_t o = off;
     off = align256(off + bytes);
     return o;
   };
-  gbk::Args& a = pl->a;
-  const size_t vec = N4 * Wz * 16;
-  a.o_r = take(vec);
-  a.o_rt = take(vec);
-  a.o_p = take(vec);
-  a.o_sp = take(vec);
-  a.o_u = take(vec);
-  a.o_w = take(vec);
-  a.o_g = take(vec);
-  a.o_d = take(vec);
-  a.o_q = take(vec);
-  a.o_x = take(vec);
-  a.o_hr = take((maxit + 1) * (size_t)pl->Mcap * 16);
-  a.o_ab = take(maxit * Wz * 2 * 16);
-  a.o_L = take((maxit + 1) * Wz * sizeof(int));
-  a.o_t = take((maxit + 1) * Wz * 16);
-  a.o_ck = take((maxit / gbk::CK + 1) * Wz * K * 2 * 16);
-  a.o_pi = take(Wz * K * 2 * 16);
-  a.o_nk = take(Wz * K * sizeof(int));
-  a.o_res = take(Wz * K * sizeof(double));
-  a.o_buf = take((gbk::CK + 1) * Wz * K * 16);
-  a.o_cp = take((maxit + 1) * Wz * pl->KG * 2 * 16);
-  a.o_cf = take((maxit + 1) * Wz * 2 * 16);
-  a.o_cg = want_g ? take((maxit + 1) * Wz * K * 16) : 0;
-  pl->team_bytes = off;
-
-  off = 0;
   pl->o_z = take(K * 16);
   pl->o_wr = take(K * 16);
   pl->o_we = take(K * 16);
@@ -948,7 +996,7 @@ gb_status gb_solve_plan(const gb_matrix* m, const gb_solve_params* p, int32_t* p
   Plan pl;
   gb_status st = make_plan(m, p, false, &pl);
   if (st != GB_OK) return st;
-  plan[0] = pl.W;
+  plan[0] = pl.C;
   plan[1] = pl.teams;
   plan[2] = pl.cg_smem;
   plan[3] = (int32_t)pl.dyn_smem;
@@ -1044,16 +1092,7 @@ gb_status gb_shifted_solve(const gb_matrix* m, const gb_solve_params* p, const g
   a.P = ho[nrhs];
 
   a.cg_smem = pl.cg_smem;
-  if (p->prec == GB_FP64) {
-    GB_CUDA(cudaFuncSetAttribute(gbk::team_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pl.dyn_smem));
-    gbk::team_kernel<false><<<pl.teams, gbk::TPB, pl.dyn_smem, s>>>(a);
-  } else {
-    GB_CUDA(cudaFuncSetAttribute(gbk::team_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pl.dyn_smem));
-    gbk::team_kernel<true><<<pl.teams, gbk::TPB, pl.dyn_smem, s>>>(a);
-  }
-  GB_CUDA(cudaGetLastError());
+  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, pl.teams, pl.dyn_smem, s)) != GB_OK) return st;
   std::vector<int> hst(nrhs);
   GB_CUDA(cudaMemcpyAsync(hst.data(), a.status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
   GB_CUDA(cudaStreamSynchronize(s));
@@ -1165,17 +1204,19 @@ gb_status gb_apply_sinv(const gb_matrix* m, gb_precision prec, int32_t w, const 
 namespace {
 
 // X[v][i][k] = sum_{m < nk[k]} c[m][k] r_m[i] for verified column v (panel
-// v / W, slot v % W): 64 rows x 32 shifts per block, 16 history steps staged
+// v / C, slot v % C of W; r_m real: the real recurrence's v_m): 64 rows x 32 shifts per block, 16 history steps staged
 // in shared memory per round, each thread 4 rows x 2 shifts.
-__global__ void __launch_bounds__(256) xk_kernel(int N4, int K, int W, int Mcap, int nver, const char* team_ws,
+template <bool REAL>
+__global__ void __launch_bounds__(256) xk_kernel(int N4, int K, int C, int W, int Mcap, int nver, const char* team_ws,
                                                  size_t team_bytes, size_t o_hr, size_t o_cg, size_t o_nk,
                                                  const int* iters_max, double2* __restrict__ X) {
-  __shared__ double2 Rs[16][64];
+  using H = typename std::conditional<REAL, double, double2>::type;
+  __shared__ H Rs[16][64];
   __shared__ double2 Cs[16][32];
-  const int v = blockIdx.z, t = v / W, cc = v % W;
+  const int v = blockIdx.z, t = v / C, cc = v % C;
   const int i0 = blockIdx.x * 64, k0 = blockIdx.y * 32;
   const char* ws = team_ws + (size_t)t * team_bytes;
-  const double2* hr = reinterpret_cast<const double2*>(ws + o_hr);
+  const H* hr = reinterpret_cast<const H*>(ws + o_hr);
   const double2* cg = reinterpret_cast<const double2*>(ws + o_cg);
   const int* nk = reinterpret_cast<const int*>(ws + o_nk);
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
@@ -1187,7 +1228,7 @@ __global__ void __launch_bounds__(256) xk_kernel(int N4, int K, int W, int Mcap,
     for (int e = threadIdx.x; e < 16 * 64; e += 256) {
       const int mm = e >> 6, i = e & 63;
       const int m = m0 + mm, row = i0 + i;
-      Rs[mm][i] = (m < M && row < N4) ? hr[(size_t)m * Mcap + (size_t)cc * N4 + row] : make_double2(0.0, 0.0);
+      Rs[mm][i] = (m < M && row < N4) ? hr[(size_t)m * Mcap + (size_t)cc * N4 + row] : H{};
     }
     for (int e = threadIdx.x; e < 16 * 32; e += 256) {
       const int mm = e >> 5, kk = e & 31;
@@ -1197,13 +1238,19 @@ __global__ void __launch_bounds__(256) xk_kernel(int N4, int K, int W, int Mcap,
     __syncthreads();
 #pragma unroll 4
     for (int mm = 0; mm < 16; ++mm) {
-      double2 r[4], c[2];
+      H r[4];
+      double2 c[2];
       for (int a = 0; a < 4; ++a) r[a] = Rs[mm][ty * 4 + a];
       for (int b = 0; b < 2; ++b) c[b] = Cs[mm][tx * 2 + b];
       for (int a = 0; a < 4; ++a)
         for (int b = 0; b < 2; ++b) {
-          acc[a][b].x = fma(r[a].x, c[b].x, fma(-r[a].y, c[b].y, acc[a][b].x));
-          acc[a][b].y = fma(r[a].x, c[b].y, fma(r[a].y, c[b].x, acc[a][b].y));
+          if constexpr (REAL) {
+            acc[a][b].x = fma(r[a], c[b].x, acc[a][b].x);
+            acc[a][b].y = fma(r[a], c[b].y, acc[a][b].y);
+          } else {
+            acc[a][b].x = fma(r[a].x, c[b].x, fma(-r[a].y, c[b].y, acc[a][b].x));
+            acc[a][b].y = fma(r[a].x, c[b].y, fma(r[a].y, c[b].x, acc[a][b].y));
+          }
         }
     }
     __syncthreads();
@@ -1277,7 +1324,7 @@ gb_status ver_layout(const gb_matrix* m, const gb_solve_params* p, int32_t nver,
   q.nrhs = nver;
   q.rhs_cols = cols.data();
   q.panel = W;
-  gb_status st = make_plan(m, &q, true, &L->pl, true);
+  gb_status st = make_plan(m, &q, true, &L->pl, true, real_recurrence(p, p->panel));
   if (st != GB_OK) return st;
   L->W = W;
   L->pl.teams = L->pl.npanels;  // verification: every panel at once, one team each
@@ -1376,21 +1423,16 @@ gb_status gb_true_residual(const gb_matrix* m, const gb_solve_params* p, int32_t
   a.Mcap = pl.Mcap;
   a.iters = reinterpret_cast<int*>(wsb + L.o_im);
   a.cg_smem = pl.cg_smem;
-  if (p->prec == GB_FP64) {
-    GB_CUDA(cudaFuncSetAttribute(gbk::team_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pl.dyn_smem));
-    gbk::team_kernel<false><<<pl.teams, gbk::TPB, pl.dyn_smem, s>>>(a);
-  } else {
-    GB_CUDA(cudaFuncSetAttribute(gbk::team_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pl.dyn_smem));
-    gbk::team_kernel<true><<<pl.teams, gbk::TPB, pl.dyn_smem, s>>>(a);
-  }
-  GB_CUDA(cudaGetLastError());
+  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, pl.teams, pl.dyn_smem, s)) != GB_OK) return st;
   double2* X = reinterpret_cast<double2*>(wsb + L.o_x);
   {
     const dim3 grid((unsigned)((N4 + 63) / 64), (unsigned)((K + 31) / 32), (unsigned)nver);
-    xk_kernel<<<grid, 256, 0, s>>>(N4, K, pl.W, pl.Mcap, nver, a.team_ws, pl.team_bytes, a.o_hr, a.o_cg, a.o_nk,
-                                   a.iters, X);
+    if (pl.real)
+      xk_kernel<true><<<grid, 256, 0, s>>>(N4, K, pl.C, 2 * pl.W, pl.Mcap, nver, a.team_ws, pl.team_bytes, a.o_hr,
+                                           a.o_cg, a.o_nk, a.iters, X);
+    else
+      xk_kernel<false><<<grid, 256, 0, s>>>(N4, K, pl.C, pl.W, pl.Mcap, nver, a.team_ws, pl.team_bytes, a.o_hr, a.o_cg,
+                                            a.o_nk, a.iters, X);
     GB_CUDA(cudaGetLastError());
   }
   {
@@ -2007,16 +2049,7 @@ gb_status gb_shifted_solve_static(const gb_matrix* m, const gb_solve_params* p, 
   a.g_proj = reinterpret_cast<double2*>(out->g_proj);
   a.P = ho[nrhs];
   a.cg_smem = pl.cg_smem;
-  if (p->prec == GB_FP64) {
-    GB_CUDA(cudaFuncSetAttribute(gbk::team_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pl.dyn_smem));
-    gbk::team_kernel<false><<<teams, gbk::TPB, pl.dyn_smem, s>>>(a);
-  } else {
-    GB_CUDA(cudaFuncSetAttribute(gbk::team_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)pl.dyn_smem));
-    gbk::team_kernel<true><<<teams, gbk::TPB, pl.dyn_smem, s>>>(a);
-  }
-  GB_CUDA(cudaGetLastError());
+  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, teams, pl.dyn_smem, s)) != GB_OK) return st;
   GB_CUDA(cudaMemcpyAsync(g_static_status, a.status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
   GB_CUDA(cudaStreamSynchronize(s));
   int any = 0;
@@ -2038,44 +2071,9 @@ size_t gb_static_scratch_bytes(void) { return kStaticScratchBytes; }
 // Many independent systems in one persistent launch (team_kernel_batched).
 namespace {
 
-// Team-workspace layout for the given maxima (same regions as a single solve).
-size_t layout_team(size_t N4, int W, int K, int KG, int maxit, int Mcap, bool want_g, gbk::Args& a) {
-  const size_t Kz = K, Wz = W, mx = maxit;
-  size_t off = 0;
-  auto take = [&](size_t bytes) {
-    const size_t o = off;
-    off = align256(off + bytes);
-    return o;
-  };
-  const size_t vec = N4 * Wz * 16;
-  a.o_r = take(vec);
-  a.o_rt = take(vec);
-  a.o_p = take(vec);
-  a.o_sp = take(vec);
-  a.o_u = take(vec);
-  a.o_w = take(vec);
-  a.o_g = take(vec);
-  a.o_d = take(vec);
-  a.o_q = take(vec);
-  a.o_x = take(vec);
-  a.o_hr = take((mx + 1) * (size_t)Mcap * 16);
-  a.o_ab = take(mx * Wz * 2 * 16);
-  a.o_L = take((mx + 1) * Wz * sizeof(int));
-  a.o_t = take((mx + 1) * Wz * 16);
-  a.o_ck = take((mx / gbk::CK + 1) * Wz * Kz * 2 * 16);
-  a.o_pi = take(Wz * Kz * 2 * 16);
-  a.o_nk = take(Wz * Kz * sizeof(int));
-  a.o_res = take(Wz * Kz * sizeof(double));
-  a.o_buf = take((gbk::CK + 1) * Wz * Kz * 16);
-  a.o_cp = take((mx + 1) * Wz * KG * 2 * 16);
-  a.o_cf = take((mx + 1) * Wz * 2 * 16);
-  a.o_cg = want_g ? take((mx + 1) * Wz * Kz * 16) : 0;
-  return off;
-}
-
 struct BatchPlan {
-  int W, teams, total_panels, maxK, maxit, Mcap, KG;
-  bool mixed, want_g;
+  int C, W, teams, total_panels, maxK, maxit, Mcap, KG;
+  bool real, mixed, want_g;
   size_t N4, team_bytes, header_bytes, total, dyn_smem;
   std::vector<int> order;  // systems, largest estimated cost first
   gbk::Args proto;
@@ -2111,8 +2109,10 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   cudaError_t e = cudaGetDeviceProperties(&prop, dev);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDeviceProperties");
   const int nsm = prop.multiProcessorCount;
-  const void* fn = prec == GB_FP64 ? (const void*)gbk::team_kernel_batched<false>
-                                   : (const void*)gbk::team_kernel_batched<true>;
+  bool real = true;  // one recurrence per launch
+  for (int s = 0; s < nsys; ++s) real = real && real_recurrence(&params[s], panel);
+  auto width = [&](int cols) { return real ? std::max(1, cols / 2) : cols; };
+  const void* fn = batched_fn(prec == GB_FP64, real);
   // dynamic shared memory: the factor solve's buffers (systems without a
   // factor leave them unused)
   auto dyn_bytes = [&](int w) -> size_t { return gbk::dyn_layout(prec == GB_FP64, w, true, 0, 63).bytes; };
@@ -2123,22 +2123,26 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
       per_sm = 1;
     return per_sm;
   };
-  int W = panel;
-  if (W <= 0) {  // widest panel that still gives every resident team a work item
-    W = 1;
+  int C = panel;
+  if (C <= 0) {  // widest panel that still gives every resident team a work item
+    C = 1;
     for (int cand : {32, 16, 8, 4, 2}) {
       long long np = 0;
       for (int s = 0; s < nsys; ++s) np += (params[s].nrhs + cand - 1) / cand;
-      if (4 * np >= 3LL * nsm * occupancy(dyn_bytes(cand))) {
-        W = cand;
+      if (4 * np >= 3LL * nsm * occupancy(dyn_bytes(width(cand)))) {
+        C = cand;
         break;
       }
     }
+    if (real && C == 1) C = 2;  // a pair costs what one of its columns does
   }
-  if (W != 1 && W != 2 && W != 4 && W != 8 && W != 16 && W != 32)
+  if (C != 1 && C != 2 && C != 4 && C != 8 && C != 16 && C != 32)
     return fail(GB_EINVAL, "panel must be 1, 2, 4, 8, 16 or 32");
+  const int W = width(C);
   bp->dyn_smem = dyn_bytes(W);
   const int per_sm = occupancy(bp->dyn_smem);
+  bp->C = C;
+  bp->real = real;
   bp->W = W;
   bp->mixed = prec == GB_MIXED;
   bp->want_g = want_g;
@@ -2146,11 +2150,12 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   bp->maxK = kmax;
   bp->KG = (kmax + 31) / 32;
   bp->maxit = itmax;
-  bp->Mcap = W * rowmax;
+  bp->Mcap = C * rowmax;
   std::memset(&bp->proto, 0, sizeof bp->proto);
-  bp->team_bytes = layout_team(n4max, W, kmax, bp->KG, itmax, bp->Mcap, want_g, bp->proto);
+  bp->team_bytes = layout_team(n4max, W, kmax, bp->KG, itmax, bp->Mcap, want_g, real, bp->proto);
+  bp->proto.C = C;
   bp->total_panels = 0;
-  for (int s = 0; s < nsys; ++s) bp->total_panels += (params[s].nrhs + W - 1) / W;
+  for (int s = 0; s < nsys; ++s) bp->total_panels += (params[s].nrhs + C - 1) / C;
   bp->teams = std::min(bp->total_panels, nsm * per_sm);
   // largest systems first (cost ~ basis size x shifts) for load balance
   bp->order.resize(nsys);
@@ -2267,7 +2272,7 @@ gb_status gb_shifted_solve_batched(int32_t nsys, const gb_matrix* const* mats, c
     a.W = bp.W;
     a.KG = (K + 31) / 32;
     a.nrhs = nrhs;
-    a.npanels = (nrhs + bp.W - 1) / bp.W;
+    a.npanels = (nrhs + bp.C - 1) / bp.C;
     a.maxit = p->maxit;
     a.inner_maxit = 500;
     a.has_rho = p->w_rho != nullptr;
@@ -2286,7 +2291,7 @@ gb_status gb_shifted_solve_batched(int32_t nsys, const gb_matrix* const* mats, c
     a.panel_counter = reinterpret_cast<int*>(wsb + o_counter);
     a.team_ws = team_ws;
     a.team_bytes = bp.team_bytes;
-    a.Mcap = bp.W * m->max_row;
+    a.Mcap = bp.C * m->max_row;
     a.cg_smem = 0;
     a.ldos = out->ldos;
     a.rho = out->rho;
@@ -2307,18 +2312,12 @@ gb_status gb_shifted_solve_batched(int32_t nsys, const gb_matrix* const* mats, c
   const gbk::Args* d_desc = reinterpret_cast<const gbk::Args*>(wsb);
   const int* d_prefix = reinterpret_cast<const int*>(wsb + o_prefix);
   int* d_counter = reinterpret_cast<int*>(wsb + o_counter);
-  if (bp.mixed) {
-    GB_CUDA(cudaFuncSetAttribute(gbk::team_kernel_batched<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)bp.dyn_smem));
-    gbk::team_kernel_batched<true><<<bp.teams, gbk::TPB, bp.dyn_smem, s>>>(d_desc, d_prefix, nsys, d_counter,
-                                                                           team_ws, bp.team_bytes);
-  } else {
-    GB_CUDA(cudaFuncSetAttribute(gbk::team_kernel_batched<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)bp.dyn_smem));
-    gbk::team_kernel_batched<false><<<bp.teams, gbk::TPB, bp.dyn_smem, s>>>(d_desc, d_prefix, nsys, d_counter,
-                                                                            team_ws, bp.team_bytes);
+  {
+    const void* fn = batched_fn(!bp.mixed, bp.real);
+    GB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.dyn_smem));
+    void* args[] = {&d_desc, &d_prefix, &nsys, &d_counter, &team_ws, &bp.team_bytes};
+    GB_CUDA(cudaLaunchKernel(fn, dim3(bp.teams), dim3(gbk::TPB), args, bp.dyn_smem, s));
   }
-  GB_CUDA(cudaGetLastError());
   GB_CUDA(cudaMemcpyAsync(hdr.data(), wsb, bp.header_bytes, cudaMemcpyDeviceToHost, s));
   GB_CUDA(cudaStreamSynchronize(s));
   int any = 0;

@@ -40,6 +40,7 @@ constexpr int kRescaleExp = 8;              // ... by 2^8 (exact)
 
 struct Args {
   DevMat m;
+  int C;  // right-hand sides per panel (seed recurrence: W; real recurrence: 2 W, or 1 of a pair)
   int K, W, KG, nrhs, npanels, maxit, inner_maxit, has_rho, has_edm, want_g;
   double tol, itol;
   double2 sigma;
@@ -53,7 +54,7 @@ struct Args {
   char* team_ws;
   size_t team_bytes;
   size_t o_r, o_rt, o_p, o_sp, o_u, o_w, o_g, o_d, o_q, o_x;
-  size_t o_hr, o_ab, o_L, o_t, o_ck, o_pi, o_nk, o_res, o_buf, o_cp, o_cf, o_cg;
+  size_t o_hr, o_ab, o_L, o_t, o_ck, o_pi, o_nk, o_res, o_buf, o_cp, o_cf, o_cg;  // real recurrence: no o_L
   int Mcap;
   int cg_smem;  // 1: the inner-CG vectors g, d, q live in dynamic shared memory
   // Chebyshev inner iteration of the mixed path (inner_cheb = 1): K steps per
@@ -93,16 +94,24 @@ constexpr int kStInner = 8;
 constexpr int kStTimeout = 16;  // a bounded wait for a staged factor tile gave up
 constexpr int kStStall = 32;    // stopped early: no shift of the column was improving
 
+// What the inner solves need of a team: a panel's W complex columns (or W pairs
+// of real columns, see panel_real.cuh), their active flags and status bits.
 struct Smem {
   RedSmem rs;
-  int panel, Wp, flag, inner_count;
-  int j[WMAX], mc[WMAX], off[WMAX + 1], act[WMAX], nc[WMAX], nact[WMAX], st[WMAX], nfresh[WMAX];
-  double2 rho[WMAX], alpha[WMAX], beta[WMAX], aprev[WMAX], bprev[WMAX], gam[WMAX];
-  double rt2[WMAX], scl[WMAX];
+  int panel, flag, inner_count;
+  int act[WMAX], st[WMAX];
   double cg_rho[2 * WMAX], cg_un[2 * WMAX], cg_gg[2 * WMAX], cg_a[2 * WMAX], cg_b[2 * WMAX];
   unsigned long long bc_bar[3];  // mbarriers of the staged factor tiles (block_chol.cuh)
   unsigned tile_base;            // factor tiles consumed so far in this launch
   int bc_fail;                   // a bounded tile wait gave up
+};
+
+// The seed recurrence's per-column state (panel.cuh).
+struct SeedSmem : Smem {
+  int Wp;
+  int j[WMAX], mc[WMAX], off[WMAX + 1], nc[WMAX], nact[WMAX], nfresh[WMAX];
+  double2 rho[WMAX], alpha[WMAX], beta[WMAX], aprev[WMAX], bprev[WMAX], gam[WMAX];
+  double rt2[WMAX], scl[WMAX];
 };
 
 // Once per launch, before the team's first panel: the block-reduce scratch in
