@@ -376,51 +376,53 @@ void block_factor(HostBSR* hb) {
   hb->bf_nblk = nblk;
 }
 
-// Fragment order of an m16n8k8 TF32 A operand (PTX mma): lane l = 4 g + t
-// holds a0 = A(g, t), a1 = A(g + 8, t), a2 = A(g, t + 4), a3 = A(g + 8, t + 4)
-// of the 16 x 8 tile (rows 16 mi.., columns 8 ks..).  A fragment is stored as
-// 128 consecutive floats, lane l's four values at 4 l .. 4 l + 3.
-static void put_fragment(const double* M, int mi, int ks, float* dst) {  // M k-major: (r, k) at k * 64 + r
-  for (int l = 0; l < 32; ++l) {
-    const int g = l >> 2, t = l & 3;
-    for (int sl = 0; sl < 4; ++sl) {
-      const int r = 16 * mi + g + 8 * (sl & 1), k = 8 * ks + t + 4 * (sl >> 1);
-      dst[l * 4 + sl] = (float)M[(size_t)k * 64 + r];
-    }
-  }
-}
-
-// Per block: the FWD tile holds the D^-1 fragments a lower-triangular product
-// needs (k-step ks, row tile mi >= ks / 2; 20 of them, by ks then mi), then
-// the E fragments of k-steps (64 - bw) / 8 .. 7 (by ks then mi); the BWD tile
-// holds the D^-T fragments with mi <= ks / 2 (20), then the F fragments of
-// k-steps 0 .. ceil(bw / 8) - 1.
-std::vector<float> mma_tiles(const HostBSR& hb) {
-  std::vector<float> out;
-  if (hb.bf_bw <= 0 || hb.bf.empty()) return out;
+// Scales and growth bounds of the mixed path's factor tiles (the tiles themselves
+// are formed from the FP64 factor on the device).
+FactorTiles factor_tiles(const HostBSR& hb) {
+  FactorTiles f;
+  if (hb.bf_bw <= 0 || hb.bf.empty()) return f;
   const int64_t nblk = hb.bf_nblk;
   const size_t part = (size_t)nblk * 4096;
-  const double* df = hb.bf.data();
-  const double* db = df + part;
-  const double* ef = db + part;
-  const double* fb = ef + part;
-  const int bw = hb.bf_bw, ksE0 = (64 - bw) / 8, nF = (bw + 7) / 8;
-  out.assign((size_t)2 * nblk * kMmaTileFloats, 0.f);
-  for (int64_t blk = 0; blk < nblk; ++blk) {
-    float* fwd = out.data() + (size_t)(2 * blk) * kMmaTileFloats;
-    float* bwd = fwd + kMmaTileFloats;
-    int p = 0;
-    for (int ks = 0; ks < 8; ++ks)
-      for (int mi = ks / 2; mi < 4; ++mi) put_fragment(df + (size_t)blk * 4096, mi, ks, fwd + 128 * p++);
-    for (int ks = ksE0; ks < 8; ++ks)
-      for (int mi = 0; mi < 4; ++mi) put_fragment(ef + (size_t)blk * 4096, mi, ks, fwd + 128 * p++);
-    p = 0;
-    for (int ks = 0; ks < 8; ++ks)
-      for (int mi = 0; mi <= ks / 2; ++mi) put_fragment(db + (size_t)blk * 4096, mi, ks, bwd + 128 * p++);
-    for (int ks = 0; ks < nF; ++ks)
-      for (int mi = 0; mi < 4; ++mi) put_fragment(fb + (size_t)blk * 4096, mi, ks, bwd + 128 * p++);
+  const double* m[4] = {hb.bf.data(), hb.bf.data() + 2 * part, hb.bf.data() + part, hb.bf.data() + 3 * part};
+  f.ne = (hb.bf_bw + 15) / 16;
+  int* ex = f.ex;  // the largest entry of D^-1, E, D^-T, F is below 2^ex
+  for (int q = 0; q < 4; ++q) {
+    double mx = 0.0;
+    for (size_t e = 0; e < part; ++e) mx = std::max(mx, std::fabs(m[q][e]));
+    std::frexp(mx > 0.0 ? mx : 1.0, &ex[q]);
   }
-  return out;
+  // Growth bounds: |y| <= 2^lg1 max|f| and, with y scaled by 2^-lg1, |x| <= 2^lg2 max|f|, from the
+  // recursions with absolute values (r_i = |D^-1| 1 + |E| r_{i-1}, then the same backward).
+  std::vector<double> r((size_t)nblk * 64), u((size_t)nblk * 64);
+  auto bound = [&](int dir, const std::vector<double>& in, std::vector<double>& out) {
+    double top = 0.0;
+    for (int64_t s = 0; s < nblk; ++s) {
+      const int64_t b = dir ? nblk - 1 - s : s, pb = dir ? b + 1 : b - 1;
+      double v[64] = {};
+      for (int k = 0; k < 64; ++k) {
+        const double *d = m[2 * dir] + b * 4096 + k * 64, *e = m[2 * dir + 1] + b * 4096 + k * 64;
+        const double fd = in[b * 64 + k], fe = s > 0 ? out[pb * 64 + k] : 0.0;
+        for (int i = 0; i < 64; ++i) v[i] += std::fabs(d[i]) * fd + std::fabs(e[i]) * fe;
+      }
+      for (int i = 0; i < 64; ++i) {
+        out[b * 64 + i] = v[i];
+        top = std::max(top, v[i]);
+      }
+    }
+    int lg = 0;
+    std::frexp(top > 0.0 && std::isfinite(top) ? top : 1.0, &lg);
+    return lg;
+  };
+  std::fill(u.begin(), u.end(), 1.0);
+  const int lg1 = bound(0, u, r);
+  for (auto& v : r) v = std::ldexp(v, -lg1);
+  const int lg2 = bound(1, r, u);
+  f.lg = lg1 + lg2;
+  f.kd[0] = (float)std::ldexp(1.0, ex[0] - 4 - lg1);  // tile entries are scaled to below 2^4
+  f.ke[0] = (float)std::ldexp(1.0, ex[1] - 4);
+  f.kd[1] = (float)std::ldexp(1.0, ex[2] - 4 - lg2);
+  f.ke[1] = (float)std::ldexp(1.0, ex[3] - 4);
+  return f;
 }
 
 }  // namespace gb

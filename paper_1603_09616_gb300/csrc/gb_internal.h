@@ -39,13 +39,16 @@ gb_status build_host_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_i
 void preconditioned_s_bounds(HostBSR* hb);
 void block_factor(HostBSR* hb);
 
-// The FP32 factor rearranged for the tensor-core passes of the exact inner
-// solve (block_chol.cuh): per 64-row block two tiles of kMmaTilePairs
-// fragments (FWD: D^-1 then E; BWD: D^-T then F), each fragment the 32 x 4
-// values one warp loads for an m16n8k8 TF32 A operand.  Returns
-// 2 * nblk * kMmaTileFloats floats (empty without a factor).
-constexpr int kMmaTilePairs = 52;                     // 20 triangular + up to 32 band fragments
-constexpr int kMmaTileFloats = kMmaTilePairs * 128;  // 26,624 bytes
-std::vector<float> mma_tiles(const HostBSR& hb);
+// What the mixed path's tensor-core passes (factor_passes.cuh) need to know of the
+// factor: its tiles hold the entries scaled to below 2^4 as FP16 heads and tails,
+// and kd / ke undo the scaling (kd: triangular tile of either direction, with the
+// growth bound of the direction; ke: band tile; lg: both bounds' exponent).
+struct FactorTiles {
+  int ne = 0;  // 16-column steps of the band tile (0: no factor)
+  int lg = 0;
+  int ex[4] = {0, 0, 0, 0};
+  float kd[2] = {1.f, 1.f}, ke[2] = {1.f, 1.f};
+};
+FactorTiles factor_tiles(const HostBSR& hb);
 
 }  // namespace gb

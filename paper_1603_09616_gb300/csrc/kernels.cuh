@@ -57,14 +57,16 @@ struct DevMat {
   double s_lam_min, s_lam_max;  // spectrum bounds of the block-Jacobi-preconditioned S
   // Block-bidiagonal Cholesky factor of S on 64-row blocks (bf_bw = 0: none).
   // FP64: four [bf_nblk][64][64] arrays, k-major (entry (r, k) at k * 64 + r):
-  // D_i^-1, D_i^-T, E_i = D_i^-1 C_i, F_i = D_i^-T C_{i+1}^T.  FP32: per block
-  // a FWD and a BWD tile of kMmaTileFloatsDev floats in tensor-core fragment
-  // order (block_chol.cuh).
+  // D_i^-1, D_i^-T, E_i = D_i^-1 C_i, F_i = D_i^-T C_{i+1}^T.  Mixed path: FP16
+  // head / tail fragments of the same tiles (gb::FactorTiles, factor_passes.cuh).
   int bf_bw, bf_nblk;
-  const float* bfm;
   const double* bf64;
+  const float* bfm;  // the seed recurrence's TF32 tiles (seed_passes.cuh)
+  const uint4* fx;
+  int fx_ne, fx_lg;
+  float fx_kd[2], fx_ke[2];
 };
-constexpr int kMmaTileFloatsDev = 52 * 128;
+constexpr int kMmaTileFloatsDev = 52 * 128;  // a TF32 tile: 20 triangular and up to 32 band fragments
 
 // ------------------------------------------------------------ complex FP64
 __device__ __forceinline__ double2 cadd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }

@@ -137,7 +137,7 @@ __device__ void solve_panel(const Args& a, SeedSmem& sm, PanelSmemExtra& sx, cha
 
   // r_0 = S^{-1} b
   if constexpr (MIX) {
-    inner_mixed(a, sm, rt, r, cg_x, cg_g, cg_d, cg_q, dyn);
+    inner_mixed<false>(a, sm, rt, r, cg_x, cg_g, cg_d, cg_q, dyn);
   } else {
     inner64(a, sm, rt, r, cg_g, cg_d, cg_q, dyn);
   }
@@ -270,7 +270,7 @@ __device__ void solve_panel(const Args& a, SeedSmem& sm, PanelSmemExtra& sx, cha
 
     // w = S^{-1} U
     if constexpr (MIX) {
-      inner_mixed(a, sm, U, w, cg_x, cg_g, cg_d, cg_q, dyn);
+      inner_mixed<false>(a, sm, U, w, cg_x, cg_g, cg_d, cg_q, dyn);
     } else {
       inner64(a, sm, U, w, cg_g, cg_d, cg_q, dyn);
     }

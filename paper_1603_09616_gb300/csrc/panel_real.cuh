@@ -148,7 +148,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
   // v = S^-1 f and b2 = f^T v for the active pairs
   auto apply_sinv = [&](const V* f) {
     if constexpr (MIX)
-      inner_mixed(a, sm, f, v, cg_x, cg_g, cg_d, cg_q, dyn);
+      inner_mixed<true>(a, sm, f, v, cg_x, cg_g, cg_d, cg_q, dyn);
     else
       inner64(a, sm, f, v, cg_g, cg_d, cg_q, dyn);
     double d[2] = {0, 0};
@@ -174,6 +174,8 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
     if (tid < R) sm.b2[tid] = sm.rs.scal[(tid & 1) * WMAX + (tid >> 1)];
     __syncthreads();
   };
+  if (tid < R) sm.fmax[tid] = __float_as_uint(1.f);
+  __syncthreads();
   apply_sinv(s);
   gather_real<MIX>(a, sm, v, hr);
   if (tid < R) ht[tid] = 1.0;  // s_0[j]
@@ -275,6 +277,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
       gbff::acc_init(d1);
       const double p0 = sm.c1[2 * c], p1 = sm.c1[2 * c + 1], q0 = sm.c2[2 * c], q1 = sm.c2[2 * c + 1];
       const double t0 = sm.c3[2 * c], t1 = sm.c3[2 * c + 1];
+      float m0 = 0.f, m1 = 0.f;  // max |s|, for the factor solve's scale
       if constexpr (MIX) {
         const gbff::ff fp0 = gbff::ff_from_double(p0), fp1 = gbff::ff_from_double(p1);
         const gbff::ff fq0 = gbff::ff_from_double(-q0), fq1 = gbff::ff_from_double(-q1);
@@ -289,11 +292,14 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
                                            gbff::ff_add(gbff::ff_mul(fq1, gbff::ff{x.z, x.w}),
                                                         gbff::ff_mul(ft1, gbff::ff{y.z, y.w})));
           so[e] = make_float4(r0.hi, r0.lo, r1.hi, r1.lo);
+          m0 = fmaxf(m0, fabsf(r0.hi));
+          m1 = fmaxf(m1, fabsf(r1.hi));
           gbff::acc_mul_add(d0, r0, r0);
           gbff::acc_mul_add(d1, r1, r1);
         }
         d[0] = gbff::acc_to_double(d0);
         d[1] = gbff::acc_to_double(d1);
+        col_max(sm, W, m0, m1);
       } else {
         for (size_t e = tid; e < NE; e += TPB) {
           if (!sm.act[c]) continue;

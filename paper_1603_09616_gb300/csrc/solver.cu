@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <vector>
 
 #include "gb_internal.h"
@@ -485,6 +486,114 @@ __global__ void spmm_kernel(const gbk::DevMat m, int which, int W, const void* _
 
 }  // namespace
 
+// ------------------------------------------------------------ what a matrix keeps beside FP64
+namespace {
+
+// Float-float splits v = hi + lo (lo may be null: hi alone) of n FP64 values.
+__global__ void split_kernel(const double* __restrict__ v, size_t n, float* __restrict__ hi, float* __restrict__ lo) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const double x = v[i];
+    const float h = (float)x;
+    hi[i] = h;
+    if (lo) lo[i] = (float)(x - (double)h);
+  }
+}
+
+// The factor's tiles in MMA fragment order, one block of threads per 64-row block
+// and direction.  Element (r, k) of a 64 x 64 factor block lies at k * 64 + r.
+//
+// FP16 tiles (factor_passes.cuh): fragments of 16 x 16 (mi, kk), the entries scaled
+// to below 2^4, 32 lanes x 4 words of FP16 heads and then the same of tails.  Lane
+// l = 4 g + t holds in word q row g + 8 (q & 1) and the column pair w = t + 4 (q >> 1),
+// a pair being columns w and w + 8: the order in which the passes pack the vector's
+// rows.  First the triangle's (FWD: kk <= mi, by mi then kk; BWD: kk >= mi), then the
+// band's (E: its last ne column steps; F: its first), by mi.
+//
+// TF32 tiles (seed_passes.cuh): fragments of 16 x 8 (mi, ks), lane l's word q is
+// A(g + 8 (q & 1), t + 4 (q >> 1)); first the triangle's (FWD: mi >= ks / 2, by ks
+// then mi; BWD: mi <= ks / 2), then the band's (E: ks from (64 - bw) / 8; F: ks below
+// ceil(bw / 8)), by ks.
+struct TileArgs {
+  const double* bf;
+  size_t part;
+  int bw, ne;
+  float sd[2], se[2];
+  uint32_t* fx;
+  float* tf;
+};
+__global__ void __launch_bounds__(256) tile_kernel(TileArgs a) {
+  const int blk = blockIdx.x >> 1, dir = blockIdx.x & 1;
+  const double* D = a.bf + dir * a.part + (size_t)blk * 4096;
+  const double* E = a.bf + (2 + dir) * a.part + (size_t)blk * 4096;
+  uint32_t* fx = a.fx + (size_t)blockIdx.x * (10 + 4 * a.ne) * 256;
+  for (int e = threadIdx.x; e < (10 + 4 * a.ne) * 128; e += 256) {
+    const int f = e >> 7, l = (e & 127) >> 2, q = e & 3;
+    int mi, kk;
+    if (f < 10) {
+      mi = 0;
+      while (f >= (dir ? 4 * (mi + 1) - (mi + 1) * mi / 2 : (mi + 1) * (mi + 2) / 2)) ++mi;
+      kk = dir ? f - (4 * mi - mi * (mi - 1) / 2) + mi : f - mi * (mi + 1) / 2;
+    } else {
+      mi = (f - 10) / a.ne;
+      kk = (f - 10) % a.ne + (dir ? 0 : 4 - a.ne);
+    }
+    const double* M = f < 10 ? D : E;
+    const double sc = f < 10 ? a.sd[dir] : a.se[dir];
+    const int r = 16 * mi + (l >> 2) + 8 * (q & 1), k = 16 * kk + (l & 3) + 4 * (q >> 1);
+    uint32_t h, t;
+    gbk::split_f16((float)(M[k * 64 + r] * sc), (float)(M[(k + 8) * 64 + r] * sc), h, t);
+    fx[(size_t)f * 256 + l * 4 + q] = h;
+    fx[(size_t)f * 256 + 128 + l * 4 + q] = t;
+  }
+  float* tf = a.tf + (size_t)blockIdx.x * gbk::kMmaTileFloatsDev;
+  const int ks0 = dir ? 0 : (64 - a.bw) / 8, n2 = dir ? (a.bw + 7) / 8 : 8 - ks0;
+  for (int e = threadIdx.x; e < (20 + 4 * n2) * 128; e += 256) {
+    const int f = e >> 7, l = (e & 127) >> 2, q = e & 3;
+    int mi, ks;
+    if (f < 20) {
+      int left = f;
+      for (ks = 0;; ++ks) {
+        const int c = dir ? ks / 2 + 1 : 4 - ks / 2;
+        if (left < c) break;
+        left -= c;
+      }
+      mi = dir ? left : ks / 2 + left;
+    } else {
+      ks = ks0 + (f - 20) / 4;
+      mi = (f - 20) & 3;
+    }
+    const int r = 16 * mi + (l >> 2) + 8 * (q & 1), k = 8 * ks + (l & 3) + 4 * (q >> 1);
+    tf[e] = (float)(f < 20 ? D : E)[k * 64 + r];
+  }
+}
+
+cudaError_t form_on_device(const gbk::DevMat& d, size_t nnzb, const FactorTiles& ft, cudaStream_t s) {
+  auto split = [&](const double* v, size_t n, const float* hi, const float* lo) {
+    const unsigned blocks = (unsigned)std::min<size_t>((n + 255) / 256, 152 * 8);
+    split_kernel<<<blocks, 256, 0, s>>>(v, n, const_cast<float*>(hi), const_cast<float*>(lo));
+  };
+  split(d.hb, nnzb * 16, d.hb_hi, d.hb_lo);
+  split(d.sb, nnzb * 16, d.sb_hi, d.sb_lo);
+  split(d.minv, (size_t)d.nb * 16, d.minv32, nullptr);
+  if (d.bf_nblk > 0) {
+    TileArgs t{};
+    t.bf = d.bf64;
+    t.part = (size_t)d.bf_nblk * 4096;
+    t.bw = d.bf_bw;
+    t.ne = ft.ne;
+    for (int q = 0; q < 2; ++q) {
+      t.sd[q] = std::ldexp(1.f, 4 - ft.ex[2 * q]);
+      t.se[q] = std::ldexp(1.f, 4 - ft.ex[2 * q + 1]);
+    }
+    t.fx = reinterpret_cast<uint32_t*>(const_cast<uint4*>(d.fx));
+    t.tf = const_cast<float*>(d.bfm);
+    tile_kernel<<<2 * d.bf_nblk, 256, 0, s>>>(t);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace
+
 // The standalone SpMM reads rows 4J..4J+3 of x for every stored block column
 // J; when n % 4 != 0 the last block column reaches past row n-1 (its matrix
 // entries are zero there), so gb_spmm reads from a zero-padded copy of x.
@@ -550,51 +659,36 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   };
   const size_t o_bp = take(sizeof(int) * (nbl + 1)), o_bc = take(sizeof(int) * nnzb);
   const size_t o_hb = take(sizeof(double) * nnzb * 16), o_sb = take(sizeof(double) * nnzb * 16);
-  const size_t o_hh = take(sizeof(float) * nnzb * 16), o_hl = take(sizeof(float) * nnzb * 16);
-  const size_t o_sh = take(sizeof(float) * nnzb * 16), o_sl = take(sizeof(float) * nnzb * 16);
-  const size_t o_mi = take(sizeof(double) * nbl * 16), o_m32 = take(sizeof(float) * nbl * 16);
+  const size_t o_mi = take(sizeof(double) * nbl * 16);
   const size_t o_rp = take(sizeof(int) * (n + 1)), o_ci = take(sizeof(int) * nnz);
   const size_t o_hv = take(sizeof(double) * nnz), o_sv = take(sizeof(double) * nnz);
   const size_t nbf = hb.bf.size();  // 4 x nblk x 4096 factor entries (0: no factor)
-  const std::vector<float> mt = mma_tiles(hb);
-  static_assert(kMmaTileFloats == gbk::kMmaTileFloatsDev, "tile size of host and device");
-  const size_t o_bf64 = take(sizeof(double) * nbf), o_bfm = take(sizeof(float) * mt.size());
+  const FactorTiles ft = factor_tiles(hb);
+  const size_t nblk = nbf ? (size_t)hb.bf_nblk : 0;
+  const size_t o_bf64 = take(sizeof(double) * nbf);
+  const size_t up = off;  // uploaded; the rest is formed from it on the device
+  const size_t o_hh = take(sizeof(float) * nnzb * 16), o_hl = take(sizeof(float) * nnzb * 16);
+  const size_t o_sh = take(sizeof(float) * nnzb * 16), o_sl = take(sizeof(float) * nnzb * 16);
+  const size_t o_m32 = take(sizeof(float) * nbl * 16);
+  const size_t o_bfm = take(sizeof(float) * 2 * nblk * gbk::kMmaTileFloatsDev);
+  const size_t o_fx = take(sizeof(uint4) * 2 * nblk * gbk::fx_block_words(ft.ne));
   const size_t total = off;
 
-  std::vector<char> host(total, 0);
-  auto put = [&](size_t o, const void* src, size_t bytes) { std::memcpy(host.data() + o, src, bytes); };
+  std::unique_ptr<char[]> host(new char[up]);
+  auto put = [&](size_t o, const void* src, size_t bytes) { std::memcpy(host.get() + o, src, bytes); };
   put(o_bp, hb.blk_ptr.data(), sizeof(int) * (nbl + 1));
   put(o_bc, hb.blk_col.data(), sizeof(int) * nnzb);
   put(o_hb, hb.blk_h.data(), sizeof(double) * nnzb * 16);
   put(o_sb, hb.blk_s.data(), sizeof(double) * nnzb * 16);
-  {
-    float* hh = reinterpret_cast<float*>(host.data() + o_hh);
-    float* hl = reinterpret_cast<float*>(host.data() + o_hl);
-    float* sh = reinterpret_cast<float*>(host.data() + o_sh);
-    float* sl = reinterpret_cast<float*>(host.data() + o_sl);
-    for (size_t i = 0; i < nnzb * 16; ++i) {
-      const float a = (float)hb.blk_h[i];
-      hh[i] = a;
-      hl[i] = (float)(hb.blk_h[i] - (double)a);
-      const float b = (float)hb.blk_s[i];
-      sh[i] = b;
-      sl[i] = (float)(hb.blk_s[i] - (double)b);
-    }
-    float* m32 = reinterpret_cast<float*>(host.data() + o_m32);
-    for (size_t i = 0; i < nbl * 16; ++i) m32[i] = (float)hb.minv[i];
-  }
   put(o_mi, hb.minv.data(), sizeof(double) * nbl * 16);
   {
-    int* rp = reinterpret_cast<int*>(host.data() + o_rp);
+    int* rp = reinterpret_cast<int*>(host.get() + o_rp);
     for (int64_t i = 0; i <= n; ++i) rp[i] = (int)hb.row_ptr[i];
   }
   put(o_ci, hb.col_idx.data(), sizeof(int) * nnz);
   put(o_hv, hb.h_val.data(), sizeof(double) * nnz);
   put(o_sv, hb.s_val.data(), sizeof(double) * nnz);
-  if (nbf) {
-    put(o_bf64, hb.bf.data(), sizeof(double) * nbf);
-    put(o_bfm, mt.data(), sizeof(float) * mt.size());
-  }
+  if (nbf) put(o_bf64, hb.bf.data(), sizeof(double) * nbf);
 
   gb_matrix* m = new gb_matrix();
   m->device = dev;
@@ -608,13 +702,6 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   if (e != cudaSuccess) {
     delete m;
     return fail(GB_ENOMEM, "cudaMalloc(%zu bytes) for the matrix failed: %s", total, cudaGetErrorString(e));
-  }
-  e = cudaMemcpyAsync(m->base, host.data(), total, cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  if (e != cudaSuccess) {
-    cudaFree(m->base);
-    delete m;
-    return cuda_fail(e, "matrix upload");
   }
   char* b = static_cast<char*>(m->base);
   gbk::DevMat& d = m->dm;
@@ -639,7 +726,22 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   d.bf_bw = nbf ? hb.bf_bw : 0;
   d.bf_nblk = nbf ? (int)hb.bf_nblk : 0;
   d.bf64 = nbf ? reinterpret_cast<const double*>(b + o_bf64) : nullptr;
+  d.fx = nbf ? reinterpret_cast<const uint4*>(b + o_fx) : nullptr;
+  d.fx_ne = ft.ne;
+  d.fx_lg = ft.lg;
+  for (int q = 0; q < 2; ++q) {
+    d.fx_kd[q] = ft.kd[q];
+    d.fx_ke[q] = ft.ke[q];
+  }
   d.bfm = nbf ? reinterpret_cast<const float*>(b + o_bfm) : nullptr;
+  e = cudaMemcpyAsync(m->base, host.get(), up, cudaMemcpyHostToDevice, s);
+  if (e == cudaSuccess) e = form_on_device(d, nnzb, ft, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) {
+    cudaFree(m->base);
+    delete m;
+    return cuda_fail(e, "matrix upload");
+  }
   *out = m;
   return GB_OK;
 }
@@ -915,7 +1017,7 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
   auto fits = [&](int w) { return want_smem && 3 * n4 * (size_t)w * cg_esz + gbk::kRedBytes <= smem_budget; };
   auto dyn_bytes = [&](int w) -> size_t {
     const unsigned cg = fits(w) ? (unsigned)(3 * n4 * (size_t)w * cg_esz) : 0u;
-    return gbk::dyn_layout(f64, w, bchol, cg, m->dm.bf_bw).bytes;
+    return gbk::dyn_layout(f64, w, bchol, cg, m->dm.bf_bw, !real).bytes;
   };
   auto occupancy = [&](size_t dyn) {
     int per_sm = 1;
@@ -1126,7 +1228,18 @@ __global__ void __launch_bounds__(gbk::TPB, 1)
   if (threadIdx.x < gbk::WMAX) sm.act[threadIdx.x] = threadIdx.x < a.W ? 1 : 0;
   if (threadIdx.x == 0) sm.inner_count = 0;
   __syncthreads();
-  gbk::bc_solve<T>(a, sm, x, y, t1, t2, dyn_smem);
+  if constexpr (sizeof(T) == 4) {
+    float m0 = 0.f, m1 = 0.f;
+    for (int e = threadIdx.x; e < 4 * a.m.nb * a.W; e += gbk::TPB) {
+      m0 = fmaxf(m0, fabsf(x[e].x));
+      m1 = fmaxf(m1, fabsf(x[e].y));
+    }
+    gbk::col_max(sm, a.W, m0, m1);
+    __syncthreads();
+    gbk::fx_solve(a, sm, x, y, t1, t2);
+  } else {
+    gbk::bc_solve64(a, sm, x, y, t1, t2);
+  }
   if (threadIdx.x == 0) *status = sm.bc_fail ? gbk::kStTimeout : 0;
 }
 
@@ -2115,7 +2228,7 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   const void* fn = batched_fn(prec == GB_FP64, real);
   // dynamic shared memory: the factor solve's buffers (systems without a
   // factor leave them unused)
-  auto dyn_bytes = [&](int w) -> size_t { return gbk::dyn_layout(prec == GB_FP64, w, true, 0, 63).bytes; };
+  auto dyn_bytes = [&](int w) -> size_t { return gbk::dyn_layout(prec == GB_FP64, w, true, 0, 63, !real).bytes; };
   auto occupancy = [&](size_t dyn) {
     int per_sm = 1;
     cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
@@ -2778,7 +2891,7 @@ __global__ void __launch_bounds__(gbk::TPB, 1)
     E[e] = make_double2((c0 + l < nrhs && cols[c0 + l] == row) ? 1.0 : 0.0, 0.0);
   }
   __syncthreads();
-  gbk::bc_solve<double>(a, sm, E, X, t1, t2, dyn_smem);  // X = S^-1 E (ends with a barrier)
+  gbk::bc_solve64(a, sm, E, X, t1, t2);  // X = S^-1 E (ends with a barrier)
   for (int it = tid; it < a.m.nb * W; it += gbk::TPB) {  // E <- H X
     const int I = it / W, l = it - I * W;
     double2 acc[4];
@@ -2787,7 +2900,7 @@ __global__ void __launch_bounds__(gbk::TPB, 1)
     for (int r = 0; r < 4; ++r) E[(size_t)(4 * I + r) * W + l] = acc[r];
   }
   __syncthreads();
-  gbk::bc_solve<double>(a, sm, E, Z, t1, t2, dyn_smem);  // Z = S^-1 H S^-1 E
+  gbk::bc_solve64(a, sm, E, Z, t1, t2);  // Z = S^-1 H S^-1 E
   for (int l = 0; l < W && c0 + l < nrhs; ++l) {
     const int c = c0 + l, j = cols[c], e0 = a.m.row_ptr[j], len = a.m.row_ptr[j + 1] - e0;
     for (int t = tid; t < len; t += gbk::TPB) {
@@ -2924,7 +3037,7 @@ __global__ void __launch_bounds__(gbk::TPB, 1)
       for (int r = 0; r < 4; ++r) HX[(size_t)(4 * I + r) * W + l] = acc[r];
     }
     __syncthreads();
-    gbk::bc_solve<double>(a, sm, HX, Y, t1, t2, dyn_smem);
+    gbk::bc_solve64(a, sm, HX, Y, t1, t2);
   };
   for (int step = 0; step < nsteps; ++step) {
     double2* tm = Tm;

@@ -101,7 +101,9 @@ struct Smem {
   int panel, flag, inner_count;
   int act[WMAX], st[WMAX];
   double cg_rho[2 * WMAX], cg_un[2 * WMAX], cg_gg[2 * WMAX], cg_a[2 * WMAX], cg_b[2 * WMAX];
-  unsigned long long bc_bar[3];  // mbarriers of the staged factor tiles (block_chol.cuh)
+  unsigned long long bc_bar[3];  // mbarriers of the staged factor tiles (factor_passes.cuh)
+  unsigned fmax[2 * WMAX];       // max |f| per real column of the next factor solve's input (FP32 bits)
+  float fsc[2 * WMAX], fun[2 * WMAX];  // its power-of-two scale, and what undoes it in the result
   unsigned tile_base;            // factor tiles consumed so far in this launch
   int bc_fail;                   // a bounded tile wait gave up
 };
@@ -132,6 +134,7 @@ __device__ __forceinline__ void team_init(Smem& sm, char* dyn) {
     sm.tile_base = 0;
     sm.bc_fail = 0;
   }
+  if (threadIdx.x < 2 * WMAX) sm.fmax[threadIdx.x] = 0;
   __syncthreads();
 }
 
@@ -518,15 +521,17 @@ __device__ __forceinline__ void cg_start_scalars(Smem& sm, int W) {
 // ------------------------------------------------------------ inner solve, mixed
 // w = S^{-1} U to ~FP64 accuracy: FP32 CG on hi(U), a float-float residual
 // e = U - S x1, FP32 CG on e, w = x1 + x2 (float-float).
+template <bool REAL>
 __device__ __noinline__ void inner_mixed_factor(const Args& a, Smem& sm, const float4* __restrict__ U, float4* __restrict__ w,
                                    float2* __restrict__ x, float2* __restrict__ g, float2* __restrict__ d,
                                    float2* __restrict__ q, char* dyn);
 
+template <bool REAL>
 __device__ __noinline__ void inner_mixed(const Args& a, Smem& sm, const float4* __restrict__ U, float4* __restrict__ w,
                             float2* __restrict__ x, float2* __restrict__ g, float2* __restrict__ d,
                             float2* __restrict__ q, char* dyn) {
   if (a.inner_bchol) {
-    inner_mixed_factor(a, sm, U, w, x, g, d, q, dyn);
+    inner_mixed_factor<REAL>(a, sm, U, w, x, g, d, q, dyn);
     return;
   }
   const int W = a.W, nb = a.m.nb, c = threadIdx.x % W;
@@ -640,10 +645,11 @@ __device__ __noinline__ void inner_mixed(const Args& a, Smem& sm, const float4* 
 // levels give ~1e-13 and three ~1e-19 (a.bc_levels, set from the tolerance).
 // g = U - S v (float-float) for the active columns; v is the FP32 vector x
 // (XV = float2) or the float-float w (XV = float4).  No barrier.
-template <typename XV>
-__device__ __noinline__ void ff_residual(const Args& a, const Smem& sm, const float4* __restrict__ U,
+template <bool REAL, typename XV>
+__device__ __noinline__ void ff_residual(const Args& a, Smem& sm, const float4* __restrict__ U,
                                          const XV* __restrict__ v, float2* __restrict__ g) {
   const int W = a.W, nb = a.m.nb, c = threadIdx.x % W;
+  float m0 = 0.f, m1 = 0.f;
   for (int it = threadIdx.x; it < nb * W; it += TPB) {
     if (!sm.act[c]) continue;
     const int I = it / W;
@@ -658,22 +664,31 @@ __device__ __noinline__ void ff_residual(const Args& a, const Smem& sm, const fl
       const float4 u = U[e];
       const gbff::ff er = gbff::ff_sub(gbff::ff{u.x, u.y}, gbff::acc_get(are[r]));
       const gbff::ff ei = gbff::ff_sub(gbff::ff{u.z, u.w}, gbff::acc_get(aim[r]));
-      g[e] = make_float2(er.hi + er.lo, ei.hi + ei.lo);
+      const float2 gv = make_float2(er.hi + er.lo, ei.hi + ei.lo);
+      g[e] = gv;
+      m0 = fmaxf(m0, fabsf(gv.x));
+      m1 = fmaxf(m1, fabsf(gv.y));
     }
   }
+  if (REAL) col_max(sm, W, m0, m1);
 }
 
+// Real recurrence: U's column maxima must have been left in sm.fmax (col_max, then a barrier).
+template <bool REAL>
 __device__ __noinline__ void inner_mixed_factor(const Args& a, Smem& sm, const float4* __restrict__ U, float4* __restrict__ w,
                                    float2* __restrict__ x, float2* __restrict__ g, float2* __restrict__ d,
                                    float2* __restrict__ q, char* dyn) {
   const int W = a.W, nb = a.m.nb, c = threadIdx.x % W;
-  bc_solve<float>(a, sm, U, x, d, q, dyn);
+  if constexpr (REAL)
+    fx_solve(a, sm, U, x, d, q);
+  else
+    seed_solve(a, sm, U, x, d);
   for (int lev = 1; lev < a.bc_levels; ++lev) {
     // e = U - S w into g; at the first refinement w = x1 is the FP32 vector x
     if (lev == 1)
-      ff_residual(a, sm, U, x, g);
+      ff_residual<REAL>(a, sm, U, x, g);
     else
-      ff_residual(a, sm, U, w, g);
+      ff_residual<REAL>(a, sm, U, w, g);
     __syncthreads();  // every read of x / w for the residual is done
     if (lev == 1) {
       for (int e = threadIdx.x; e < 4 * nb * W; e += TPB) {
@@ -683,7 +698,10 @@ __device__ __noinline__ void inner_mixed_factor(const Args& a, Smem& sm, const f
       }
       __syncthreads();
     }
-    bc_solve<float>(a, sm, g, x, d, q, dyn);
+    if constexpr (REAL)
+      fx_solve(a, sm, g, x, d, q);
+    else
+      seed_solve(a, sm, g, x, d);
     for (int e = threadIdx.x; e < 4 * nb * W; e += TPB) {
       if (!sm.act[c]) continue;
       const float4 wv = w[e];
@@ -709,7 +727,7 @@ __device__ __noinline__ void inner_mixed_factor(const Args& a, Smem& sm, const f
 __device__ __noinline__ void inner64(const Args& a, Smem& sm, const double2* __restrict__ f, double2* __restrict__ x,
                         double2* __restrict__ g, double2* __restrict__ d, double2* __restrict__ q, char* dyn) {
   if (a.inner_bchol)
-    bc_solve<double>(a, sm, f, x, d, q, dyn);
+    bc_solve64(a, sm, f, x, d, q);
   else
     cg64(a, sm, f, x, g, d, q);
 }
