@@ -385,10 +385,16 @@ FactorTiles factor_tiles(const HostBSR& hb) {
   const size_t part = (size_t)nblk * 4096;
   const double* m[4] = {hb.bf.data(), hb.bf.data() + 2 * part, hb.bf.data() + part, hb.bf.data() + 3 * part};
   f.ne = (hb.bf_bw + 15) / 16;
+  // rows of a block that are not padding (whose unit diagonal says nothing of S's scale)
+  auto rows_of = [&](int64_t b) { return (int)std::min<int64_t>(64, hb.n - 64 * b); };
   int* ex = f.ex;  // the largest entry of D^-1, E, D^-T, F is below 2^ex
   for (int q = 0; q < 4; ++q) {
     double mx = 0.0;
-    for (size_t e = 0; e < part; ++e) mx = std::max(mx, std::fabs(m[q][e]));
+    for (int64_t b = 0; b < nblk; ++b) {
+      const int rows = rows_of(b);
+      for (int k = 0; k < 64; ++k)
+        for (int i = 0; i < rows; ++i) mx = std::max(mx, std::fabs(m[q][(size_t)b * 4096 + k * 64 + i]));
+    }
     std::frexp(mx > 0.0 ? mx : 1.0, &ex[q]);
   }
   // Growth bounds: |y| <= 2^lg1 max|f| and, with y scaled by 2^-lg1, |x| <= 2^lg2 max|f|, from the
@@ -405,8 +411,8 @@ FactorTiles factor_tiles(const HostBSR& hb) {
         for (int i = 0; i < 64; ++i) v[i] += std::fabs(d[i]) * fd + std::fabs(e[i]) * fe;
       }
       for (int i = 0; i < 64; ++i) {
-        out[b * 64 + i] = v[i];
-        top = std::max(top, v[i]);
+        out[b * 64 + i] = i < rows_of(b) ? v[i] : 0.0;
+        top = std::max(top, out[b * 64 + i]);
       }
     }
     int lg = 0;

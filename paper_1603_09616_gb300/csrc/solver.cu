@@ -516,7 +516,7 @@ __global__ void split_kernel(const double* __restrict__ v, size_t n, float* __re
 struct TileArgs {
   const double* bf;
   size_t part;
-  int bw, ne;
+  int n, bw, ne;
   float sd[2], se[2];
   uint32_t* fx;
   float* tf;
@@ -540,8 +540,10 @@ __global__ void __launch_bounds__(256) tile_kernel(TileArgs a) {
     const double* M = f < 10 ? D : E;
     const double sc = f < 10 ? a.sd[dir] : a.se[dir];
     const int r = 16 * mi + (l >> 2) + 8 * (q & 1), k = 16 * kk + (l & 3) + 4 * (q >> 1);
+    // the padding's unit diagonal would not fit the scale; its rows of the vector are zero
+    const bool in = 64 * blk + r < a.n;
     uint32_t h, t;
-    gbk::split_f16((float)(M[k * 64 + r] * sc), (float)(M[(k + 8) * 64 + r] * sc), h, t);
+    gbk::split_f16(in ? (float)(M[k * 64 + r] * sc) : 0.f, in ? (float)(M[(k + 8) * 64 + r] * sc) : 0.f, h, t);
     fx[(size_t)f * 256 + l * 4 + q] = h;
     fx[(size_t)f * 256 + 128 + l * 4 + q] = t;
   }
@@ -579,6 +581,7 @@ cudaError_t form_on_device(const gbk::DevMat& d, size_t nnzb, const FactorTiles&
     TileArgs t{};
     t.bf = d.bf64;
     t.part = (size_t)d.bf_nblk * 4096;
+    t.n = d.n;
     t.bw = d.bf_bw;
     t.ne = ft.ne;
     for (int q = 0; q < 2; ++q) {
