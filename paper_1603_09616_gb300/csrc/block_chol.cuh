@@ -33,7 +33,7 @@ struct CplxOf<double> {
 };
 
 constexpr int kTileBufs = 3;  // band tiles staged: two in flight ahead of the one in use
-constexpr unsigned kRedBytes = NWARP * NVMAX * 32 * 8;  // block_reduce's partials
+constexpr unsigned kRedBytes = TPB_WIDE / 32 * NVMAX * 32 * 8;  // block_reduce's partials
 
 // Dynamic shared memory of a team (host and device agree through this):
 //   FP32 factor passes: the tensor-core layout below (mma_layout);
@@ -76,21 +76,21 @@ __host__ __device__ inline MmaLayout mma_layout(int W, int bw) {
 
 // Mixed path (factor_passes.cuh): [S staged band tiles][output block x 2, FP16
 // head and tail words].  A stage holds the band tile's 4 ne fragment pairs (1 KB
-// each); a block's words are 32 row pairs of P >= R columns, P = 8 mod 16 so that
-// the B-fragment loads hit every bank once.  block_reduce's partials alias the
-// stages (the passes and the reductions never overlap).
+// each); a block's words are kOutWords for each of max(R, 8) columns: 32 row pairs
+// and 4 of padding, so that stores and ldmatrix rows hit every bank once.
+// block_reduce's partials alias the stages (the passes and the reductions never
+// overlap).
+constexpr int kOutWords = 36;
 struct PassLayout {
-  int P;
   unsigned stage, o_y, bytes;
 };
 __host__ __device__ inline PassLayout pass_layout(int W, int ne) {
   PassLayout L;
-  L.P = 2 * W <= 8 ? 8 : 2 * W + 8;
   L.stage = (unsigned)ne * 4096u;
   unsigned off = (unsigned)kTileBufs * L.stage;
   if (off < kRedBytes) off = kRedBytes;
   L.o_y = off;
-  off += 2u * 2u * 32u * (unsigned)L.P * 4u;
+  off += 2u * 2u * (unsigned)(2 * W > 8 ? 2 * W : 8) * kOutWords * 4u;
   L.bytes = (off + 127u) & ~127u;
   return L;
 }

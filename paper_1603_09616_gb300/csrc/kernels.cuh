@@ -35,6 +35,13 @@ constexpr int NWARP = TPB / 32;
 #define GB_WARP_SPMM 0
 #endif
 constexpr int MIN_TEAMS_PER_SM = GB_MIN_TEAMS;
+// The real recurrence's mixed teams run 512 threads, two per SM, or 1024 (the same
+// 64 registers a thread) where a launch has no more panels than SMs: its products
+// are bound by load latency with 16 warps on an SM (46 % of issue slots) and by
+// issue with 32.  Everything else runs TPB threads.
+constexpr int TPB_WIDE = 2 * TPB;
+__device__ __forceinline__ int tpb() { return (int)blockDim.x; }
+__device__ __forceinline__ int nwarp() { return (int)blockDim.x >> 5; }
 constexpr int WMAX = 32;
 constexpr int NVMAX = 4;
 
@@ -90,7 +97,7 @@ struct RedSmem {
 
 // Sum NV per-thread partials over all threads sharing column c = tid % W.
 // Result for (value i, column c) lands in rs.scal[i * WMAX + c].  Fixed order.
-// The per-warp partials (NWARP * NVMAX * 32 doubles) live at the start of the
+// The per-warp partials (warps * NVMAX * 32 doubles) live at the start of the
 // kernel's dynamic shared memory, which every team kernel sizes for them.
 template <int NV>
 __device__ __forceinline__ void block_reduce(double (&v)[NV], int W, RedSmem& rs) {
@@ -105,11 +112,66 @@ __device__ __forceinline__ void block_reduce(double (&v)[NV], int W, RedSmem& rs
     for (int i = 0; i < NV; ++i) br_dyn[(warp * NV + i) * 32 + lane] = v[i];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < NV * W; t += TPB) {
+  for (int t = threadIdx.x; t < NV * W; t += tpb()) {
     const int i = t / W, c = t - i * W;
     double s = 0.0;
-    for (int w = 0; w < NWARP; ++w) s += br_dyn[(w * NV + i) * 32 + c];
+    for (int w = 0; w < nwarp(); ++w) s += br_dyn[(w * NV + i) * 32 + c];
     rs.scal[i * WMAX + c] = s;
+  }
+  __syncthreads();
+}
+
+// The same sums for the real recurrence: the warps' partials meet in a shuffle tree
+// (one lane per warp) instead of a chain of 16 or 32 dependent FP64 adds, which
+// took 2000 of the 26,000 cycles of an update pass.  warps: a power of two.
+template <int NV>
+__device__ __forceinline__ void block_reduce_tree(double (&v)[NV], int W, RedSmem& rs) {
+  extern __shared__ __align__(16) double br_dyn[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nwarp();
+  for (int off = W; off < 32; off <<= 1) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) v[i] += __shfl_xor_sync(0xffffffffu, v[i], off);
+  }
+  if (lane < W) {
+#pragma unroll
+    for (int i = 0; i < NV; ++i) br_dyn[(i * W + lane) * nw + warp] = v[i];
+  }
+  __syncthreads();
+  // whole warps: NV * W * nw is a multiple of 32 for every W >= 1 (nw >= 16, NV = 2)
+  static_assert(NV % 2 == 0, "whole warps take the partials");
+  for (int t = threadIdx.x; t < NV * W * nw; t += tpb()) {
+    double s = br_dyn[t];
+    for (int off = nw >> 1; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    const int o = t / nw;
+    if (t - o * nw == 0) rs.scal[(o / W) * WMAX + o % W] = s;
+  }
+  __syncthreads();
+}
+
+// The same for two compensated accumulators per thread (the mixed path's dots): the
+// lanes of a warp meet in FP32 pairs and FP64 starts with one lane per warp and
+// column.  A warp's FP64 instruction holds its scheduler for 64 cycles on GB300, so
+// converting and adding in every lane cost 6000 cycles a reduction.
+__device__ __forceinline__ void acc_xor_combine(gbff::acc& a, int off);
+__device__ __forceinline__ void block_reduce_acc(gbff::acc d0, gbff::acc d1, int W, RedSmem& rs) {
+  extern __shared__ __align__(16) double br_dyn[];
+  float2* part = reinterpret_cast<float2*>(br_dyn);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = nwarp();
+  for (int off = W; off < 32; off <<= 1) {
+    acc_xor_combine(d0, off);
+    acc_xor_combine(d1, off);
+  }
+  if (lane < W) {
+    part[lane * nw + warp] = make_float2(d0.hi, d0.err);
+    part[(W + lane) * nw + warp] = make_float2(d1.hi, d1.err);
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < 2 * W * nw; t += tpb()) {  // whole warps
+    const float2 p = part[t];
+    double s = (double)p.x + (double)p.y;
+    for (int off = nw >> 1; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    const int o = t / nw;
+    if (t - o * nw == 0) rs.scal[(o / W) * WMAX + o % W] = s;
   }
   __syncthreads();
 }
@@ -272,6 +334,114 @@ __device__ __forceinline__ void bsr_row_ffx(const DevMat& m, const float* __rest
   }
 }
 
+
+// ------------------------------------------------------------ one scalar row per thread
+// The real recurrence's products: thread = (row i = 4 I + r, column pair c), that
+// is element e = i W + c of the panel, so results and dots are coalesced.  The four
+// rows of a block share its x loads through the warp (same addresses), and each
+// loads its own matrix row.  Against one block row per thread (above) a panel has
+// four times the threads at work and a quarter of the accumulators each: the team
+// waits on load latency (ncu: 29 % of issue slots used with one team per SM), and
+// two blocks in flight fit the 64 registers without spills.  Measured, 912
+// orbitals, 8 columns, one team per SM: see panel_real.cuh.
+// float-float row times a float-float vector (float4 pairs).
+__device__ __forceinline__ void row_ff(const DevMat& m, const float* __restrict__ Ahi, const float* __restrict__ Alo,
+                                       const float4* x, int W, int c, int row, gbff::acc& a0, gbff::acc& a1) {
+  gbff::acc_init(a0);
+  gbff::acc_init(a1);
+  const float4* ah = reinterpret_cast<const float4*>(Ahi) + (row & 3);
+  const float4* al = reinterpret_cast<const float4*>(Alo) + (row & 3);
+  const int I = row >> 2, b1 = m.blk_ptr[I + 1];
+#pragma unroll 2
+  for (int b = m.blk_ptr[I]; b < b1; ++b) {
+    const float4* xr = x + (size_t)(4 * m.blk_col[b]) * W + c;
+    const float4 h = __ldg(ah + 4 * (size_t)b), l = __ldg(al + 4 * (size_t)b);
+    float4 xv[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) xv[t] = xr[t * W];
+    const float hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      gbff::acc_mul_add(a0, gbff::ff{hv[t], lv[t]}, gbff::ff{xv[t].x, xv[t].y});
+      gbff::acc_mul_add(a1, gbff::ff{hv[t], lv[t]}, gbff::ff{xv[t].z, xv[t].w});
+    }
+  }
+}
+
+// float-float row times an FP32 vector (float2 pairs), compensated.
+__device__ __forceinline__ void row_ffx(const DevMat& m, const float* __restrict__ Ahi, const float* __restrict__ Alo,
+                                        const float2* x, int W, int c, int row, gbff::acc& a0, gbff::acc& a1) {
+  gbff::acc_init(a0);
+  gbff::acc_init(a1);
+  const float4* ah = reinterpret_cast<const float4*>(Ahi) + (row & 3);
+  const float4* al = reinterpret_cast<const float4*>(Alo) + (row & 3);
+  const int I = row >> 2, b1 = m.blk_ptr[I + 1];
+#pragma unroll 2
+  for (int b = m.blk_ptr[I]; b < b1; ++b) {
+    const float2* xr = x + (size_t)(4 * m.blk_col[b]) * W + c;
+    const float4 h = __ldg(ah + 4 * (size_t)b), l = __ldg(al + 4 * (size_t)b);
+    float2 xv[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) xv[t] = xr[t * W];
+    const float hv[4] = {h.x, h.y, h.z, h.w}, lv[4] = {l.x, l.y, l.z, l.w};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      gbff::acc_mul_add(a0, gbff::ff{hv[t], lv[t]}, xv[t].x);
+      gbff::acc_mul_add(a1, gbff::ff{hv[t], lv[t]}, xv[t].y);
+    }
+  }
+}
+
+// FP32 row (the heads) times an FP32 vector: float2 pairs, or the heads of float4 pairs.
+template <typename XV>
+__device__ __forceinline__ float2 row_f(const DevMat& m, const float* __restrict__ A, const XV* x, int W, int c,
+                                        int row) {
+  float2 acc = make_float2(0.f, 0.f);
+  const float4* ah = reinterpret_cast<const float4*>(A) + (row & 3);
+  const int I = row >> 2, b1 = m.blk_ptr[I + 1];
+#pragma unroll 4
+  for (int b = m.blk_ptr[I]; b < b1; ++b) {
+    const XV* xr = x + (size_t)(4 * m.blk_col[b]) * W + c;
+    const float4 h = __ldg(ah + 4 * (size_t)b);
+    const float hv[4] = {h.x, h.y, h.z, h.w};
+    XV xv[4];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) xv[t] = xr[t * W];
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      if constexpr (sizeof(XV) == 16) {
+        acc.x = fmaf(hv[t], xv[t].x, acc.x);
+        acc.y = fmaf(hv[t], xv[t].z, acc.y);
+      } else {
+        acc.x = fmaf(hv[t], xv[t].x, acc.x);
+        acc.y = fmaf(hv[t], xv[t].y, acc.y);
+      }
+    }
+  }
+  return acc;
+}
+
+__device__ __forceinline__ double2 row_d(const DevMat& m, const double* __restrict__ A, const double2* x, int W, int c,
+                                         int row) {
+  double2 acc = make_double2(0.0, 0.0);
+  const double2* ar = reinterpret_cast<const double2*>(A) + 2 * (row & 3);
+  const int I = row >> 2, b1 = m.blk_ptr[I + 1];
+#pragma unroll 2
+  for (int b = m.blk_ptr[I]; b < b1; ++b) {
+    const double2* xr = x + (size_t)(4 * m.blk_col[b]) * W + c;
+    const double2 a01 = __ldg(ar + 8 * (size_t)b), a23 = __ldg(ar + 8 * (size_t)b + 1);
+    const double2 x0 = xr[0], x1 = xr[W], x2 = xr[2 * W], x3 = xr[3 * W];
+    acc.x = fma(a01.x, x0.x, acc.x);
+    acc.y = fma(a01.x, x0.y, acc.y);
+    acc.x = fma(a01.y, x1.x, acc.x);
+    acc.y = fma(a01.y, x1.y, acc.y);
+    acc.x = fma(a23.x, x2.x, acc.x);
+    acc.y = fma(a23.x, x2.y, acc.y);
+    acc.x = fma(a23.y, x3.x, acc.x);
+    acc.y = fma(a23.y, x3.y, acc.y);
+  }
+  return acc;
+}
 
 // ------------------------------------------------------------ warp-cooperative block rows
 // The 32 lanes of a warp share one block row I: lane = slot * Wp + c with Wp a

@@ -30,7 +30,8 @@ constexpr int RMAX = 32;  // right-hand sides per panel
 
 struct RealSmem : Smem {
   int j[RMAX], mc[RMAX], off[RMAX + 1], on[RMAX], nc[RMAX], nact[RMAX], nfresh[RMAX], cst[RMAX];
-  double b2[RMAX], bprev[RMAX], c1[RMAX], c2[RMAX], c3[RMAX], s2[RMAX];
+  double b2[RMAX], c1prev[RMAX], c1[RMAX], c2[RMAX], c3[RMAX], s2[RMAX];
+  float2 f1[RMAX], f2[RMAX], f3[RMAX];  // c1, -c2, -c3 as float-floats
   int Mt[RMAX * 8];  // replay length per (column, 32-shift group)
   int Mc[RMAX];
 };
@@ -55,14 +56,14 @@ __device__ void gather_real(const Args& a, const RealSmem& sm, const SeedT<MIX>*
   const int R = 2 * a.W;
   if (a.full_hist) {  // every row of every column: row[cc * N4 + i]
     const int N4 = 4 * a.m.nb;
-    for (int e = threadIdx.x; e < N4 * R; e += TPB) {
+    for (int e = threadIdx.x; e < N4 * R; e += tpb()) {
       const int cc = e / N4, i = e - cc * N4;
       row[e] = pair_part(v[(size_t)i * a.W + (cc >> 1)], cc & 1);
     }
     return;
   }
   const int M = sm.off[R];
-  for (int e = threadIdx.x; e < M; e += TPB) {
+  for (int e = threadIdx.x; e < M; e += tpb()) {
     int cc = 0;
     while (sm.off[cc + 1] <= e) ++cc;
     const int i = a.m.col_idx[a.m.row_ptr[sm.j[cc]] + e - sm.off[cc]];
@@ -73,8 +74,8 @@ __device__ void gather_real(const Args& a, const RealSmem& sm, const SeedT<MIX>*
 template <bool MIX>
 __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dyn) {
   using V = SeedT<MIX>;
-  const int W = a.W, R = 2 * W, K = a.K, nb = a.m.nb, tid = threadIdx.x, c = tid % W;
-  const size_t NE = (size_t)4 * nb * W;
+  const int W = a.W, R = 2 * W, K = a.K, tid = threadIdx.x, c = tid % W;
+  const size_t NE = (size_t)4 * a.m.nb * W;
   V* s = wsp<V>(ws, a.o_r);    // s_n
   V* so = wsp<V>(ws, a.o_rt);  // s_{n-1}, then s_{n+1}
   V* v = wsp<V>(ws, a.o_w);
@@ -109,7 +110,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
     sm.cst[tid] = 0;
     sm.nact[tid] = 0;
     sm.nfresh[tid] = 0;
-    sm.bprev[tid] = 1.0;
+    sm.c1prev[tid] = 0.0;
     sm.c1[tid] = sm.c2[tid] = sm.c3[tid] = 0.0;
     sm.s2[tid] = 1.0;
   }
@@ -121,7 +122,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
     sm.inner_count = 0;
   }
   if (tid < W) sm.act[tid] = sm.on[2 * tid] | sm.on[2 * tid + 1];
-  for (int e = tid; e < RK; e += TPB) {
+  for (int e = tid; e < RK; e += tpb()) {
     nk[e] = sm.on[e / K] ? -1 : 0;
     resk[e] = 0.0;
     pis[2 * e] = make_double2(1.0, 0.0);
@@ -129,7 +130,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
     ck[2 * e] = make_double2(1.0, 0.0);
     ck[2 * e + 1] = make_double2(0.0, 0.0);
   }
-  for (size_t e = tid; e < NE; e += TPB) {
+  for (size_t e = tid; e < NE; e += tpb()) {
     const int row = (int)(e / W);
     const double x = sm.on[2 * c] && row == sm.j[2 * c] ? 1.0 : 0.0;
     const double y = sm.on[2 * c + 1] && row == sm.j[2 * c + 1] ? 1.0 : 0.0;
@@ -147,30 +148,61 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
 
   // v = S^-1 f and b2 = f^T v for the active pairs
   auto apply_sinv = [&](const V* f) {
-    if constexpr (MIX)
-      inner_mixed<true>(a, sm, f, v, cg_x, cg_g, cg_d, cg_q, dyn);
-    else
-      inner64(a, sm, f, v, cg_g, cg_d, cg_q, dyn);
     double d[2] = {0, 0};
-    gbff::acc d0, d1;
-    gbff::acc_init(d0);
-    gbff::acc_init(d1);
-    for (size_t e = tid; e < NE; e += TPB) {
-      if (!sm.act[c]) continue;
-      const V fv = f[e], vv = v[e];
-      if constexpr (MIX) {
+    if constexpr (MIX) {
+      gbff::acc d0, d1;
+      gbff::acc_init(d0);
+      gbff::acc_init(d1);
+      const int e0 = sm.act[c] ? tid : (int)NE;
+      const bool factor = a.inner_bchol != 0;
+      if (factor)
+        inner_real_factor(a, sm, f, cg_x, cg_g, cg_d, cg_q, U);
+      else
+        inner_mixed<true>(a, sm, f, v, cg_x, cg_g, cg_d, cg_q, dyn);
+      const float2 *x0 = cg_x, *x1 = cg_x + NE, *x2 = cg_g + NE, *x3 = cg_d + NE;
+#pragma unroll 2
+      for (int e = e0; e < (int)NE; e += tpb()) {
+        const float4 fv = f[e];
+        float4 vv;
+        if (factor) {  // v = the levels' sum, smallest first
+          gbff::ff p{0.f, 0.f}, q{0.f, 0.f};
+          if (a.bc_levels > 3) {
+            const float2 t = x3[e];
+            p.hi = t.x;
+            q.hi = t.y;
+          }
+          if (a.bc_levels > 2) {
+            const float2 t = x2[e];
+            p = gbff::two_sum(t.x, p.hi);
+            q = gbff::two_sum(t.y, q.hi);
+          }
+          if (a.bc_levels > 1) {
+            const float2 t = x1[e];
+            p = gbff::ff_add(gbff::ff{t.x, 0.f}, p);
+            q = gbff::ff_add(gbff::ff{t.y, 0.f}, q);
+          }
+          const float2 t = x0[e];
+          p = gbff::ff_add(gbff::ff{t.x, 0.f}, p);
+          q = gbff::ff_add(gbff::ff{t.y, 0.f}, q);
+          vv = make_float4(p.hi, p.lo, q.hi, q.lo);
+          v[e] = vv;
+        } else {
+          vv = v[e];
+        }
         gbff::acc_mul_add(d0, gbff::ff{fv.x, fv.y}, gbff::ff{vv.x, vv.y});
         gbff::acc_mul_add(d1, gbff::ff{fv.z, fv.w}, gbff::ff{vv.z, vv.w});
-      } else {
+      }
+      block_reduce_acc(d0, d1, W, sm.rs);
+    } else {
+      inner64(a, sm, f, v, cg_g, cg_d, cg_q, dyn);
+#pragma unroll 4
+      for (size_t e = sm.act[c] ? tid : NE; e < NE; e += tpb()) {
+        const V fv = f[e], vv = v[e];
         d[0] = fma(fv.x, vv.x, d[0]);
         d[1] = fma(fv.y, vv.y, d[1]);
       }
+      block_reduce_tree<2>(d, W, sm.rs);
     }
-    if constexpr (MIX) {
-      d[0] = gbff::acc_to_double(d0);
-      d[1] = gbff::acc_to_double(d1);
-    }
-    block_reduce<2>(d, W, sm.rs);
     if (tid < R) sm.b2[tid] = sm.rs.scal[(tid & 1) * WMAX + (tid >> 1)];
     __syncthreads();
   };
@@ -197,56 +229,41 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
       gbff::acc d0, d1;
       gbff::acc_init(d0);
       gbff::acc_init(d1);
-      for (int it = tid; it < nb * W; it += TPB) {
+      for (int e = tid; e < (int)NE; e += tpb()) {
         if (!sm.act[c]) continue;
-        const int I = it / W;
+        const int row = e / W;
         if constexpr (MIX) {
-          gbff::acc x0[4], x1[4];
+          gbff::acc x0, x1;
           if (a.hp_fp32) {  // unrefined FP32 product: U = H hi(v), accumulated in FP32
-            float2 acc[4];
-            bsr_row_fhi(a.m, a.m.hb_hi, v, W, c, I, acc);
-#pragma unroll
-            for (int rr = 0; rr < 4; ++rr) {
-              x0[rr] = gbff::acc{acc[rr].x, 0.f};
-              x1[rr] = gbff::acc{acc[rr].y, 0.f};
-            }
+            const float2 u = row_f(a.m, a.m.hb_hi, v, W, c, row);
+            x0 = gbff::acc{u.x, 0.f};
+            x1 = gbff::acc{u.y, 0.f};
           } else {
-            bsr_row_ff(a.m, a.m.hb_hi, a.m.hb_lo, v, W, c, I, x0, x1);
+            row_ff(a.m, a.m.hb_hi, a.m.hb_lo, v, W, c, row, x0, x1);
           }
-#pragma unroll
-          for (int rr = 0; rr < 4; ++rr) {
-            const size_t e = (size_t)(4 * I + rr) * W + c;
-            const gbff::ff u0 = gbff::acc_get(x0[rr]), u1 = gbff::acc_get(x1[rr]);
-            const float4 vv = v[e];
-            U[e] = make_float4(u0.hi, u0.lo, u1.hi, u1.lo);
-            gbff::acc_mul_add(d0, gbff::ff{vv.x, vv.y}, u0);
-            gbff::acc_mul_add(d1, gbff::ff{vv.z, vv.w}, u1);
-          }
+          const gbff::ff u0 = gbff::acc_get(x0), u1 = gbff::acc_get(x1);
+          const float4 vv = v[e];
+          U[e] = make_float4(u0.hi, u0.lo, u1.hi, u1.lo);
+          gbff::acc_mul_add(d0, gbff::ff{vv.x, vv.y}, u0);
+          gbff::acc_mul_add(d1, gbff::ff{vv.z, vv.w}, u1);
         } else {
-          double2 acc[4];
-          bsr_row_d(a.m, a.m.hb, v, W, c, I, acc);
-#pragma unroll
-          for (int rr = 0; rr < 4; ++rr) {
-            const size_t e = (size_t)(4 * I + rr) * W + c;
-            const double2 vv = v[e];
-            U[e] = acc[rr];
-            d[0] = fma(vv.x, acc[rr].x, d[0]);
-            d[1] = fma(vv.y, acc[rr].y, d[1]);
-          }
+          const double2 u = row_d(a.m, a.m.hb, v, W, c, row), vv = v[e];
+          U[e] = u;
+          d[0] = fma(vv.x, u.x, d[0]);
+          d[1] = fma(vv.y, u.y, d[1]);
         }
       }
-      if constexpr (MIX) {
-        d[0] = gbff::acc_to_double(d0);
-        d[1] = gbff::acc_to_double(d1);
-      }
-      block_reduce<2>(d, W, sm.rs);
+      if constexpr (MIX)
+        block_reduce_acc(d0, d1, W, sm.rs);
+      else
+        block_reduce_tree<2>(d, W, sm.rs);
       if (tid < R) {
         double c1 = 0.0, c2 = 0.0, c3 = 0.0;
         if (sm.on[tid]) {
-          const double b2 = sm.b2[tid], b = sqrt(b2);
-          c1 = 1.0 / b;
-          c2 = sm.rs.scal[(tid & 1) * WMAX + (tid >> 1)] / (b2 * b);
-          c3 = n > 0 ? b / sm.bprev[tid] : 0.0;
+          const double b2 = sm.b2[tid];
+          c1 = rsqrt(b2);
+          c2 = sm.rs.scal[(tid & 1) * WMAX + (tid >> 1)] * (c1 * c1) * c1;
+          c3 = b2 * c1 * sm.c1prev[tid];
           if (!(b2 > 0.0) || !isfinite(c1) || !isfinite(c2) || !isfinite(c3)) {
             // s^T S^-1 s <= 0 for a nonzero s: S is not positive definite
             sm.cst[tid] |= b2 < 0.0 ? kStNotSPD : kStBreakdown;
@@ -254,7 +271,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
             sm.nc[tid] = n;
             c1 = c2 = c3 = 0.0;
           } else {
-            sm.bprev[tid] = b;
+            sm.c1prev[tid] = c1;
             double* h = hc + ((size_t)n * R + tid) * 3;
             h[0] = c1;
             h[1] = c2;
@@ -264,6 +281,12 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
         sm.c1[tid] = c1;
         sm.c2[tid] = c2;
         sm.c3[tid] = c3;
+        if constexpr (MIX) {
+          const gbff::ff g1 = gbff::ff_from_double(c1), g2 = gbff::ff_from_double(-c2), g3 = gbff::ff_from_double(-c3);
+          sm.f1[tid] = make_float2(g1.hi, g1.lo);
+          sm.f2[tid] = make_float2(g2.hi, g2.lo);
+          sm.f3[tid] = make_float2(g3.hi, g3.lo);
+        }
         sm.nact[tid] = 0;
         sm.nfresh[tid] = 0;
       }
@@ -275,15 +298,13 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
       gbff::acc d0, d1;
       gbff::acc_init(d0);
       gbff::acc_init(d1);
-      const double p0 = sm.c1[2 * c], p1 = sm.c1[2 * c + 1], q0 = sm.c2[2 * c], q1 = sm.c2[2 * c + 1];
-      const double t0 = sm.c3[2 * c], t1 = sm.c3[2 * c + 1];
       float m0 = 0.f, m1 = 0.f;  // max |s|, for the factor solve's scale
       if constexpr (MIX) {
-        const gbff::ff fp0 = gbff::ff_from_double(p0), fp1 = gbff::ff_from_double(p1);
-        const gbff::ff fq0 = gbff::ff_from_double(-q0), fq1 = gbff::ff_from_double(-q1);
-        const gbff::ff ft0 = gbff::ff_from_double(-t0), ft1 = gbff::ff_from_double(-t1);
-        for (size_t e = tid; e < NE; e += TPB) {
-          if (!sm.act[c]) continue;
+        const gbff::ff fp0{sm.f1[2 * c].x, sm.f1[2 * c].y}, fp1{sm.f1[2 * c + 1].x, sm.f1[2 * c + 1].y};
+        const gbff::ff fq0{sm.f2[2 * c].x, sm.f2[2 * c].y}, fq1{sm.f2[2 * c + 1].x, sm.f2[2 * c + 1].y};
+        const gbff::ff ft0{sm.f3[2 * c].x, sm.f3[2 * c].y}, ft1{sm.f3[2 * c + 1].x, sm.f3[2 * c + 1].y};
+#pragma unroll 2
+        for (size_t e = sm.act[c] ? tid : NE; e < NE; e += tpb()) {
           const float4 u = U[e], x = s[e], y = so[e];
           const gbff::ff r0 = gbff::ff_add(gbff::ff_mul(fp0, gbff::ff{u.x, u.y}),
                                            gbff::ff_add(gbff::ff_mul(fq0, gbff::ff{x.x, x.y}),
@@ -297,12 +318,12 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
           gbff::acc_mul_add(d0, r0, r0);
           gbff::acc_mul_add(d1, r1, r1);
         }
-        d[0] = gbff::acc_to_double(d0);
-        d[1] = gbff::acc_to_double(d1);
         col_max(sm, W, m0, m1);
       } else {
-        for (size_t e = tid; e < NE; e += TPB) {
-          if (!sm.act[c]) continue;
+        const double p0 = sm.c1[2 * c], p1 = sm.c1[2 * c + 1], q0 = sm.c2[2 * c], q1 = sm.c2[2 * c + 1];
+        const double t0 = sm.c3[2 * c], t1 = sm.c3[2 * c + 1];
+#pragma unroll 2
+        for (size_t e = sm.act[c] ? tid : NE; e < NE; e += tpb()) {
           const double2 u = U[e], x = s[e], y = so[e];
           const double r0 = fma(p0, u.x, fma(-q0, x.x, -t0 * y.x)), r1 = fma(p1, u.y, fma(-q1, x.y, -t1 * y.y));
           so[e] = make_double2(r0, r1);
@@ -310,7 +331,10 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
           d[1] = fma(r1, r1, d[1]);
         }
       }
-      block_reduce<2>(d, W, sm.rs);
+      if constexpr (MIX)
+        block_reduce_acc(d0, d1, W, sm.rs);
+      else
+        block_reduce_tree<2>(d, W, sm.rs);
       if (tid < R && sm.on[tid]) {
         const double s2 = sm.rs.scal[(tid & 1) * WMAX + (tid >> 1)];
         if (isfinite(s2)) {
@@ -328,7 +352,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
     }
 
     // shift polynomials, convergence, checkpoints
-    for (int e = tid; e < RK; e += TPB) {
+    for (int e = tid; e < RK; e += tpb()) {
       const int cc = e / K;
       if (!sm.on[cc] || nk[e] >= 0) continue;
       const double2 cur = pis[2 * e], nxt = real_step(cur, pis[2 * e + 1], sm.c1[cc], sm.c2[cc], sm.c3[cc], a.z[e - cc * K]);
@@ -382,7 +406,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
     sm.cst[tid] |= kStNoConv;
   }
   __syncthreads();
-  for (int e = tid; e < RK; e += TPB) {
+  for (int e = tid; e < RK; e += tpb()) {
     const int cc = e / K;
     if (sm.mc[cc] != 0 && nk[e] < 0) {
       nk[e] = sm.nc[cc];
@@ -396,7 +420,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
   // F1: backward sums per (column, 32 shifts), the polynomials replayed from checkpoints
   {
     const int lane = tid & 31, warp = tid >> 5;
-    for (int task = warp; task < R * KG; task += NWARP) {
+    for (int task = warp; task < R * KG; task += nwarp()) {
       const int cc = task / KG, kg = task - cc * KG;
       if (sm.mc[cc] == 0) {
         if (lane == 0) sm.Mt[task] = 0;
@@ -479,7 +503,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
   if (a.has_rho || a.has_edm) {
     int mmax = 0;
     for (int i = 0; i < R; ++i) mmax = max(mmax, sm.Mc[i]);
-    for (int e = tid; e < mmax * R; e += TPB) {
+    for (int e = tid; e < mmax * R; e += tpb()) {
       const int m = e / R, cc = e - m * R;
       if (m >= sm.Mc[cc]) continue;
       double sr = 0.0, se = 0.0;
@@ -495,7 +519,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
     __syncthreads();
     // F3: rho_ij = sum_m C^rho_m v_m[i], edm_ij likewise
     const int Mt_ = sm.off[R];
-    for (int e = tid; e < Mt_; e += TPB) {
+    for (int e = tid; e < Mt_; e += tpb()) {
       int cc = 0;
       while (sm.off[cc + 1] <= e) ++cc;
       const int t = e - sm.off[cc];
@@ -536,7 +560,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
   if (cgs && a.g_proj) {
     __syncthreads();
     const int Mt_ = sm.off[R];
-    for (int e = tid; e < Mt_ * K; e += TPB) {
+    for (int e = tid; e < Mt_ * K; e += tpb()) {
       const int k = e / Mt_, f = e - k * Mt_;
       int cc = 0;
       while (sm.off[cc + 1] <= f) ++cc;

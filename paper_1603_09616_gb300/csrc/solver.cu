@@ -956,16 +956,17 @@ const void* batched_fn(bool fp64, bool real) {
     return fp64 ? (const void*)gbk::team_kernel_batched<false, true> : (const void*)gbk::team_kernel_batched<true, true>;
   return fp64 ? (const void*)gbk::team_kernel_batched<false, false> : (const void*)gbk::team_kernel_batched<true, false>;
 }
-gb_status launch_team(gbk::Args& a, bool fp64, bool real, int teams, size_t dyn, cudaStream_t s) {
+gb_status launch_team(gbk::Args& a, bool fp64, bool real, int teams, int threads, size_t dyn, cudaStream_t s) {
   const void* fn = team_fn(fp64, real);
   GB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
   void* args[] = {&a};
-  GB_CUDA(cudaLaunchKernel(fn, dim3(teams), dim3(gbk::TPB), args, dyn, s));
+  GB_CUDA(cudaLaunchKernel(fn, dim3(teams), dim3(threads), args, dyn, s));
   return GB_OK;
 }
 
 struct Plan {
   int C;  // right-hand sides per panel
+  int threads;
   bool real;
   int W, KG, npanels, teams, teams_per_sm, Mcap, inner_maxit, cg_smem;
   size_t dyn_smem;
@@ -1035,11 +1036,23 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
     // panels (measured on the 1900-orbital chain: 8 columns, 238 panels on 304
     // slots, ~20% faster than 4)
     C = 1;
-    for (int cand : {32, 16, 8, 4, 2}) {
-      const size_t dyn = dyn_bytes(width(cand));
-      if (4LL * ((p->nrhs + cand - 1) / cand) >= 3LL * nsm * occupancy(dyn)) {
-        C = cand;
-        break;
+    if (real && !f64) {
+      // one wide team per SM: the narrowest panels that fit one wave (912
+      // orbitals, all columns: 8 columns 275 us an iteration, 4 columns two teams
+      // per SM 325, 16 columns 427; 1900 orbitals: 16 columns 490, 8 columns 502)
+      C = 2;
+      while (C < 32 && (p->nrhs + C - 1) / C > nsm) C *= 2;
+    }
+    if (C == 1 || (p->nrhs + C - 1) / C > nsm) {
+      // two teams per SM: one wave that fills >= 3/4 of the team slots beats 1.5
+      // waves of half-size panels
+      C = 1;
+      for (int cand : {32, 16, 8, 4, 2}) {
+        const size_t dyn = dyn_bytes(width(cand));
+        if (4LL * ((p->nrhs + cand - 1) / cand) >= 3LL * nsm * occupancy(dyn)) {
+          C = cand;
+          break;
+        }
       }
     }
     if (real && C == 1 && p->nrhs > 1) C = 2;  // a pair costs what one of its columns does
@@ -1056,6 +1069,8 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
   pl->KG = (p->nshift + 31) / 32;
   pl->npanels = (p->nrhs + C - 1) / C;
   pl->teams = std::min(pl->npanels, nsm * pl->teams_per_sm);
+  // one wide team per SM where the launch would leave SMs with a single team
+  pl->threads = real && !f64 && pl->npanels <= nsm ? gbk::TPB_WIDE : gbk::TPB;
   pl->Mcap = full_hist ? (real ? 2 * W : W) * 4 * (int)m->nb : C * m->max_row;
   pl->inner_maxit = 500;
   // Inner-solve accuracy: the seed recurrence treats w = S^{-1} H p as exact,
@@ -1197,7 +1212,7 @@ gb_status gb_shifted_solve(const gb_matrix* m, const gb_solve_params* p, const g
   a.P = ho[nrhs];
 
   a.cg_smem = pl.cg_smem;
-  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, pl.teams, pl.dyn_smem, s)) != GB_OK) return st;
+  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, pl.teams, pl.threads, pl.dyn_smem, s)) != GB_OK) return st;
   std::vector<int> hst(nrhs);
   GB_CUDA(cudaMemcpyAsync(hst.data(), a.status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
   GB_CUDA(cudaStreamSynchronize(s));
@@ -1239,7 +1254,7 @@ __global__ void __launch_bounds__(gbk::TPB, 1)
     }
     gbk::col_max(sm, a.W, m0, m1);
     __syncthreads();
-    gbk::fx_solve(a, sm, x, y, t1, t2);
+    gbk::fx_solve<true>(a, sm, x, y, t1, t2);
   } else {
     gbk::bc_solve64(a, sm, x, y, t1, t2);
   }
@@ -1539,7 +1554,7 @@ gb_status gb_true_residual(const gb_matrix* m, const gb_solve_params* p, int32_t
   a.Mcap = pl.Mcap;
   a.iters = reinterpret_cast<int*>(wsb + L.o_im);
   a.cg_smem = pl.cg_smem;
-  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, pl.teams, pl.dyn_smem, s)) != GB_OK) return st;
+  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, pl.teams, pl.threads, pl.dyn_smem, s)) != GB_OK) return st;
   double2* X = reinterpret_cast<double2*>(wsb + L.o_x);
   {
     const dim3 grid((unsigned)((N4 + 63) / 64), (unsigned)((K + 31) / 32), (unsigned)nver);
@@ -2165,7 +2180,7 @@ gb_status gb_shifted_solve_static(const gb_matrix* m, const gb_solve_params* p, 
   a.g_proj = reinterpret_cast<double2*>(out->g_proj);
   a.P = ho[nrhs];
   a.cg_smem = pl.cg_smem;
-  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, teams, pl.dyn_smem, s)) != GB_OK) return st;
+  if ((st = launch_team(a, p->prec == GB_FP64, pl.real, teams, pl.threads, pl.dyn_smem, s)) != GB_OK) return st;
   GB_CUDA(cudaMemcpyAsync(g_static_status, a.status, sizeof(int) * nrhs, cudaMemcpyDeviceToHost, s));
   GB_CUDA(cudaStreamSynchronize(s));
   int any = 0;
@@ -2188,7 +2203,7 @@ size_t gb_static_scratch_bytes(void) { return kStaticScratchBytes; }
 namespace {
 
 struct BatchPlan {
-  int C, W, teams, total_panels, maxK, maxit, Mcap, KG;
+  int C, W, teams, threads, total_panels, maxK, maxit, Mcap, KG;
   bool real, mixed, want_g;
   size_t N4, team_bytes, header_bytes, total, dyn_smem;
   std::vector<int> order;  // systems, largest estimated cost first
@@ -2241,14 +2256,23 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   };
   int C = panel;
   if (C <= 0) {  // widest panel that still gives every resident team a work item
-    C = 1;
-    for (int cand : {32, 16, 8, 4, 2}) {
+    auto panels = [&](int cand) {
       long long np = 0;
       for (int s = 0; s < nsys; ++s) np += (params[s].nrhs + cand - 1) / cand;
-      if (4 * np >= 3LL * nsm * occupancy(dyn_bytes(width(cand)))) {
-        C = cand;
-        break;
-      }
+      return np;
+    };
+    C = 1;
+    if (real && prec == GB_MIXED) {  // as in make_plan
+      C = 2;
+      while (C < 32 && panels(C) > nsm) C *= 2;
+    }
+    if (C == 1 || panels(C) > nsm) {
+      C = 1;
+      for (int cand : {32, 16, 8, 4, 2})
+        if (4 * panels(cand) >= 3LL * nsm * occupancy(dyn_bytes(width(cand)))) {
+          C = cand;
+          break;
+        }
     }
     if (real && C == 1) C = 2;  // a pair costs what one of its columns does
   }
@@ -2273,6 +2297,7 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   bp->total_panels = 0;
   for (int s = 0; s < nsys; ++s) bp->total_panels += (params[s].nrhs + C - 1) / C;
   bp->teams = std::min(bp->total_panels, nsm * per_sm);
+  bp->threads = real && prec != GB_FP64 && bp->total_panels <= nsm ? gbk::TPB_WIDE : gbk::TPB;
   // largest systems first (cost ~ basis size x shifts) for load balance
   bp->order.resize(nsys);
   for (int s = 0; s < nsys; ++s) bp->order[s] = s;
@@ -2432,7 +2457,7 @@ gb_status gb_shifted_solve_batched(int32_t nsys, const gb_matrix* const* mats, c
     const void* fn = batched_fn(!bp.mixed, bp.real);
     GB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.dyn_smem));
     void* args[] = {&d_desc, &d_prefix, &nsys, &d_counter, &team_ws, &bp.team_bytes};
-    GB_CUDA(cudaLaunchKernel(fn, dim3(bp.teams), dim3(gbk::TPB), args, bp.dyn_smem, s));
+    GB_CUDA(cudaLaunchKernel(fn, dim3(bp.teams), dim3(bp.threads), args, bp.dyn_smem, s));
   }
   GB_CUDA(cudaMemcpyAsync(hdr.data(), wsb, bp.header_bytes, cudaMemcpyDeviceToHost, s));
   GB_CUDA(cudaStreamSynchronize(s));

@@ -21,8 +21,14 @@ struct Team<MIX, true> {
   __device__ __forceinline__ void solve(const Args& a, char* ws, char* dyn) { solve_panel_real<MIX>(a, sm, ws, dyn); }
 };
 
+// 64 registers a thread either way: two teams of TPB threads per SM, or one of TPB_WIDE
 template <bool MIX, bool REAL>
-__global__ void __launch_bounds__(TPB, MIN_TEAMS_PER_SM) team_kernel(const __grid_constant__ Args a) {
+constexpr int kMaxThreads = MIX && REAL ? TPB_WIDE : TPB;
+template <bool MIX, bool REAL>
+constexpr int kMinTeams = MIX && REAL ? MIN_TEAMS_PER_SM / 2 : MIN_TEAMS_PER_SM;
+
+template <bool MIX, bool REAL>
+__global__ void __launch_bounds__(kMaxThreads<MIX, REAL>, kMinTeams<MIX, REAL>) team_kernel(const __grid_constant__ Args a) {
   __shared__ Team<MIX, REAL> team;
   auto& sm = team.sm;
   extern __shared__ __align__(16) char dyn_smem[];
@@ -50,7 +56,7 @@ __global__ void __launch_bounds__(TPB, MIN_TEAMS_PER_SM) team_kernel(const __gri
 // memory and runs the same panel solver.  The team workspace is laid out for
 // the largest system.
 template <bool MIX, bool REAL>
-__global__ void __launch_bounds__(TPB, MIN_TEAMS_PER_SM)
+__global__ void __launch_bounds__(kMaxThreads<MIX, REAL>, kMinTeams<MIX, REAL>)
     team_kernel_batched(const Args* __restrict__ sys, const int* __restrict__ panel_prefix, int nsys,
                         int* __restrict__ counter, char* team_ws, size_t team_bytes) {
   __shared__ Team<MIX, REAL> team;
@@ -80,7 +86,7 @@ __global__ void __launch_bounds__(TPB, MIN_TEAMS_PER_SM)
     if (s_sys < 0) return;
     const unsigned* src = reinterpret_cast<const unsigned*>(sys + s_sys);
     unsigned* dst = reinterpret_cast<unsigned*>(&sa);
-    for (int i = threadIdx.x; i < (int)(sizeof(Args) / sizeof(unsigned)); i += TPB) dst[i] = src[i];
+    for (int i = threadIdx.x; i < (int)(sizeof(Args) / sizeof(unsigned)); i += tpb()) dst[i] = src[i];
     __syncthreads();
     team.solve(sa, ws, dyn_smem);
     __syncthreads();

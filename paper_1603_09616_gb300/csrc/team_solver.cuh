@@ -337,12 +337,12 @@ __device__ __noinline__ void cg32_loop(const Args& a, Smem& sm, float2* __restri
 #if GB_WARP_SPMM
       const int lane = threadIdx.x & 31;
       const bool act = sm.act[c] != 0;
-      for (int I = threadIdx.x >> 5; I < nb; I += NWARP) {
+      for (int I = threadIdx.x >> 5; I < nb; I += nwarp()) {
         float2 acc[4];
         wbsr_row_f(a.m, a.m.sb_hi, d, W, W, lane, I, act, acc);
         if (lane < W && act) {
 #else
-      for (int it = threadIdx.x; it < nb * W; it += TPB) {
+      for (int it = threadIdx.x; it < nb * W; it += tpb()) {
         if (!sm.act[c]) continue;
         const int I = it / W;
         float2 acc[4];
@@ -381,7 +381,7 @@ __device__ __noinline__ void cg32_loop(const Args& a, Smem& sm, float2* __restri
     {
       float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
       const float ar = (float)sm.cg_a[2 * c], ai = (float)sm.cg_a[2 * c + 1];
-      for (int it = threadIdx.x; it < nb * W; it += TPB) {
+      for (int it = threadIdx.x; it < nb * W; it += tpb()) {
         if (!sm.act[c]) continue;
         const int I = it / W;
         float2 gv[4];
@@ -426,7 +426,7 @@ __device__ __noinline__ void cg32_loop(const Args& a, Smem& sm, float2* __restri
       __syncthreads();
     }
     const float br = (float)sm.cg_b[2 * c], bi = (float)sm.cg_b[2 * c + 1];
-    for (int e = threadIdx.x; e < 4 * nb * W; e += TPB) {
+    for (int e = threadIdx.x; e < 4 * nb * W; e += tpb()) {
       if (!sm.act[c]) continue;
       const float2 zv = q[e];
       float2 dv = d[e];
@@ -453,7 +453,7 @@ __device__ __noinline__ void cheb32_loop(const Args& a, Smem& sm, float2* __rest
     const bool last = k + 1 == a.cheb_K, even = !(k & 1);
     const float2* __restrict__ dk = (k & 1) ? dB : dA;
     float2* __restrict__ dn = (k & 1) ? dA : dB;
-    for (int it = threadIdx.x; it < nb * W; it += TPB) {
+    for (int it = threadIdx.x; it < nb * W; it += tpb()) {
       if (!sm.act[c]) continue;
       const int I = it / W;
       float2 acc[4];
@@ -521,8 +521,7 @@ __device__ __forceinline__ void cg_start_scalars(Smem& sm, int W) {
 // ------------------------------------------------------------ inner solve, mixed
 // w = S^{-1} U to ~FP64 accuracy: FP32 CG on hi(U), a float-float residual
 // e = U - S x1, FP32 CG on e, w = x1 + x2 (float-float).
-template <bool REAL>
-__device__ __noinline__ void inner_mixed_factor(const Args& a, Smem& sm, const float4* __restrict__ U, float4* __restrict__ w,
+__device__ __noinline__ void inner_seed_factor(const Args& a, Smem& sm, const float4* __restrict__ U, float4* __restrict__ w,
                                    float2* __restrict__ x, float2* __restrict__ g, float2* __restrict__ d,
                                    float2* __restrict__ q, char* dyn);
 
@@ -530,15 +529,17 @@ template <bool REAL>
 __device__ __noinline__ void inner_mixed(const Args& a, Smem& sm, const float4* __restrict__ U, float4* __restrict__ w,
                             float2* __restrict__ x, float2* __restrict__ g, float2* __restrict__ d,
                             float2* __restrict__ q, char* dyn) {
-  if (a.inner_bchol) {
-    inner_mixed_factor<REAL>(a, sm, U, w, x, g, d, q, dyn);
-    return;
+  if constexpr (!REAL) {
+    if (a.inner_bchol) {
+      inner_seed_factor(a, sm, U, w, x, g, d, q, dyn);
+      return;
+    }
   }
   const int W = a.W, nb = a.m.nb, c = threadIdx.x % W;
   const double itol = a.itol;
   {  // level 1 start: g = hi(U), d = M^-1 g, x = 0
     float f0 = 0.f, f1 = 0.f, f2 = 0.f, f3 = 0.f;
-    for (int it = threadIdx.x; it < nb * W; it += TPB) {
+    for (int it = threadIdx.x; it < nb * W; it += tpb()) {
       if (!sm.act[c]) continue;
       const int I = it / W;
       float2 gv[4];
@@ -578,12 +579,12 @@ __device__ __noinline__ void inner_mixed(const Args& a, Smem& sm, const float4* 
 #if GB_WARP_SPMM
     const int lane = threadIdx.x & 31;
     const bool act = sm.act[c] != 0;
-    for (int I = threadIdx.x >> 5; I < nb; I += NWARP) {
+    for (int I = threadIdx.x >> 5; I < nb; I += nwarp()) {
       gbff::acc are[4], aim[4];
       wbsr_row_ffx(a.m, a.m.sb_hi, a.m.sb_lo, x, W, W, lane, I, act, are, aim);
       if (lane >= W || !act) continue;
 #else
-    for (int it = threadIdx.x; it < nb * W; it += TPB) {
+    for (int it = threadIdx.x; it < nb * W; it += tpb()) {
       if (!sm.act[c]) continue;
       const int I = it / W;
       gbff::acc are[4], aim[4];
@@ -615,7 +616,7 @@ __device__ __noinline__ void inner_mixed(const Args& a, Smem& sm, const float4* 
     }
     double v[4] = {f0, f1, f2, f3};
     block_reduce<4>(v, W, sm.rs);  // contains the barrier that ends all reads of x1
-    for (int e = threadIdx.x; e < 4 * nb * W; e += TPB) {
+    for (int e = threadIdx.x; e < 4 * nb * W; e += tpb()) {
       if (!sm.act[c]) continue;
       const float2 xv = x[e];
       w[e] = make_float4(xv.x, 0.f, xv.y, 0.f);
@@ -627,7 +628,7 @@ __device__ __noinline__ void inner_mixed(const Args& a, Smem& sm, const float4* 
     cheb32_loop(a, sm, x, g, d, q);
   else
     cg32_loop(a, sm, x, g, d, q, itol);
-  for (int e = threadIdx.x; e < 4 * nb * W; e += TPB) {
+  for (int e = threadIdx.x; e < 4 * nb * W; e += tpb()) {
     if (!sm.act[c]) continue;
     const float4 wv = w[e];
     const float2 xv = x[e];
@@ -645,11 +646,10 @@ __device__ __noinline__ void inner_mixed(const Args& a, Smem& sm, const float4* 
 // levels give ~1e-13 and three ~1e-19 (a.bc_levels, set from the tolerance).
 // g = U - S v (float-float) for the active columns; v is the FP32 vector x
 // (XV = float2) or the float-float w (XV = float4).  No barrier.
-template <bool REAL, typename XV>
-__device__ __noinline__ void ff_residual(const Args& a, Smem& sm, const float4* __restrict__ U,
+template <typename XV>
+__device__ __noinline__ void ff_residual(const Args& a, const Smem& sm, const float4* __restrict__ U,
                                          const XV* __restrict__ v, float2* __restrict__ g) {
   const int W = a.W, nb = a.m.nb, c = threadIdx.x % W;
-  float m0 = 0.f, m1 = 0.f;
   for (int it = threadIdx.x; it < nb * W; it += TPB) {
     if (!sm.act[c]) continue;
     const int I = it / W;
@@ -664,31 +664,22 @@ __device__ __noinline__ void ff_residual(const Args& a, Smem& sm, const float4* 
       const float4 u = U[e];
       const gbff::ff er = gbff::ff_sub(gbff::ff{u.x, u.y}, gbff::acc_get(are[r]));
       const gbff::ff ei = gbff::ff_sub(gbff::ff{u.z, u.w}, gbff::acc_get(aim[r]));
-      const float2 gv = make_float2(er.hi + er.lo, ei.hi + ei.lo);
-      g[e] = gv;
-      m0 = fmaxf(m0, fabsf(gv.x));
-      m1 = fmaxf(m1, fabsf(gv.y));
+      g[e] = make_float2(er.hi + er.lo, ei.hi + ei.lo);
     }
   }
-  if (REAL) col_max(sm, W, m0, m1);
 }
 
-// Real recurrence: U's column maxima must have been left in sm.fmax (col_max, then a barrier).
-template <bool REAL>
-__device__ __noinline__ void inner_mixed_factor(const Args& a, Smem& sm, const float4* __restrict__ U, float4* __restrict__ w,
+__device__ __noinline__ void inner_seed_factor(const Args& a, Smem& sm, const float4* __restrict__ U, float4* __restrict__ w,
                                    float2* __restrict__ x, float2* __restrict__ g, float2* __restrict__ d,
                                    float2* __restrict__ q, char* dyn) {
   const int W = a.W, nb = a.m.nb, c = threadIdx.x % W;
-  if constexpr (REAL)
-    fx_solve(a, sm, U, x, d, q);
-  else
-    seed_solve(a, sm, U, x, d);
+  seed_solve(a, sm, U, x, d);
   for (int lev = 1; lev < a.bc_levels; ++lev) {
     // e = U - S w into g; at the first refinement w = x1 is the FP32 vector x
     if (lev == 1)
-      ff_residual<REAL>(a, sm, U, x, g);
+      ff_residual(a, sm, U, x, g);
     else
-      ff_residual<REAL>(a, sm, U, w, g);
+      ff_residual(a, sm, U, w, g);
     __syncthreads();  // every read of x / w for the residual is done
     if (lev == 1) {
       for (int e = threadIdx.x; e < 4 * nb * W; e += TPB) {
@@ -698,10 +689,7 @@ __device__ __noinline__ void inner_mixed_factor(const Args& a, Smem& sm, const f
       }
       __syncthreads();
     }
-    if constexpr (REAL)
-      fx_solve(a, sm, g, x, d, q);
-    else
-      seed_solve(a, sm, g, x, d);
+    seed_solve(a, sm, g, x, d);
     for (int e = threadIdx.x; e < 4 * nb * W; e += TPB) {
       if (!sm.act[c]) continue;
       const float4 wv = w[e];
@@ -719,6 +707,61 @@ __device__ __noinline__ void inner_mixed_factor(const Args& a, Smem& sm, const f
       w[e] = make_float4(xv.x, 0.f, xv.y, 0.f);
     }
     __syncthreads();
+  }
+}
+
+// The same refinement for the real recurrence (W pairs of real columns).  The
+// residual is updated, not formed anew: e1 = U - S x0 and e2 = e1 - S x1 with the
+// float-float S and an FP32 x (products of a float-float and an FP32 vector are the
+// cheaper ones), e1 kept as float-float because e2 is its 1e-6.  From there on e is
+// below 1e-12 of U, and one FP32 rounding of it is beyond U's own 2^-48: e3 = e2 -
+// S x2 is a plain FP32 product.  er: a
+// panel-sized float-float scratch.  U's column maxima must have been left in
+// sm.fmax (col_max, then a barrier).  Ends with a barrier.
+template <int LEV>
+__device__ __noinline__ void real_residual(const Args& a, Smem& sm, const float4* f, const float2* x, float4* er,
+                                           float2* g) {
+  const int W = a.W, c = threadIdx.x % W, NE = 4 * a.m.nb * W;
+  float m0 = 0.f, m1 = 0.f;
+  for (int e = sm.act[c] ? threadIdx.x : NE; e < NE; e += tpb()) {
+    float2 o;
+    if constexpr (LEV < 3) {
+      gbff::acc a0, a1;
+      row_ffx(a.m, a.m.sb_hi, a.m.sb_lo, x, W, c, e / W, a0, a1);
+      const float4 u = LEV == 1 ? f[e] : er[e];
+      const gbff::ff r0 = gbff::ff_sub(gbff::ff{u.x, u.y}, gbff::acc_get(a0));
+      const gbff::ff r1 = gbff::ff_sub(gbff::ff{u.z, u.w}, gbff::acc_get(a1));
+      if (LEV == 1) er[e] = make_float4(r0.hi, r0.lo, r1.hi, r1.lo);
+      o = make_float2(r0.hi, r1.hi);
+    } else {
+      const float2 p = row_f(a.m, a.m.sb_hi, x, W, c, e / W), u = g[e];
+      o = make_float2(u.x - p.x, u.y - p.y);
+    }
+    if (LEV != 1) g[e] = o;
+    m0 = fmaxf(m0, fabsf(o.x));
+    m1 = fmaxf(m1, fabsf(o.y));
+  }
+  col_max(sm, W, m0, m1);
+  __syncthreads();
+}
+
+// x, g, d and q have room for two FP32 panels each: level l's solution goes to the
+// first half of x (l = 0) or the second of x, g, d (l = 1, 2, 3); the caller sums.
+__device__ __noinline__ void inner_real_factor(const Args& a, Smem& sm, const float4* U, float2* x, float2* g,
+                                               float2* d, float2* q, float4* er) {
+  const size_t NE = (size_t)4 * a.m.nb * a.W;
+  fx_solve(a, sm, U, x, d, q);
+  if (a.bc_levels > 1) {
+    real_residual<1>(a, sm, U, x, er, g);
+    fx_solve(a, sm, er, x + NE, d, q);
+  }
+  if (a.bc_levels > 2) {
+    real_residual<2>(a, sm, U, x + NE, er, g);
+    fx_solve(a, sm, g, g + NE, d, q);
+  }
+  if (a.bc_levels > 3) {
+    real_residual<3>(a, sm, U, g + NE, er, g);
+    fx_solve(a, sm, g, d + NE, d, q);
   }
 }
 
