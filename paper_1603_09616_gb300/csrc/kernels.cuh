@@ -61,6 +61,7 @@ struct DevMat {
   const int* col_idx;
   const double* h_val;
   const double* s_val;
+  const float* h_diag;  // H_ii
   double s_lam_min, s_lam_max;  // spectrum bounds of the block-Jacobi-preconditioned S
   // Block-bidiagonal Cholesky factor of S on 64-row blocks (bf_bw = 0: none).
   // FP64: four [bf_nblk][64][64] arrays, k-major (entry (r, k) at k * 64 + r):

@@ -499,6 +499,19 @@ __global__ void split_kernel(const double* __restrict__ v, size_t n, float* __re
   }
 }
 
+// The onsite energies (every row of the pattern has its diagonal entry).
+__global__ void diag_kernel(const gbk::DevMat m, float* __restrict__ d) {
+  const int i = blockIdx.x * 256 + threadIdx.x;
+  if (i >= m.n) return;
+  int lo = m.row_ptr[i], hi = m.row_ptr[i + 1];
+  while (lo < hi) {  // first column >= i of the sorted row
+    const int mid = (lo + hi) >> 1;
+    if (m.col_idx[mid] < i) lo = mid + 1;
+    else hi = mid;
+  }
+  d[i] = lo < m.row_ptr[i + 1] && m.col_idx[lo] == i ? (float)m.h_val[lo] : 0.f;
+}
+
 // The factor's tiles in MMA fragment order, one block of threads per 64-row block
 // and direction.  Element (r, k) of a 64 x 64 factor block lies at k * 64 + r.
 //
@@ -577,6 +590,7 @@ cudaError_t form_on_device(const gbk::DevMat& d, size_t nnzb, const FactorTiles&
   split(d.hb, nnzb * 16, d.hb_hi, d.hb_lo);
   split(d.sb, nnzb * 16, d.sb_hi, d.sb_lo);
   split(d.minv, (size_t)d.nb * 16, d.minv32, nullptr);
+  diag_kernel<<<(d.n + 255) / 256, 256, 0, s>>>(d, const_cast<float*>(d.h_diag));
   if (d.bf_nblk > 0) {
     TileArgs t{};
     t.bf = d.bf64;
@@ -672,7 +686,7 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   const size_t up = off;  // uploaded; the rest is formed from it on the device
   const size_t o_hh = take(sizeof(float) * nnzb * 16), o_hl = take(sizeof(float) * nnzb * 16);
   const size_t o_sh = take(sizeof(float) * nnzb * 16), o_sl = take(sizeof(float) * nnzb * 16);
-  const size_t o_m32 = take(sizeof(float) * nbl * 16);
+  const size_t o_m32 = take(sizeof(float) * nbl * 16), o_hd = take(sizeof(float) * n);
   const size_t o_bfm = take(sizeof(float) * 2 * nblk * gbk::kMmaTileFloatsDev);
   const size_t o_fx = take(sizeof(uint4) * 2 * nblk * gbk::fx_block_words(ft.ne));
   const size_t total = off;
@@ -724,6 +738,7 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   d.col_idx = reinterpret_cast<const int*>(b + o_ci);
   d.h_val = reinterpret_cast<const double*>(b + o_hv);
   d.s_val = reinterpret_cast<const double*>(b + o_sv);
+  d.h_diag = reinterpret_cast<const float*>(b + o_hd);
   d.s_lam_min = hb.lam_min;
   d.s_lam_max = hb.lam_max;
   d.bf_bw = nbf ? hb.bf_bw : 0;

@@ -25,7 +25,7 @@ constexpr float kRbfW = 0.03f;    // nm, radial Gaussian width
 
 __device__ __forceinline__ float cutoff_fn(float r) { return r < kRc ? 0.5f * (cospif(r / kRc) + 1.0f) : 0.0f; }
 
-// One thread per orbital j.  Features (all from the pattern row j, whose
+// One warp per orbital j.  Features (all from the pattern row j, whose
 // orbitals belong to the atoms within the interaction cutoff):
 //   0-15  radial Gaussians (centres 0.1..0.5 nm) over carbon neighbour atoms
 //   16-31 the same over hydrogen neighbour atoms
@@ -38,81 +38,118 @@ __device__ __forceinline__ float cutoff_fn(float r) { return r < kRc ? 0.5f * (c
 //         weighted by H_ji^2
 //   56 sum H_ji^2, 57 sum S_ji^2, 58 sum H_ji S_ji, 59 sum H_ji^2 H_ii,
 //   60 sum |H_ji|, 61 |R_j| / 100, 62 sum S_ji H_ii (all over i != j), 63 = 1
-__global__ void descriptor_kernel(const gbk::DevMat m, const float* __restrict__ pos, const int* __restrict__ orb_atom,
-                                  const int* __restrict__ atom_first, const int* __restrict__ species,
-                                  float* __restrict__ out) {
-  const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= m.n) return;
-  float f[kDesc];
-#pragma unroll
-  for (int k = 0; k < kDesc; ++k) f[k] = 0.f;
+//
+// The lanes take the row's entries (coalesced) and sum the coupling features in a
+// shuffle tree; each neighbour atom a lane finds is then shown to the whole warp,
+// lane t adding to radial feature t and lanes 0 .. 8 to the nine angular moments.
+// A row has ~126 entries and ~45 neighbour atoms: bound by issue, not by memory
+// (3420 orbitals, 20 bytes an entry: under 2 us of HBM).  One thread per orbital
+// with its 64 features in local memory and a search for every H_ii took 710 us for
+// 3420 orbitals (27 blocks of 128 threads).
+__global__ void __launch_bounds__(256)
+    descriptor_kernel(const gbk::DevMat m, const float* __restrict__ pos, const int* __restrict__ orb_atom,
+                      const int* __restrict__ atom_first, const int* __restrict__ species, float* __restrict__ out) {
+  const int j = (int)((blockIdx.x * 256LL + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+  if (j >= m.n) return;  // uniform per warp
   const int a = orb_atom[j];
   const float ax = pos[3 * a], ay = pos[3 * a + 1], az = pos[3 * a + 2];
-  float dip[4][3] = {};
-  float quad[4][6] = {};
   const int lo = m.row_ptr[j], hi = m.row_ptr[j + 1];
-  for (int e = lo; e < hi; ++e) {
-    const int i = m.col_idx[e];
-    const int b = orb_atom[i];
-    const double hji = m.h_val[e], sji = m.s_val[e];
-    if (i == j) {
-      f[46] = (float)hji;
-      f[47] = (float)sji;
-      continue;
-    }
-    // H_ii: diagonal entry of row i (binary search in the sorted row)
-    int l0 = m.row_ptr[i], l1 = m.row_ptr[i + 1] - 1;
-    while (l0 < l1) {
-      const int mid = (l0 + l1) >> 1;
-      if (m.col_idx[mid] < i) l0 = mid + 1;
-      else l1 = mid;
-    }
-    const float hii = (float)m.h_val[l0];
-    const float h2 = (float)(hji * hji);
-    for (int t = 0; t < 8; ++t) {
-      const float c = -3.0f + 6.0f * t / 7.0f, d = (hii - c) / 0.75f;
-      f[48 + t] += h2 * __expf(-d * d);
-    }
-    f[56] += h2;
-    f[57] += (float)(sji * sji);
-    f[58] += (float)(hji * sji);
-    f[59] += h2 * hii;
-    f[60] += fabsf((float)hji);
-    f[62] += (float)sji * hii;
-    if (b == a || i != atom_first[b]) continue;  // geometric part: each neighbour atom once
-    const float dx = pos[3 * b] - ax, dy = pos[3 * b + 1] - ay, dz = pos[3 * b + 2] - az;
-    const float r = sqrtf(dx * dx + dy * dy + dz * dz);
-    if (!(r > 1e-6f) || r >= kRc) continue;
-    const float w = cutoff_fn(r);
-    const int sb = species[b] ? 16 : 0;
-    for (int t = 0; t < 16; ++t) {
-      const float mu = 0.1f + 0.4f * t / 15.0f, d = (r - mu) / kRbfW;
-      f[sb + t] += w * __expf(-d * d);
-    }
-    const int sh = min(3, (int)(r / (kRc / 4)));
-    const float ux = dx / r, uy = dy / r, uz = dz / r;
-    dip[sh][0] += w * ux;
-    dip[sh][1] += w * uy;
-    dip[sh][2] += w * uz;
-    quad[sh][0] += w * (ux * ux - 1.0f / 3);
-    quad[sh][1] += w * (uy * uy - 1.0f / 3);
-    quad[sh][2] += w * (uz * uz - 1.0f / 3);
-    quad[sh][3] += w * ux * uy;
-    quad[sh][4] += w * ux * uz;
-    quad[sh][5] += w * uy * uz;
-  }
-  for (int s = 0; s < 4; ++s) {
-    f[32 + 2 * s] = dip[s][0] * dip[s][0] + dip[s][1] * dip[s][1] + dip[s][2] * dip[s][2];
-    f[33 + 2 * s] = quad[s][0] * quad[s][0] + quad[s][1] * quad[s][1] + quad[s][2] * quad[s][2] +
-                    2.f * (quad[s][3] * quad[s][3] + quad[s][4] * quad[s][4] + quad[s][5] * quad[s][5]);
-  }
-  f[40 + (species[a] ? 1 : 0)] = 1.f;
-  f[42 + min(3, j - atom_first[a])] = 1.f;
-  f[61] = (hi - lo) / 100.0f;
-  f[63] = 1.f;
   float* o = out + (size_t)j * kDesc;
+  float bin[8] = {}, sum[6] = {};  // sum: features 56 .. 60 and 62
+  float rad = 0.f, mom[4] = {}, hjj = 0.f, sjj = 0.f;
+  const float mu = 0.1f + 0.4f * (lane & 15) / 15.0f;
+  for (int e0 = lo; e0 < hi; e0 += 32) {
+    const int e = e0 + lane;
+    bool atom = false;
+    float r = 0.f, w = 0.f, ux = 0.f, uy = 0.f, uz = 0.f;
+    int code = 0;  // species, shell
+    if (e < hi) {
+      const int i = m.col_idx[e];
+      const double hji = m.h_val[e], sji = m.s_val[e];
+      if (i == j) {
+        hjj = (float)hji;
+        sjj = (float)sji;
+      } else {
+        const int b = orb_atom[i];
+        const float hii = m.h_diag[i], h2 = (float)(hji * hji);
 #pragma unroll
-  for (int k = 0; k < kDesc; ++k) o[k] = f[k];
+        for (int t = 0; t < 8; ++t) {
+          const float c = -3.0f + 6.0f * t / 7.0f, d = (hii - c) / 0.75f;
+          bin[t] += h2 * __expf(-d * d);
+        }
+        sum[0] += h2;
+        sum[1] += (float)(sji * sji);
+        sum[2] += (float)(hji * sji);
+        sum[3] += h2 * hii;
+        sum[4] += fabsf((float)hji);
+        sum[5] += (float)sji * hii;
+        if (b != a && i == atom_first[b]) {  // geometric part: each neighbour atom once
+          const float dx = pos[3 * b] - ax, dy = pos[3 * b + 1] - ay, dz = pos[3 * b + 2] - az;
+          r = sqrtf(dx * dx + dy * dy + dz * dz);
+          if (r > 1e-6f && r < kRc) {
+            atom = true;
+            w = cutoff_fn(r);
+            ux = dx / r;
+            uy = dy / r;
+            uz = dz / r;
+            code = (species[b] ? 1 : 0) | min(3, (int)(r / (kRc / 4))) << 1;
+          }
+        }
+      }
+    }
+    for (unsigned left = __ballot_sync(0xffffffffu, atom); left; left &= left - 1) {
+      const int src = __ffs(left) - 1;
+      const float rr = __shfl_sync(0xffffffffu, r, src), ww = __shfl_sync(0xffffffffu, w, src);
+      const float x = __shfl_sync(0xffffffffu, ux, src), y = __shfl_sync(0xffffffffu, uy, src);
+      const float z = __shfl_sync(0xffffffffu, uz, src);
+      const int cd = __shfl_sync(0xffffffffu, code, src);
+      const float d = (rr - mu) / kRbfW, g = ww * __expf(-d * d);
+      if ((lane >> 4) == (cd & 1)) rad += g;
+      // lanes 0 .. 2: dipole, 3 .. 8: quadrupole xx yy zz xy xz yz
+      const float p = lane == 0 || lane == 3 || lane == 6 || lane == 7 ? x : (lane == 2 || lane == 5 ? z : y);
+      const float q = lane < 3 ? 1.f : (lane == 3 ? x : (lane == 4 || lane == 6 ? y : z));
+      const float v = ww * (p * q - (lane >= 3 && lane < 6 ? 1.0f / 3 : 0.f));
+      const int sh = cd >> 1;
+#pragma unroll
+      for (int s = 0; s < 4; ++s) mom[s] += s == sh ? v : 0.f;
+    }
+  }
+#pragma unroll
+  for (int k = 16; k > 0; k >>= 1) {
+#pragma unroll
+    for (int t = 0; t < 8; ++t) bin[t] += __shfl_xor_sync(0xffffffffu, bin[t], k);
+#pragma unroll
+    for (int t = 0; t < 6; ++t) sum[t] += __shfl_xor_sync(0xffffffffu, sum[t], k);
+    hjj += __shfl_xor_sync(0xffffffffu, hjj, k);  // one lane has the diagonal entry
+    sjj += __shfl_xor_sync(0xffffffffu, sjj, k);
+  }
+  o[lane] = rad;
+#pragma unroll
+  for (int s = 0; s < 4; ++s) {  // squared norms: moments 0 .. 2, and 3 .. 8 (off-diagonal ones twice)
+    const float v = lane < 9 ? mom[s] * mom[s] * (lane >= 6 ? 2.f : 1.f) : 0.f;
+    float dip = lane < 3 ? v : 0.f, quad = lane < 3 ? 0.f : v;
+#pragma unroll
+    for (int k = 8; k > 0; k >>= 1) {
+      dip += __shfl_xor_sync(0xffffffffu, dip, k);
+      quad += __shfl_xor_sync(0xffffffffu, quad, k);
+    }
+    if (lane == 0) {
+      o[32 + 2 * s] = dip;
+      o[33 + 2 * s] = quad;
+    }
+  }
+  if (lane < 6) o[40 + lane] = lane == (species[a] ? 1 : 0) || lane == 2 + min(3, j - atom_first[a]) ? 1.f : 0.f;
+  if (lane == 0) {
+    o[46] = hjj;
+    o[47] = sjj;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) o[48 + t] = bin[t];
+#pragma unroll
+    for (int t = 0; t < 5; ++t) o[56 + t] = sum[t];
+    o[61] = (hi - lo) / 100.0f;
+    o[62] = sum[5];
+    o[63] = 1.f;
+  }
 }
 
 // ------------------------------------------------------------ MLP kernels
@@ -263,9 +300,8 @@ gb_status gb_descriptors(const gb_matrix* m, int32_t n_atoms, const float* pos, 
   if (!m || !pos || !orb_atom || !atom_first || !species || !out || n_atoms < 1)
     return gb::fail(GB_EINVAL, "gb_descriptors: NULL argument or no atoms");
   const gbk::DevMat* dm = gb::devmat_of(m);
-  const int threads = 128;
-  descriptor_kernel<<<(dm->n + threads - 1) / threads, threads, 0, static_cast<cudaStream_t>(stream)>>>(
-      *dm, pos, orb_atom, atom_first, species, out);
+  descriptor_kernel<<<(dm->n + 7) / 8, 256, 0, static_cast<cudaStream_t>(stream)>>>(*dm, pos, orb_atom, atom_first,
+                                                                                    species, out);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return gb::fail(GB_ECUDA, "descriptor kernel: %s", cudaGetErrorString(e));
   return GB_OK;
