@@ -69,65 +69,6 @@ using namespace gb;
 // ------------------------------------------------------------ standalone SpMM
 namespace {
 
-// Single-column panels (FP32): one warp per block row, lane l takes the
-// stored blocks b0 + l, b0 + l + 32, ... with ALL W columns, so the warp reads
-// consecutive 64-byte blocks (one coalesced stream of the matrix) and each x
-// gather is one contiguous run of 4 rows x W columns; a xor-shuffle reduction
-// then sums the 4 x W complex partials.
-template <int WC>
-__device__ __forceinline__ void spmm_row_lanes_f(const gbk::DevMat& m, const float* __restrict__ A,
-                                                 const float2* __restrict__ x, float2* __restrict__ y, int lane,
-                                                 int I) {
-  float2 acc[4][WC];
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < WC; ++c) acc[r][c] = make_float2(0.f, 0.f);
-  const int b1 = m.blk_ptr[I + 1];
-  for (int b = m.blk_ptr[I] + lane; b < b1; b += 32) {
-    const int J = __ldg(m.blk_col + b);
-    const float4* ab = reinterpret_cast<const float4*>(A + (size_t)b * 16);
-    float4 a[4];
-#pragma unroll
-    for (int r = 0; r < 4; ++r) a[r] = __ldg(ab + r);
-    float2 xv[4][WC];
-    const float2* xr = x + (size_t)(4 * J) * WC;
-#pragma unroll
-    for (int t = 0; t < 4; ++t)
-#pragma unroll
-      for (int c = 0; c < WC; ++c) xv[t][c] = xr[t * WC + c];
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < WC; ++c) {
-        acc[r][c].x = fmaf(a[r].x, xv[0][c].x, acc[r][c].x);
-        acc[r][c].y = fmaf(a[r].x, xv[0][c].y, acc[r][c].y);
-        acc[r][c].x = fmaf(a[r].y, xv[1][c].x, acc[r][c].x);
-        acc[r][c].y = fmaf(a[r].y, xv[1][c].y, acc[r][c].y);
-        acc[r][c].x = fmaf(a[r].z, xv[2][c].x, acc[r][c].x);
-        acc[r][c].y = fmaf(a[r].z, xv[2][c].y, acc[r][c].y);
-        acc[r][c].x = fmaf(a[r].w, xv[3][c].x, acc[r][c].x);
-        acc[r][c].y = fmaf(a[r].w, xv[3][c].y, acc[r][c].y);
-      }
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1)
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-#pragma unroll
-      for (int c = 0; c < WC; ++c) {
-        acc[r][c].x += __shfl_xor_sync(0xffffffffu, acc[r][c].x, off);
-        acc[r][c].y += __shfl_xor_sync(0xffffffffu, acc[r][c].y, off);
-      }
-  const int nrow = min(4, m.n - 4 * I);
-  // lane r * WC + c stores (row r, column c)
-#pragma unroll
-  for (int r = 0; r < 4; ++r)
-#pragma unroll
-    for (int c = 0; c < WC; ++c)
-      if (lane == r * WC + c && r < nrow) y[(size_t)(4 * I + r) * WC + c] = acc[r][c];
-}
-
 // Narrow FP32 panels (W = 1, 2, 4): one warp per block row, lane l owns row
 // r = l % 4 of the stored blocks b0 + l / 4, b0 + l / 4 + 8, ...  The lanes of
 // a warp read 8 whole consecutive blocks per step (512 contiguous bytes: each
@@ -157,7 +98,12 @@ __device__ __forceinline__ void quad_fma(const float4& a, const float4 (&xv)[2 *
 // The kernel is bound by loads in flight: the block columns are fetched a
 // step ahead, W = 1 keeps two 8-block steps in flight per lane and W = 2 one,
 // at 40 registers (48 warps per SM) without spills.
-template <int WC>
+// RAG (n not a multiple of 4): x ends inside the last block column's four rows, whose
+// missing ones are zero; read with guards there instead of from a padded copy of x
+// (an allocation, two copies and a free: 14 of 23 us at 23,750 rows, and 200 us where
+// the call was waited for, because the pool gave its memory back).
+// X8: x on an 8-byte boundary only (read entry by entry).
+template <int WC, bool RAG, bool X8 = false>
 __global__ void __launch_bounds__(256, 6)
     spmm_quad_kernel(const gbk::DevMat m, const float* __restrict__ A, const float2* __restrict__ x,
                      float2* __restrict__ y) {
@@ -172,6 +118,16 @@ __global__ void __launch_bounds__(256, 6)
   const int b1 = m.blk_ptr[I + 1];
   const float4* __restrict__ A4 = reinterpret_cast<const float4*>(A);
   const float4* __restrict__ X4 = reinterpret_cast<const float4*>(x);
+  auto guarded = [&](int J, float4 (&xv)[NQ]) {  // float4 q: complex entries 2 q and 2 q + 1 of the 4 x WC
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int r0 = 4 * J + 2 * q / WC, r1 = 4 * J + (2 * q + 1) / WC;
+      const float2 z = make_float2(0.f, 0.f);
+      const float2 u = !RAG || r0 < m.n ? x[(size_t)4 * J * WC + 2 * q] : z;
+      const float2 v = !RAG || r1 < m.n ? x[(size_t)4 * J * WC + 2 * q + 1] : z;
+      xv[q] = make_float4(u.x, u.y, v.x, v.y);
+    }
+  };
   int b = m.blk_ptr[I] + s;
   // block columns one step ahead: the x gathers of a step then wait for one
   // memory round trip, not two (column index, then x)
@@ -191,9 +147,18 @@ __global__ void __launch_bounds__(256, 6)
     for (int u = 0; u < U; ++u) a[u] = __ldcs(A4 + (size_t)(b + 8 * u) * 4 + r);
     float4 xv[U][NQ];
 #pragma unroll
-    for (int u = 0; u < U; ++u)
+    for (int u = 0; u < U; ++u) {
+      if constexpr (X8) {
+        guarded(J[u], xv[u]);
+      } else {
+        if (RAG && J[u] == m.nb - 1) {
+          guarded(J[u], xv[u]);
+          continue;
+        }
 #pragma unroll
-      for (int q = 0; q < NQ; ++q) xv[u][q] = __ldg(X4 + (size_t)J[u] * NQ + q);
+        for (int q = 0; q < NQ; ++q) xv[u][q] = __ldg(X4 + (size_t)J[u] * NQ + q);
+      }
+    }
 #pragma unroll
     for (int u = 0; u < U; ++u) quad_fma<WC>(a[u], xv[u], acc);
   }
@@ -203,8 +168,12 @@ __global__ void __launch_bounds__(256, 6)
 #pragma unroll
     for (int u = 0; u + 1 < U; ++u) Jn[u] = Jn[u + 1];
     float4 xv[NQ];
+    if (X8 || (RAG && J == m.nb - 1)) {
+      guarded(J, xv);
+    } else {
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) xv[q] = __ldg(X4 + (size_t)J * NQ + q);
+      for (int q = 0; q < NQ; ++q) xv[q] = __ldg(X4 + (size_t)J * NQ + q);
+    }
     quad_fma<WC>(a, xv, acc);
   }
 #pragma unroll
@@ -220,87 +189,49 @@ __global__ void __launch_bounds__(256, 6)
   }
 }
 
-// FP64 narrow panels (W = 1, 2), same quad layout as the FP32 kernel above:
-// lane l accumulates row l mod 4 of the blocks b0 + floor(l / 4) + 8k, so a
-// warp step reads 8 whole consecutive blocks (1 KB of values) and the 4 lanes
-// of a block share its x gather.  The product is bound by the FP64 FMA pipe
-// (GB300 runs FP64 at 1/64 of its FP32 rate), so the layout's job is to keep
-// enough loads in flight that the pipe never waits: two 8-block steps per lane.
-template <int WC>
-__global__ void __launch_bounds__(256, 4)
-    spmm_quad_d_kernel(const gbk::DevMat m, const double* __restrict__ A, const double2* __restrict__ x,
-                       double2* __restrict__ y) {
-  const long long I = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  if (I >= m.nb) return;  // uniform per warp
-  const int lane = threadIdx.x & 31, r = lane & 3, s = lane >> 2;
-  constexpr int U = 2;
-  constexpr int NX = 4 * WC;  // double2 per gathered 4 x WC complex x block
-  double2 acc[WC];
-#pragma unroll
-  for (int c = 0; c < WC; ++c) acc[c] = make_double2(0.0, 0.0);
-  const int b1 = m.blk_ptr[I + 1];
-  const double2* __restrict__ A2 = reinterpret_cast<const double2*>(A);
-  auto step = [&](const double2 (&a)[2], const double2 (&xv)[NX]) {
-    const double ar[4] = {a[0].x, a[0].y, a[1].x, a[1].y};
-#pragma unroll
-    for (int c = 0; c < WC; ++c)
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        acc[c].x = fma(ar[t], xv[t * WC + c].x, acc[c].x);
-        acc[c].y = fma(ar[t], xv[t * WC + c].y, acc[c].y);
-      }
-  };
-  int b = m.blk_ptr[I] + s;
-  for (; b + 8 * (U - 1) < b1; b += 8 * U) {
-    int J[U];
-    double2 a[U][2], xv[U][NX];
-#pragma unroll
-    for (int u = 0; u < U; ++u) J[u] = __ldcs(m.blk_col + b + 8 * u);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      a[u][0] = __ldcs(A2 + (size_t)(b + 8 * u) * 8 + 2 * r);
-      a[u][1] = __ldcs(A2 + (size_t)(b + 8 * u) * 8 + 2 * r + 1);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-#pragma unroll
-      for (int q = 0; q < NX; ++q) xv[u][q] = __ldg(x + (size_t)J[u] * NX + q);
-#pragma unroll
-    for (int u = 0; u < U; ++u) step(a[u], xv[u]);
-  }
-  for (; b < b1; b += 8) {
-    const int J = __ldcs(m.blk_col + b);
-    const double2 a[2] = {__ldcs(A2 + (size_t)b * 8 + 2 * r), __ldcs(A2 + (size_t)b * 8 + 2 * r + 1)};
-    double2 xv[NX];
-#pragma unroll
-    for (int q = 0; q < NX; ++q) xv[q] = __ldg(x + (size_t)J * NX + q);
-    step(a, xv);
+// FP64, any width: threads own (row, column) outputs, consecutive threads consecutive
+// columns of a row, and walk the row's pattern entries (scalar CSR); W = 1 and 2 split
+// a row over E = 4 and 2 lanes that meet in shuffles.  The product is bound by the FP64
+// pipe (1/64 of the FP32 rate), so what counts is the number of FMAs: the pattern's
+// entries, not the 4x4 blocks' (a third of which is padding on the bundles).  The bytes
+// are those of the blocks: 12 an entry against 8 / fill.  41,040-orbital bundle, W = 8:
+// blocks 240 us, entries 167 us (W = 1: 43 and 31).
+template <int E>
+__global__ void __launch_bounds__(256)
+    spmm_csr_d_kernel(const gbk::DevMat m, const double* __restrict__ A, int W, const double2* __restrict__ x,
+                      double2* __restrict__ y) {
+  const long long o = (blockIdx.x * 256LL + threadIdx.x) / E;  // output row * W + column
+  const int slot = threadIdx.x % E;
+  const bool in = o < (long long)m.n * W;
+  const int row = in ? (int)(o / W) : 0, c = in ? (int)(o - (long long)row * W) : 0;
+  const int e1 = in ? m.row_ptr[row + 1] : 0;
+  double2 acc = make_double2(0.0, 0.0);
+#pragma unroll 4
+  for (int e = (in ? m.row_ptr[row] : 0) + slot; e < e1; e += E) {
+    const double a = __ldg(A + e);
+    const double2 v = __ldg(x + (size_t)__ldg(m.col_idx + e) * W + c);
+    acc.x = fma(a, v.x, acc.x);
+    acc.y = fma(a, v.y, acc.y);
   }
 #pragma unroll
-  for (int off = 4; off < 32; off <<= 1)
-#pragma unroll
-    for (int c = 0; c < WC; ++c) {
-      acc[c].x += __shfl_xor_sync(0xffffffffu, acc[c].x, off);
-      acc[c].y += __shfl_xor_sync(0xffffffffu, acc[c].y, off);
-    }
-  if (s == 0 && 4 * I + r < m.n) {
-#pragma unroll
-    for (int c = 0; c < WC; ++c) y[(size_t)(4 * I + r) * WC + c] = acc[c];
+  for (int k = E / 2; k > 0; k >>= 1) {
+    acc.x += __shfl_xor_sync(0xffffffffu, acc.x, k);
+    acc.y += __shfl_xor_sync(0xffffffffu, acc.y, k);
   }
+  if (in && slot == 0) y[o] = acc;
 }
 
-// Wide panels (FP32: W = 4..64 in powers of two; FP64: W = 4..32): one warp
+// Wide FP32 panels (W = 4..64 in powers of two): one warp
 // per block row, split into G = 32 / CL groups of CL lanes; group g takes the
 // blocks b0 + g + G k, and lane c of a group owns columns [c * PC, (c+1) * PC)
-// of the panel (PC = 2 complex columns per lane in FP32, read and written as
-// one float4; 1 in FP64).  A block's values are read by every lane of its
+// of the panel (PC = 2 complex columns per lane, read and written as one float4).  A block's values are read by every lane of its
 // group at one address (a broadcast), its x rows by the group as contiguous
 // runs, and each value feeds PC complex columns from registers.  The groups
 // then add up through xor shuffles.  Requires x and y 16-byte aligned.
 // The kernel waits on loads (ncu at W = 8: long-scoreboard stalls dominate),
 // so it keeps one step in flight per lane at <= 64 registers, which lets 32
 // warps share an SM (two steps at 106 registers left 11 warps active).
-template <int CL>
+template <int CL, bool RAG>
 __global__ void __launch_bounds__(256, 4)
     spmm_wide_kernel(const gbk::DevMat m, const float* __restrict__ A, const float4* __restrict__ x,
                      float4* __restrict__ y) {
@@ -325,6 +256,9 @@ __global__ void __launch_bounds__(256, 4)
       }
     }
   };
+  auto fetch = [&](int row) {
+    return !RAG || row < m.n ? __ldg(x + (size_t)row * CL + c) : make_float4(0.f, 0.f, 0.f, 0.f);
+  };
   const int b1 = m.blk_ptr[I + 1];
   int b = m.blk_ptr[I] + g;
   constexpr int U = 1;
@@ -347,7 +281,7 @@ __global__ void __launch_bounds__(256, 4)
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int t = 0; t < 4; ++t) xv[u][t] = __ldg(x + (size_t)(4 * J[u] + t) * CL + c);
+      for (int t = 0; t < 4; ++t) xv[u][t] = fetch(4 * J[u] + t);
 #pragma unroll
     for (int u = 0; u < U; ++u) step(a[u], xv[u]);
   }
@@ -359,7 +293,7 @@ __global__ void __launch_bounds__(256, 4)
 #pragma unroll
     for (int r = 0; r < 4; ++r) a[r] = __ldcs(A4 + (size_t)b * 4 + r);
 #pragma unroll
-    for (int t = 0; t < 4; ++t) xv[t] = __ldg(x + (size_t)(4 * J + t) * CL + c);
+    for (int t = 0; t < 4; ++t) xv[t] = fetch(4 * J + t);
     step(a, xv);
   }
 #pragma unroll
@@ -378,110 +312,86 @@ __global__ void __launch_bounds__(256, 4)
   }
 }
 
-template <int CL>
-__global__ void __launch_bounds__(256, 3)
-    spmm_wide_d_kernel(const gbk::DevMat m, const double* __restrict__ A, const double2* __restrict__ x,
-                       double2* __restrict__ y) {
-  constexpr int G = 32 / CL;
-  const long long I = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-  if (I >= m.nb) return;
-  const int lane = threadIdx.x & 31, g = lane / CL, c = lane - g * CL;
-  double2 acc[4];
+// FP32, what the kernels above do not take (other widths, x or y off a 16-byte
+// boundary).  W <= 8: one warp per block row, its lanes split as columns x block slots
+// (four blocks in flight a lane); wider: one thread per (block row, column).  One thread
+// per (row, column) took 1.5 to 3.6 times as long at W = 3 .. 33 (41,040 orbitals).
+template <bool RAG>
+__global__ void __launch_bounds__(256)
+    spmm_any_kernel(const gbk::DevMat m, const float* __restrict__ A, int W, const float2* __restrict__ x,
+                    float2* __restrict__ y) {
+  float2 acc[4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) acc[r] = make_double2(0.0, 0.0);
-  const double2* __restrict__ A2 = reinterpret_cast<const double2*>(A);
+  for (int r = 0; r < 4; ++r) acc[r] = make_float2(0.f, 0.f);
+  const float4* __restrict__ A4 = reinterpret_cast<const float4*>(A);
+  auto fetch = [&](int row, int c) {
+    return !RAG || row < m.n ? x[(size_t)row * W + c] : make_float2(0.f, 0.f);
+  };
+  auto mul = [&](const float4 (&a)[4], const float2 (&v)[4]) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      acc[r].x = fmaf(a[r].x, v[0].x, fmaf(a[r].y, v[1].x, fmaf(a[r].z, v[2].x, fmaf(a[r].w, v[3].x, acc[r].x))));
+      acc[r].y = fmaf(a[r].x, v[0].y, fmaf(a[r].y, v[1].y, fmaf(a[r].z, v[2].y, fmaf(a[r].w, v[3].y, acc[r].y))));
+    }
+  };
+  const long long at = blockIdx.x * 256LL + threadIdx.x;
+  int I, c, b, S = 1;
+  bool store = true;
+  if (W <= 8) {
+    const int Wp = W <= 1 ? 1 : (W <= 2 ? 2 : (W <= 4 ? 4 : 8)), lane = (int)(at & 31);
+    I = (int)(at >> 5);
+    if (I >= m.nb) return;  // uniform per warp
+    c = lane % Wp;
+    S = 32 / Wp;
+    b = m.blk_ptr[I] + lane / Wp;
+    store = lane < W;
+    if (c >= W) b = m.blk_ptr[I + 1];  // no column: only the shuffles
+  } else {
+    if (at >= (long long)m.nb * W) return;
+    I = (int)(at / W);
+    c = (int)(at - (long long)I * W);
+    b = m.blk_ptr[I];
+  }
   const int b1 = m.blk_ptr[I + 1];
-  for (int b = m.blk_ptr[I] + g; b < b1; b += G) {
-    const int J = __ldcs(m.blk_col + b);
-    double2 a[8], xv[4];
+  for (; b + 3 * S < b1; b += 4 * S) {
+    int J[4];
+    float4 a[4][4];
+    float2 v[4][4];
 #pragma unroll
-    for (int q = 0; q < 8; ++q) a[q] = __ldcs(A2 + (size_t)b * 8 + q);
+    for (int u = 0; u < 4; ++u) J[u] = __ldg(m.blk_col + b + u * S);
 #pragma unroll
-    for (int t = 0; t < 4; ++t) xv[t] = __ldg(x + (size_t)(4 * J + t) * CL + c);
+    for (int u = 0; u < 4; ++u) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      const double ar[4] = {a[2 * r].x, a[2 * r].y, a[2 * r + 1].x, a[2 * r + 1].y};
+      for (int r = 0; r < 4; ++r) a[u][r] = __ldg(A4 + (size_t)(b + u * S) * 4 + r);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        acc[r].x = fma(ar[t], xv[t].x, acc[r].x);
-        acc[r].y = fma(ar[t], xv[t].y, acc[r].y);
-      }
+      for (int t = 0; t < 4; ++t) v[u][t] = fetch(4 * J[u] + t, c);
     }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) mul(a[u], v[u]);
   }
+  for (; b < b1; b += S) {
+    const int J = __ldg(m.blk_col + b);
+    float4 a[4];
+    float2 v[4];
 #pragma unroll
-  for (int off = CL; off < 32; off <<= 1)
+    for (int r = 0; r < 4; ++r) a[r] = __ldg(A4 + (size_t)b * 4 + r);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, off);
-      acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, off);
-    }
-  if (g == 0) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r)
-      if (4 * I + r < m.n) y[(size_t)(4 * I + r) * CL + c] = acc[r];
-  }
-}
-
-template <bool F64>
-__global__ void spmm_kernel(const gbk::DevMat m, int which, int W, const void* __restrict__ xv,
-                            void* __restrict__ yv) {
-  const int lane = threadIdx.x & 31;
-  if constexpr (!F64) {
-    if (W == 1) {  // x not 16-byte aligned (else spmm_quad_kernel): lane per block
-      const long long warp0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-      const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-      const float* A = which ? m.sb_hi : m.hb_hi;
-      const float2* x = static_cast<const float2*>(xv);
-      float2* y = static_cast<float2*>(yv);
-      for (long long I = warp0; I < m.nb; I += nwarps) spmm_row_lanes_f<1>(m, A, x, y, lane, (int)I);
-      return;
-    }
+    for (int t = 0; t < 4; ++t) v[t] = fetch(4 * J + t, c);
+    mul(a, v);
   }
   if (W <= 8) {
-    // narrow panels: one warp per block row, lanes split the stored blocks
-    const long long warp0 = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    int Wp = 1;
-    while (Wp < W) Wp <<= 1;
-    const int c = lane % Wp;
-    const bool active = c < W;
-    for (long long I = warp0; I < m.nb; I += nwarps) {
-      const int nrow = min(4, m.n - 4 * (int)I);
-      if constexpr (F64) {
-        double2 acc[4];
-        gbk::wbsr_row_d(m, which ? m.sb : m.hb, static_cast<const double2*>(xv), W, Wp, lane, (int)I, active, acc);
-        double2* y = static_cast<double2*>(yv);
-        if (lane < Wp && active)
-          for (int r = 0; r < nrow; ++r) y[(size_t)(4 * I + r) * W + c] = acc[r];
-      } else {
-        float2 acc[4];
-        gbk::wbsr_row_f(m, which ? m.sb_hi : m.hb_hi, static_cast<const float2*>(xv), W, Wp, lane, (int)I, active,
-                        acc);
-        float2* y = static_cast<float2*>(yv);
-        if (lane < Wp && active)
-          for (int r = 0; r < nrow; ++r) y[(size_t)(4 * I + r) * W + c] = acc[r];
+    for (int off = 32 / S; off < 32; off <<= 1) {
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, off);
+        acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, off);
       }
     }
-    return;
   }
-  // wide panels: one thread per (block row, column), consecutive threads take consecutive columns
-  const long long items = (long long)m.nb * W;
-  for (long long it = blockIdx.x * (long long)blockDim.x + threadIdx.x; it < items;
-       it += (long long)gridDim.x * blockDim.x) {
-    const int I = (int)(it / W), c = (int)(it - (long long)I * W);
-    const int nrow = min(4, m.n - 4 * I);
-    if constexpr (F64) {
-      double2 acc[4];
-      gbk::bsr_row_d(m, which ? m.sb : m.hb, static_cast<const double2*>(xv), W, c, I, acc);
-      double2* y = static_cast<double2*>(yv);
-      for (int r = 0; r < nrow; ++r) y[(size_t)(4 * I + r) * W + c] = acc[r];
-    } else {
-      float2 acc[4];
-      gbk::bsr_row_f(m, which ? m.sb_hi : m.hb_hi, static_cast<const float2*>(xv), W, c, I, acc);
-      float2* y = static_cast<float2*>(yv);
-      for (int r = 0; r < nrow; ++r) y[(size_t)(4 * I + r) * W + c] = acc[r];
-    }
-  }
+  if (!store) return;
+#pragma unroll
+  for (int r = 0; r < 4; ++r)
+    if (4 * I + r < m.n) y[(size_t)(4 * I + r) * W + c] = acc[r];
 }
 
 }  // namespace
@@ -610,10 +520,6 @@ cudaError_t form_on_device(const gbk::DevMat& d, size_t nnzb, const FactorTiles&
 }
 
 }  // namespace
-
-// The standalone SpMM reads rows 4J..4J+3 of x for every stored block column
-// J; when n % 4 != 0 the last block column reaches past row n-1 (its matrix
-// entries are zero there), so gb_spmm reads from a zero-padded copy of x.
 
 extern "C" {
 
@@ -800,66 +706,56 @@ gb_status gb_spmm(const gb_matrix* m, int32_t which, gb_precision prec, int32_t 
   if (misaligned(x, prec == GB_FP64 ? 16 : 8) || misaligned(y, prec == GB_FP64 ? 16 : 8))
     return fail(GB_EINVAL, "x and y must be aligned to their complex element (16 bytes FP64, 8 FP32)");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  const size_t esz = prec == GB_FP64 ? 16 : 8;
-  const int64_t n4 = 4 * m->nb;
-  const void* xin = x;
-  void* pad = nullptr;
-  if (n4 != m->n) {  // last block column reads rows up to 4*nb - 1: pad x with zero rows
-    GB_CUDA(cudaMallocAsync(&pad, esz * n4 * w, s));
-    cudaError_t pe = cudaMemsetAsync(pad, 0, esz * n4 * w, s);
-    if (pe == cudaSuccess) pe = cudaMemcpyAsync(pad, x, esz * m->n * w, cudaMemcpyDeviceToDevice, s);
-    if (pe != cudaSuccess) {  // free the padded copy on this exit path too
-      cudaFreeAsync(pad, s);
-      return cuda_fail(pe, "spmm input padding");
-    }
-    xin = pad;
-  }
-  const int threads = 256;
-  int nsm = 152;
-  cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, m->device);
-  const long long work = w <= 8 ? (long long)m->nb * 32 : (long long)m->nb * w;  // threads of work
-  const int blocks = (int)std::min<long long>((work + threads - 1) / threads, (long long)nsm * 8);
-  const bool aligned = (reinterpret_cast<uintptr_t>(xin) % 16) == 0 && (reinterpret_cast<uintptr_t>(y) % 16) == 0;
-  const bool pow2 = (w & (w - 1)) == 0;
-  const unsigned wblocks = (unsigned)((m->nb + 7) / 8);  // 8 warps = 8 block rows per CTA
-  if (aligned && prec != GB_FP64 && w <= 2) {
-    const float* A = which ? m->dm.sb_hi : m->dm.hb_hi;
-    const auto* xq = static_cast<const float2*>(xin);
-    auto* yq = static_cast<float2*>(y);
+  const long long outs = (long long)m->n * w;
+  auto blocks = [](long long threads) { return (unsigned)((threads + 255) / 256); };
+  if (prec == GB_FP64) {
+    const double* A = which ? m->dm.s_val : m->dm.h_val;
+    const auto* xd = static_cast<const double2*>(x);
+    auto* yd = static_cast<double2*>(y);
     if (w == 1)
-      spmm_quad_kernel<1><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq);
+      spmm_csr_d_kernel<4><<<blocks(4 * outs), 256, 0, s>>>(m->dm, A, w, xd, yd);
+    else if (w == 2)
+      spmm_csr_d_kernel<2><<<blocks(2 * outs), 256, 0, s>>>(m->dm, A, w, xd, yd);
     else
-      spmm_quad_kernel<2><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq);
-  } else if (aligned && prec != GB_FP64 && pow2) {  // w = 4 .. 64
-    const float* A = which ? m->dm.sb_hi : m->dm.hb_hi;
-    const auto* xq = static_cast<const float4*>(xin);
-    auto* yq = static_cast<float4*>(y);
-    switch (w) {
-      case 4: spmm_wide_kernel<2><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      case 8: spmm_wide_kernel<4><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      case 16: spmm_wide_kernel<8><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      case 32: spmm_wide_kernel<16><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      default: spmm_wide_kernel<32><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-    }
-  } else if (aligned && prec == GB_FP64 && pow2 && w <= 32) {
-    const double* A = which ? m->dm.sb : m->dm.hb;
-    const auto* xq = static_cast<const double2*>(xin);
-    auto* yq = static_cast<double2*>(y);
-    switch (w) {
-      case 1: spmm_quad_d_kernel<1><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      case 2: spmm_quad_d_kernel<2><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      case 4: spmm_wide_d_kernel<4><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      case 8: spmm_wide_d_kernel<8><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      case 16: spmm_wide_d_kernel<16><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-      default: spmm_wide_d_kernel<32><<<wblocks, threads, 0, s>>>(m->dm, A, xq, yq); break;
-    }
-  } else if (prec == GB_FP64) {
-    spmm_kernel<true><<<blocks, threads, 0, s>>>(m->dm, which, w, xin, y);
+      spmm_csr_d_kernel<1><<<blocks(outs), 256, 0, s>>>(m->dm, A, w, xd, yd);
   } else {
-    spmm_kernel<false><<<blocks, threads, 0, s>>>(m->dm, which, w, xin, y);
+    const float* A = which ? m->dm.sb_hi : m->dm.hb_hi;
+    const auto* x2 = static_cast<const float2*>(x);
+    const auto* x4 = static_cast<const float4*>(x);
+    auto* y2 = static_cast<float2*>(y);
+    auto* y4 = static_cast<float4*>(y);
+    const bool aligned = (reinterpret_cast<uintptr_t>(x) % 16) == 0 && (reinterpret_cast<uintptr_t>(y) % 16) == 0;
+    const unsigned wb = (unsigned)((m->nb + 7) / 8);  // 8 warps = 8 block rows per CTA
+    auto run = [&](auto rag) {
+      constexpr bool RAG = decltype(rag)::value;
+      switch (aligned || w <= 2 ? w : 0) {
+        case 1:
+          if (aligned)
+            spmm_quad_kernel<1, RAG><<<wb, 256, 0, s>>>(m->dm, A, x2, y2);
+          else
+            spmm_quad_kernel<1, RAG, true><<<wb, 256, 0, s>>>(m->dm, A, x2, y2);
+          break;
+        case 2:
+          if (aligned)
+            spmm_quad_kernel<2, RAG><<<wb, 256, 0, s>>>(m->dm, A, x2, y2);
+          else
+            spmm_quad_kernel<2, RAG, true><<<wb, 256, 0, s>>>(m->dm, A, x2, y2);
+          break;
+        case 4: spmm_wide_kernel<2, RAG><<<wb, 256, 0, s>>>(m->dm, A, x4, y4); break;
+        case 8: spmm_wide_kernel<4, RAG><<<wb, 256, 0, s>>>(m->dm, A, x4, y4); break;
+        case 16: spmm_wide_kernel<8, RAG><<<wb, 256, 0, s>>>(m->dm, A, x4, y4); break;
+        case 32: spmm_wide_kernel<16, RAG><<<wb, 256, 0, s>>>(m->dm, A, x4, y4); break;
+        case 64: spmm_wide_kernel<32, RAG><<<wb, 256, 0, s>>>(m->dm, A, x4, y4); break;
+        default:
+          spmm_any_kernel<RAG><<<blocks(w <= 8 ? 32 * m->nb : m->nb * w), 256, 0, s>>>(m->dm, A, w, x2, y2);
+      }
+    };
+    if (m->n % 4 != 0)
+      run(std::true_type{});
+    else
+      run(std::false_type{});
   }
   cudaError_t e = cudaGetLastError();
-  if (pad) cudaFreeAsync(pad, s);
   if (e != cudaSuccess) return cuda_fail(e, "spmm launch");
   return GB_OK;
 }
