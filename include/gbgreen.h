@@ -19,7 +19,8 @@
  * shift or ask for panels of one or two columns build the same space by a
  * conjugate orthogonal CG (COCG) in the S-bilinear form with that seed.
  * S^{-1} is applied exactly by a block-bidiagonal Cholesky factor of S where
- * S's half-bandwidth is at most 63 (chains), else by an inner
+ * S's half-bandwidth is at most 63 (chains); else, in the mixed path, by the
+ * dense inverse of an S of at most 1024 orbitals; else by an inner
  * block-Jacobi-preconditioned iteration (CG, or Chebyshev in the mixed path).
  * The paper defers the method's details to its references; the recurrences
  * used are the standard ones.
@@ -199,9 +200,12 @@ typedef struct {
                             block-bidiagonal Cholesky solve where S's
                             half-bandwidth is <= 63 (FP64: one solve; mixed: two
                             FP32 solves around a float-float residual), else
+                            (mixed, the real recurrence) the dense inverse of
+                            an S of at most 1024 orbitals, refined as well, else
                             an iteration (FP64: CG; mixed: Chebyshev).
                             bit 1: keep the inner-iteration vectors of a panel
-                            in shared memory when they fit (iterations only);
+                            in shared memory when they fit (iterations only;
+                            no dense inverse);
                             bit 2: iterate with CG instead of the factor solve
                             (and instead of Chebyshev in the mixed path);
                             bit 4: mixed path iterates with Chebyshev instead
@@ -237,7 +241,7 @@ typedef struct {
   int32_t* inner_iters; /* [nrhs] inner steps of the column's panel summed over
                            the whole solve and all refinement levels: CG
                            iterations, Chebyshev steps, or one per level for
-                           the exact factor solve                            */
+                           the exact factor solve and the dense inverse      */
   int32_t* col_status;  /* [nrhs] bit flags per column: 1 COCG breakdown, 2 S not
                            SPD, 4 a shift missed tol, 8 inner CG hit its cap,
                            16 a bounded wait for a factor tile gave up,
@@ -255,7 +259,7 @@ size_t gb_solve_workspace_size(const gb_matrix* m, const gb_solve_params* p);
  * plan[0] = RHS columns per panel, plan[1] = teams (CTAs) launched,
  * plan[2] = 1 if the inner-iteration vectors live in shared memory,
  * plan[3] = dynamic shared-memory bytes per team, plan[4] = inner solve
- * (0 CG, 1 Chebyshev, 2 exact factor), plan[5] = teams resident per SM.
+ * (0 CG, 1 Chebyshev, 2 exact factor, 3 dense inverse), plan[5] = teams resident per SM.
  * `plan` is a caller-owned host int32[6].
  */
 gb_status gb_solve_plan(const gb_matrix* m, const gb_solve_params* p, int32_t* plan);

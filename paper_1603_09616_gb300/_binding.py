@@ -356,7 +356,7 @@ def solve_plan(mat: Matrix, z, cols, tol=1e-10, maxit=1000, prec="fp64", panel=0
     plan = np.zeros(6, np.int32)
     _check(load().gb_solve_plan(mat.handle, C.byref(p), _ptr(plan)))
     return dict(panel=int(plan[0]), teams=int(plan[1]), cg_smem=bool(plan[2]), dyn_smem=int(plan[3]),
-                inner=("cg", "chebyshev", "factor")[int(plan[4])], teams_per_sm=int(plan[5]))
+                inner=("cg", "chebyshev", "factor", "inverse")[int(plan[4])], teams_per_sm=int(plan[5]))
 
 
 def shifted_solve(mat: Matrix, z, cols, tol=1e-10, maxit=1000, prec="fp64", w_rho=None, w_edm=None,

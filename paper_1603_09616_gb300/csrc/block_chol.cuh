@@ -380,4 +380,5 @@ __device__ __forceinline__ void bc_solve64(const Args& a, Smem& sm, const double
 }  // namespace gbk
 
 #include "factor_passes.cuh"
+#include "dense_inverse.cuh"
 #include "seed_passes.cuh"

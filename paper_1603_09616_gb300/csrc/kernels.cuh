@@ -73,6 +73,10 @@ struct DevMat {
   const uint4* fx;
   int fx_ne, fx_lg;
   float fx_kd[2], fx_ke[2];
+  // S^-1 as FP16 fragments (dense_inverse.cuh), di_nt x di_nt tiles of 16 x 16 that
+  // 2^di_ex scales back; null: not formed
+  const uint4* di;
+  int di_nt, di_ex;
 };
 constexpr int kMmaTileFloatsDev = 52 * 128;  // a TF32 tile: 20 triangular and up to 32 band fragments
 

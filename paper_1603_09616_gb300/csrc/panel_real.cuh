@@ -154,7 +154,7 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
       gbff::acc_init(d0);
       gbff::acc_init(d1);
       const int e0 = sm.act[c] ? tid : (int)NE;
-      const bool factor = a.inner_bchol != 0;
+      const bool factor = a.inner_bchol || a.inner_dense;
       if (factor)
         inner_real_factor(a, sm, f, cg_x, cg_g, cg_d, cg_q, U);
       else

@@ -519,6 +519,64 @@ cudaError_t form_on_device(const gbk::DevMat& d, size_t nnzb, const FactorTiles&
   return cudaGetLastError();
 }
 
+// The dense inverse of S (dense_inverse.cuh) is kept for matrices without a banded
+// factor of up to kDenseMax orbitals.  Solves gain beyond that too (1710 orbitals: 1944
+// -> 860 ms), but every matrix pays for forming it, 4 n^2 bytes and O(n^3) FP64 work, used
+// or not: at 1024 orbitals that is 4 MB and a few milliseconds, near what the rest of
+// building the matrix takes.
+constexpr int kDenseMax = 1024;
+bool dense_wanted(int64_t n, bool factor) { return !factor && n <= kDenseMax; }
+
+// Forms d.di; leaves it null where S is not SPD or the scratch cannot be had (the
+// solves then iterate, and report such an S as before).
+cudaError_t form_dense_inverse(gbk::DevMat& d, uint4* frags, cudaStream_t s) {
+  const int np = (d.n + gbk::kDiB - 1) / gbk::kDiB * gbk::kDiB, nblk = np / gbk::kDiB, nt = (4 * d.nb + 15) / 16;
+  const size_t one = sizeof(double) * (size_t)np * np, piv = sizeof(double) * gbk::kDiB * np;
+  char* tmp = nullptr;
+  if (cudaMalloc(&tmp, 2 * one + piv + 16) != cudaSuccess) {
+    cudaGetLastError();
+    return cudaSuccess;
+  }
+  double *A = reinterpret_cast<double*>(tmp), *B = reinterpret_cast<double*>(tmp + one);
+  double* R = reinterpret_cast<double*>(tmp + 2 * one);
+  auto* top = reinterpret_cast<unsigned long long*>(tmp + 2 * one + piv);
+  int* bad = reinterpret_cast<int*>(top + 1);
+  struct {
+    unsigned long long top;
+    int bad, pad;
+  } h{};
+  cudaError_t e = cudaMemsetAsync(top, 0, 16, s);
+  if (e == cudaSuccess) {
+    gbk::di_fill_kernel<<<np / 8, 256, 0, s>>>(d, A, np);
+    for (int k = 0; k < nblk; ++k) {
+      gbk::di_pivot_kernel<<<nblk, 256, 0, s>>>(A, np, k, R, bad);
+      gbk::di_step_kernel<<<dim3(nblk, nblk), 256, 0, s>>>(A, B, np, k, R);
+      std::swap(A, B);
+    }
+    gbk::di_max_kernel<<<152, 256, 0, s>>>(A, np, d.n, top);
+    e = cudaGetLastError();
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(&h, top, 16, cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  double mx;
+  std::memcpy(&mx, &h.top, sizeof mx);
+  if (e == cudaSuccess && !h.bad && std::isfinite(mx) && mx > 0.0) {
+    int ex;
+    std::frexp(mx, &ex);
+    if (ex > -40 && ex < 40) {  // largest entry in [2^14, 2^15)
+      gbk::di_frag_kernel<<<dim3(nt, nt), 128, 0, s>>>(A, np, d.n, nt, std::ldexp(1.0, 15 - ex),
+                                                        reinterpret_cast<uint32_t*>(frags));
+      e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      d.di = frags;
+      d.di_nt = nt;
+      d.di_ex = ex - 15;
+    }
+  }
+  cudaFree(tmp);
+  return e;
+}
+
 }  // namespace
 
 extern "C" {
@@ -595,6 +653,9 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   const size_t o_m32 = take(sizeof(float) * nbl * 16), o_hd = take(sizeof(float) * n);
   const size_t o_bfm = take(sizeof(float) * 2 * nblk * gbk::kMmaTileFloatsDev);
   const size_t o_fx = take(sizeof(uint4) * 2 * nblk * gbk::fx_block_words(ft.ne));
+  const bool dense = dense_wanted(n, nbf != 0);
+  const size_t dnt = dense ? (4 * nbl + 15) / 16 : 0;
+  const size_t o_di = take(sizeof(uint4) * 64 * dnt * dnt);
   const size_t total = off;
 
   std::unique_ptr<char[]> host(new char[up]);
@@ -660,6 +721,8 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   d.bfm = nbf ? reinterpret_cast<const float*>(b + o_bfm) : nullptr;
   e = cudaMemcpyAsync(m->base, host.get(), up, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = form_on_device(d, nnzb, ft, s);
+  d.di = nullptr;
+  if (e == cudaSuccess && dense) e = form_dense_inverse(d, reinterpret_cast<uint4*>(b + o_di), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     cudaFree(m->base);
@@ -774,24 +837,34 @@ namespace {
 // (sqrt(kappa) + 1)), with the Lanczos bounds widened by 2% on each side.
 constexpr int kFlagSmem = 2, kFlagCG = 4, kFlagCheb = 16, kFlagHpF32 = 32, kFlagStall = 64;
 constexpr int kStallWindow = 3000;  // iterations without halving the best residual
-void set_inner_method(const gb_matrix* m, const gb_solve_params* p, double itol, gbk::Args& a) {
+// Without a factor the mixed path's real recurrence takes the dense inverse where
+// the matrix keeps one, unless flags ask for an iteration or its shared-memory vectors.
+bool dense_inner(const gb_matrix* m, const gb_solve_params* p, bool real) {
+  return m->dm.di && real && p->prec == GB_MIXED && !(p->flags & (kFlagCG | kFlagCheb | kFlagSmem));
+}
+// Refinement levels of the FP32 solves: two for tol >= 1e-6, three down to 1e-9, four
+// below (at tol 1e-10 a near-threshold pair of a 114-orbital chain stagnated at 7.7e-10
+// with three levels and converged with four).  An explicit bound on the application's
+// error asks for (2e-6)^levels <= bound, two at least (2e-6: the measured accuracy of
+// one FP32 factor solve).
+int refinement_levels(double tol, double bound) {
+  if (!(bound > 0)) return tol >= 1e-6 ? 2 : (tol >= 1e-9 ? 3 : 4);
+  int l = 2;
+  while (l < 4 && std::pow(2e-6, l) > bound) ++l;
+  return l;
+}
+void set_inner_method(const gb_matrix* m, const gb_solve_params* p, double itol, bool real, gbk::Args& a) {
   std::memset(&a, 0, sizeof a);
   a.hp_fp32 = (p->prec == GB_MIXED && (p->flags & kFlagHpF32)) ? 1 : 0;
   a.stall = (p->flags & kFlagStall) ? kStallWindow : 0;
   if (!(p->flags & (kFlagCG | kFlagCheb)) && m->dm.bf_bw > 0) {
     a.inner_bchol = 1;  // exact: block-bidiagonal Cholesky factor solves
-    // mixed: FP32 factor solves on TF32 tensor cores with a three-term split,
-    // each accurate to ~2e-6 (measured), refined around float-float
-    // residuals: two levels for tol >= 1e-6, three down to 1e-9, four below
-    // (measured: at tol 1e-10 a near-threshold pair of a 114-orbital chain
-    // stagnated at 7.7e-10 with three levels and converged with four); an
-    // explicit inner_tol asks for (2e-6)^levels <= inner_tol, two at least
-    if (p->inner_tol > 0) {
-      a.bc_levels = 2;
-      while (a.bc_levels < 4 && std::pow(2e-6, a.bc_levels) > p->inner_tol) ++a.bc_levels;
-    } else {
-      a.bc_levels = p->tol >= 1e-6 ? 2 : (p->tol >= 1e-9 ? 3 : 4);
-    }
+    a.bc_levels = refinement_levels(p->tol, p->inner_tol);
+    return;
+  }
+  if (dense_inner(m, p, real)) {
+    a.inner_dense = 1;  // an iteration's inner_tol holds per level, of which there are two
+    a.bc_levels = refinement_levels(p->tol, p->inner_tol * p->inner_tol);
     return;
   }
   const double lmin = m->dm.s_lam_min * 0.98, lmax = m->dm.s_lam_max * 1.02;
@@ -993,7 +1066,7 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
   else
     pl->itol = p->inner_tol > 0 ? p->inner_tol : 1e-7;
 
-  set_inner_method(m, p, pl->itol, pl->a);
+  set_inner_method(m, p, pl->itol, real, pl->a);
   pl->a.bc_bw_alloc = m->dm.bf_bw;
   const size_t K = p->nshift, N4 = 4 * (size_t)m->nb;
   pl->team_bytes = layout_team(N4, W, (int)K, pl->KG, p->maxit, pl->Mcap, want_g, real, pl->a);
@@ -1031,7 +1104,7 @@ gb_status gb_solve_plan(const gb_matrix* m, const gb_solve_params* p, int32_t* p
   plan[1] = pl.teams;
   plan[2] = pl.cg_smem;
   plan[3] = (int32_t)pl.dyn_smem;
-  plan[4] = pl.a.inner_bchol ? 2 : (pl.a.inner_cheb ? 1 : 0);
+  plan[4] = pl.a.inner_dense ? 3 : (pl.a.inner_bchol ? 2 : (pl.a.inner_cheb ? 1 : 0));
   plan[5] = pl.teams_per_sm;
   return GB_OK;
 }
@@ -2307,8 +2380,9 @@ gb_status gb_shifted_solve_batched(int32_t nsys, const gb_matrix* const* mats, c
     gbk::Args a = bp.proto;  // workspace regions laid out for the maxima
     {
       gbk::Args im;
-      set_inner_method(m, p, p->inner_tol > 0 ? p->inner_tol : (p->prec == GB_FP64 ? 1e-14 : 1e-7), im);
+      set_inner_method(m, p, p->inner_tol > 0 ? p->inner_tol : (p->prec == GB_FP64 ? 1e-14 : 1e-7), bp.real, im);
       a.inner_cheb = im.inner_cheb;
+      a.inner_dense = im.inner_dense;
       a.inner_bchol = im.inner_bchol;
       a.bc_levels = im.bc_levels;
       a.hp_fp32 = im.hp_fp32;

@@ -61,6 +61,7 @@ struct Args {
   // FP32 level with d_{k+1} = A_k d_k + B_k M^-1 r_{k+1}, d_0 = c0 M^-1 r_0.
   int inner_cheb, cheb_K;
   int inner_bchol;  // 1: S x = f by the block-bidiagonal Cholesky factor (exact; block_chol.cuh)
+  int inner_dense;  // 1: mixed path, real recurrence: S x = f by the dense inverse (dense_inverse.cuh)
   int bc_levels;    // mixed path: FP32 factor solves per application (refinement levels)
   int bc_bw_alloc;  // half-bandwidth the dynamic shared memory of the FP32 factor passes is sized for
   // Verification mode: team b solves panel b only and records r_m on every row
@@ -750,18 +751,24 @@ __device__ __noinline__ void real_residual(const Args& a, Smem& sm, const float4
 __device__ __noinline__ void inner_real_factor(const Args& a, Smem& sm, const float4* U, float2* x, float2* g,
                                                float2* d, float2* q, float4* er) {
   const size_t NE = (size_t)4 * a.m.nb * a.W;
-  fx_solve(a, sm, U, x, d, q);
+  auto solve = [&](auto* f, float2* out) {
+    if (a.inner_dense)
+      di_solve(a, sm, f, out, q);
+    else
+      fx_solve(a, sm, f, out, d, q);
+  };
+  solve(U, x);
   if (a.bc_levels > 1) {
     real_residual<1>(a, sm, U, x, er, g);
-    fx_solve(a, sm, er, x + NE, d, q);
+    solve(er, x + NE);
   }
   if (a.bc_levels > 2) {
     real_residual<2>(a, sm, U, x + NE, er, g);
-    fx_solve(a, sm, g, g + NE, d, q);
+    solve(g, g + NE);
   }
   if (a.bc_levels > 3) {
     real_residual<3>(a, sm, U, g + NE, er, g);
-    fx_solve(a, sm, g, d + NE, d, q);
+    solve(g, d + NE);
   }
 }
 
