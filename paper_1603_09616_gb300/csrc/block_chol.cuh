@@ -112,7 +112,10 @@ __host__ __device__ inline DynLayout dyn_layout(bool fp64, int W, bool bchol, un
   L.G = TPB / (64 / RPT);
   L.cw = W < CW ? W : CW;
   L.nchunk = W / L.cw;
-  L.nks = L.nchunk >= L.G ? 1 : L.G / L.nchunk;
+  // FP64 chain: slices of k.  Two give four warps even for one column, one per scheduler,
+  // which keep its FP64 pipe busy; more only add partial sums (eight: 1024 more additions
+  // a block against 1920 FMAs at a half-bandwidth of 15).
+  L.nks = L.nchunk >= L.G ? 1 : (fp64 ? 2 : L.G / L.nchunk);
   unsigned red = kRedBytes;
   if (bchol) {
     const unsigned part = (unsigned)(L.nks * 64 * (W + 1)) * esz, xin = 64u * (unsigned)W * esz;
@@ -213,56 +216,58 @@ __device__ __forceinline__ float2 cadd_(float2 a, float2 b) { return make_float2
 __device__ __forceinline__ double2 cadd_(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 
 // ------------------------------------------------------------ triangular pass, FP64
-// Same products in FP64: one warp per (block, column chunk), lane l owns rows
-// l and l + 32, each over its triangle; tiles read through L2 (the pass is
-// bound by the FP64 FMA rate).  No barrier at the end.
+// The triangles of D_i^-1 and D_i^-T for a warp that owns row pairs: lane l takes the
+// rows l and 63 - l, whose entries together are 65 for every lane.  Entry j of lane l
+// lies at j * 32 + l of the tile: the shorter row's l + 1 entries first, then the
+// longer one's, each by ascending k.
+constexpr int kTriTile = 65 * 32;
+struct TriEntry {
+  int row, k;
+};
+__host__ __device__ __forceinline__ TriEntry tri_entry(bool lower, int lane, int j) {
+  if (lower) return j <= lane ? TriEntry{lane, j} : TriEntry{63 - lane, j - lane - 1};
+  return j <= lane ? TriEntry{63 - lane, 63 - lane + j} : TriEntry{lane, j - 1};
+}
+
+// One warp per (block, column chunk); tiles read through L2.  The FP64 FMA rate bounds
+// it (two lanes a clock and SM), so what counts is the FMAs issued: with rows l and
+// l + 32 a lane, every warp instruction ran its masked half too, 96 per column and block
+// against 65 here (with the chain's two slices: 480 orbitals, all columns, 247.9 ->
+// 209.3 ms).  No barrier at the end.
 template <bool LOWER, int CWV, typename InT>
-__device__ __noinline__ void bc_tri_f64(const Args& a, const Smem& sm, const double* __restrict__ Mall,
-                                        const InT* __restrict__ in, double2* __restrict__ out) {
+__device__ __noinline__ void bc_tri_f64(const Args& a, const Smem& sm, const InT* __restrict__ in,
+                                        double2* __restrict__ out) {
   const int W = a.W, N4 = 4 * a.m.nb, nblk = a.m.bf_nblk;
   const int nchunk = W / CWV, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const TriEntry s0 = tri_entry(LOWER, lane, 0), s1 = tri_entry(LOWER, lane, lane + 1);
   for (int task = warp; task < nblk * nchunk; task += NWARP) {
     const int blk = task / nchunk, ch = task - blk * nchunk, c0 = ch * CWV, base = 64 * blk;
-    const double* __restrict__ M = Mall + (size_t)blk * 4096;
-    double2 acc0[CWV], acc1[CWV];
+    const double* __restrict__ M = a.m.bft + (size_t)(2 * blk + (LOWER ? 0 : 1)) * kTriTile + lane;
+    const int kmax = N4 - base;  // rows of the vector from the block on
+    double2 acc[CWV], res[CWV];
 #pragma unroll
-    for (int j = 0; j < CWV; ++j) {
-      acc0[j] = czero<double2>();
-      acc1[j] = czero<double2>();
-    }
-    const int kmax = min(64, N4 - base);
-    const int k32 = min(32, kmax);
-#pragma unroll 4
-    for (int k = 0; k < k32; ++k) {  // LOWER: row l needs k <= l, row l+32 all; UPPER: only row l (k >= l)
-      const size_t e = (size_t)(base + k) * W + c0;
-      const bool u0 = LOWER ? k <= lane : k >= lane;
-      const double m0 = u0 ? __ldg(M + k * 64 + lane) : 0.0;
-      const double m1 = LOWER ? __ldg(M + k * 64 + 32 + lane) : 0.0;
+    for (int c = 0; c < CWV; ++c) acc[c] = res[c] = czero<double2>();
+    int k = s0.k;
+#pragma unroll (CWV == 1 ? 4 : 2)
+    for (int j = 0; j < 65; ++j, ++k) {
+      if (j == lane + 1) {
+        k = s1.k;
 #pragma unroll
-      for (int j = 0; j < CWV; ++j) {
-        const double2 v = bc_in(in, e + j);
-        if (u0) cfma(acc0[j], m0, v);
-        if (LOWER) cfma(acc1[j], m1, v);
+        for (int c = 0; c < CWV; ++c) {
+          res[c] = acc[c];
+          acc[c] = czero<double2>();
+        }
       }
-    }
-#pragma unroll 4
-    for (int k = 32; k < kmax; ++k) {  // LOWER: only row l+32 (k <= l+32); UPPER: row l all, row l+32 k >= l+32
-      const size_t e = (size_t)(base + k) * W + c0;
-      const bool u1 = LOWER ? k <= lane + 32 : k >= lane + 32;
-      const double m0 = LOWER ? 0.0 : __ldg(M + k * 64 + lane);
-      const double m1 = u1 ? __ldg(M + k * 64 + 32 + lane) : 0.0;
+      const double m = __ldg(M + j * 32);
 #pragma unroll
-      for (int j = 0; j < CWV; ++j) {
-        const double2 v = bc_in(in, e + j);
-        if (!LOWER) cfma(acc0[j], m0, v);
-        if (u1) cfma(acc1[j], m1, v);
-      }
+      for (int c = 0; c < CWV; ++c)
+        cfma(acc[c], m, k < kmax ? bc_in(in, (size_t)(base + k) * W + c0 + c) : czero<double2>());
     }
 #pragma unroll
-    for (int j = 0; j < CWV; ++j) {
-      if (!sm.act[c0 + j]) continue;
-      if (base + lane < N4) out[(size_t)(base + lane) * W + c0 + j] = acc0[j];
-      if (base + lane + 32 < N4) out[(size_t)(base + lane + 32) * W + c0 + j] = acc1[j];
+    for (int c = 0; c < CWV; ++c) {
+      if (!sm.act[c0 + c]) continue;
+      if (s0.row < kmax) out[(size_t)(base + s0.row) * W + c0 + c] = res[c];
+      if (s1.row < kmax) out[(size_t)(base + s1.row) * W + c0 + c] = acc[c];
     }
   }
 }
@@ -355,10 +360,10 @@ template <int CWV, int PF>
 __device__ void bc_solve_w(const Args& a, Smem& sm, const double2* f, double2* x, double2* t1, double2* t2) {
   const size_t part = (size_t)a.m.bf_nblk * 4096;
   const double* bf = a.m.bf64;
-  bc_tri_f64<true, CWV>(a, sm, bf, f, t1);
+  bc_tri_f64<true, CWV>(a, sm, f, t1);
   __syncthreads();
   bc_chain64<CWV, PF, true>(a, sm, bf + 2 * part, t1, t1);
-  bc_tri_f64<false, CWV>(a, sm, bf + part, t1, t2);
+  bc_tri_f64<false, CWV>(a, sm, t1, t2);
   __syncthreads();
   bc_chain64<CWV, PF, false>(a, sm, bf + 3 * part, t2, x);
   if (threadIdx.x == 0) ++sm.inner_count;

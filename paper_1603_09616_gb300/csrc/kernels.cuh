@@ -69,6 +69,7 @@ struct DevMat {
   // head / tail fragments of the same tiles (gb::FactorTiles, factor_passes.cuh).
   int bf_bw, bf_nblk;
   const double* bf64;
+  const double* bft;  // the FP64 triangles, by row pairs (bc_tri_f64)
   const float* bfm;  // the seed recurrence's TF32 tiles (seed_passes.cuh)
   const uint4* fx;
   int fx_ne, fx_lg;

@@ -492,6 +492,18 @@ __global__ void __launch_bounds__(256) tile_kernel(TileArgs a) {
   }
 }
 
+// The FP64 solve's triangles by row pairs (bc_tri_f64), one block of threads per 64-row
+// block and direction.
+__global__ void __launch_bounds__(256) tri_pack_kernel(const double* __restrict__ bf, size_t part,
+                                                       double* __restrict__ out) {
+  const int blk = blockIdx.x >> 1, dir = blockIdx.x & 1;
+  const double* D = bf + dir * part + (size_t)blk * 4096;
+  for (int e = threadIdx.x; e < gbk::kTriTile; e += 256) {
+    const gbk::TriEntry t = gbk::tri_entry(dir == 0, e & 31, e >> 5);
+    out[(size_t)blockIdx.x * gbk::kTriTile + e] = D[t.k * 64 + t.row];
+  }
+}
+
 cudaError_t form_on_device(const gbk::DevMat& d, size_t nnzb, const FactorTiles& ft, cudaStream_t s) {
   auto split = [&](const double* v, size_t n, const float* hi, const float* lo) {
     const unsigned blocks = (unsigned)std::min<size_t>((n + 255) / 256, 152 * 8);
@@ -515,6 +527,7 @@ cudaError_t form_on_device(const gbk::DevMat& d, size_t nnzb, const FactorTiles&
     t.fx = reinterpret_cast<uint32_t*>(const_cast<uint4*>(d.fx));
     t.tf = const_cast<float*>(d.bfm);
     tile_kernel<<<2 * d.bf_nblk, 256, 0, s>>>(t);
+    tri_pack_kernel<<<2 * d.bf_nblk, 256, 0, s>>>(d.bf64, t.part, const_cast<double*>(d.bft));
   }
   return cudaGetLastError();
 }
@@ -652,6 +665,7 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   const size_t o_sh = take(sizeof(float) * nnzb * 16), o_sl = take(sizeof(float) * nnzb * 16);
   const size_t o_m32 = take(sizeof(float) * nbl * 16), o_hd = take(sizeof(float) * n);
   const size_t o_bfm = take(sizeof(float) * 2 * nblk * gbk::kMmaTileFloatsDev);
+  const size_t o_bft = take(sizeof(double) * 2 * nblk * gbk::kTriTile);
   const size_t o_fx = take(sizeof(uint4) * 2 * nblk * gbk::fx_block_words(ft.ne));
   const bool dense = dense_wanted(n, nbf != 0);
   const size_t dnt = dense ? (4 * nbl + 15) / 16 : 0;
@@ -711,6 +725,7 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   d.bf_bw = nbf ? hb.bf_bw : 0;
   d.bf_nblk = nbf ? (int)hb.bf_nblk : 0;
   d.bf64 = nbf ? reinterpret_cast<const double*>(b + o_bf64) : nullptr;
+  d.bft = nbf ? reinterpret_cast<const double*>(b + o_bft) : nullptr;
   d.fx = nbf ? reinterpret_cast<const uint4*>(b + o_fx) : nullptr;
   d.fx_ne = ft.ne;
   d.fx_lg = ft.lg;
