@@ -233,15 +233,15 @@ __host__ __device__ __forceinline__ TriEntry tri_entry(bool lower, int lane, int
 // it (two lanes a clock and SM), so what counts is the FMAs issued: with rows l and
 // l + 32 a lane, every warp instruction ran its masked half too, 96 per column and block
 // against 65 here (with the chain's two slices: 480 orbitals, all columns, 247.9 ->
-// 209.3 ms).  No barrier at the end.
+// 209.3 ms).  Blocks b0 .. b0 + nblk - 1.  No barrier at the end.
 template <bool LOWER, int CWV, typename InT>
-__device__ __noinline__ void bc_tri_f64(const Args& a, const Smem& sm, const InT* __restrict__ in,
-                                        double2* __restrict__ out) {
-  const int W = a.W, N4 = 4 * a.m.nb, nblk = a.m.bf_nblk;
+__device__ __noinline__ void bc_tri_f64(const Args& a, const Smem& sm, const InT* in, double2* out, int b0,
+                                        int nblk) {
+  const int W = a.W, N4 = 4 * a.m.nb;
   const int nchunk = W / CWV, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const TriEntry s0 = tri_entry(LOWER, lane, 0), s1 = tri_entry(LOWER, lane, lane + 1);
   for (int task = warp; task < nblk * nchunk; task += NWARP) {
-    const int blk = task / nchunk, ch = task - blk * nchunk, c0 = ch * CWV, base = 64 * blk;
+    const int at = task / nchunk, ch = task - at * nchunk, blk = b0 + at, c0 = ch * CWV, base = 64 * blk;
     const double* __restrict__ M = a.m.bft + (size_t)(2 * blk + (LOWER ? 0 : 1)) * kTriTile + lane;
     const int kmax = N4 - base;  // rows of the vector from the block on
     double2 acc[CWV], res[CWV];
@@ -360,10 +360,10 @@ template <int CWV, int PF>
 __device__ void bc_solve_w(const Args& a, Smem& sm, const double2* f, double2* x, double2* t1, double2* t2) {
   const size_t part = (size_t)a.m.bf_nblk * 4096;
   const double* bf = a.m.bf64;
-  bc_tri_f64<true, CWV>(a, sm, f, t1);
+  bc_tri_f64<true, CWV>(a, sm, f, t1, 0, a.m.bf_nblk);
   __syncthreads();
   bc_chain64<CWV, PF, true>(a, sm, bf + 2 * part, t1, t1);
-  bc_tri_f64<false, CWV>(a, sm, t1, t2);
+  bc_tri_f64<false, CWV>(a, sm, t1, t2, 0, a.m.bf_nblk);
   __syncthreads();
   bc_chain64<CWV, PF, false>(a, sm, bf + 3 * part, t2, x);
   if (threadIdx.x == 0) ++sm.inner_count;

@@ -11,6 +11,7 @@
 
 #include "gb_internal.h"
 #include "team_kernels.cuh"
+#include "wavepacket_cluster.cuh"
 
 namespace gb {
 
@@ -3024,7 +3025,8 @@ gb_status gb_add_sinv_terms(const gb_matrix* m, const gb_solve_params* p, double
 // with T_{k+1} = 2 A~ T_k - T_{k-1}.  Each term costs one H product and one
 // FP64 factor solve; the series stops where |J_k(a tau)| < 1e-17.  One team
 // per chunk of W wavepackets runs every step (persistent); W is the smallest
-// power of two that spreads the packets over the SMs (at most 32).
+// power of two that spreads the packets over the SMs (at most 32).  Where two or more
+// SMs are left for each packet, a cluster of teams shares it (wavepacket_cluster.cuh).
 namespace {
 
 constexpr int kWpMaxTerms = 256;
@@ -3107,6 +3109,30 @@ __global__ void __launch_bounds__(gbk::TPB, 1)
   if (tid == 0 && sm.bc_fail) atomicOr(status, gbk::kStTimeout);
 }
 
+// Launches the cluster kernel if clusters of CS for all packets are resident at once; *e:
+// the launch's result.
+template <int CS, typename... A>
+bool wp_cluster(int nwp, cudaStream_t s, cudaError_t* e, A... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(nwp * CS));
+  cfg.blockDim = dim3(gbk::TPB);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CS;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  int resident = 0;
+  if (cudaOccupancyMaxActiveClusters(&resident, gbk::wavepacket_cluster_kernel<CS>, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (resident < nwp) return false;
+  *e = cudaLaunchKernelEx(&cfg, gbk::wavepacket_cluster_kernel<CS>, args...);
+  return true;
+}
+
 }  // namespace
 
 extern "C" {
@@ -3172,19 +3198,30 @@ gb_status gb_wavepacket(const gb_matrix* m, int32_t nwp, void* psi, int32_t nste
   const unsigned chunks = (unsigned)((nwp + wc - 1) / wc);
   GB_CUDA(cudaMemcpyAsync(d_coef, coef.data(), 16 * (size_t)nterms, cudaMemcpyHostToDevice, s));
   GB_CUDA(cudaMemsetAsync(d_st, 0, sizeof(int), s));
-  GB_CUDA(cudaMemsetAsync(scratch, 0, (size_t)chunks * 7 * panel, s));
   gbk::Args a;
   std::memset(&a, 0, sizeof a);
   a.m = m->dm;
   a.W = wc;
   a.inner_bchol = 1;
   a.bc_bw_alloc = m->dm.bf_bw;
-  const size_t dyn = gbk::dyn_layout(true, wc, true, 0, m->dm.bf_bw).bytes;
-  GB_CUDA(cudaFuncSetAttribute(wavepacket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
   const double2 phase = make_double2(std::cos(cb * tau), -std::sin(cb * tau));
-  wavepacket_kernel<<<chunks, gbk::TPB, dyn, s>>>(a, static_cast<double2*>(psi), nwp, nsteps, d_coef, nterms, ca, cb,
-                                                   phase, scratch, panel, d_st);
-  GB_CUDA(cudaGetLastError());
+  auto* x = static_cast<double2*>(psi);
+  cudaError_t ce = cudaSuccess;
+  auto cluster = [&](auto cs) {
+    return wp_cluster<decltype(cs)::value>(nwp, s, &ce, a, x, (int)nwp, (int)nsteps, (const double2*)d_coef, nterms, ca,
+                                           cb, phase, scratch, panel, d_st);
+  };
+  if (wc == 1 && (cluster(std::integral_constant<int, 8>{}) || cluster(std::integral_constant<int, 4>{}) ||
+                  cluster(std::integral_constant<int, 2>{}))) {
+    GB_CUDA(ce);
+  } else {
+    const size_t dyn = gbk::dyn_layout(true, wc, true, 0, m->dm.bf_bw).bytes;
+    GB_CUDA(cudaFuncSetAttribute(wavepacket_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn));
+    GB_CUDA(cudaMemsetAsync(scratch, 0, (size_t)chunks * 7 * panel, s));
+    wavepacket_kernel<<<chunks, gbk::TPB, dyn, s>>>(a, x, nwp, nsteps, d_coef, nterms, ca, cb, phase, scratch, panel,
+                                                     d_st);
+    GB_CUDA(cudaGetLastError());
+  }
   int hst = 0;
   GB_CUDA(cudaMemcpyAsync(&hst, d_st, sizeof(int), cudaMemcpyDeviceToHost, s));
   GB_CUDA(cudaStreamSynchronize(s));
