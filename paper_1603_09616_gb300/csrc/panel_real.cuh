@@ -155,8 +155,9 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
       gbff::acc_init(d1);
       const int e0 = sm.act[c] ? tid : (int)NE;
       const bool factor = a.inner_bchol || a.inner_dense;
+      int levels = 0;
       if (factor)
-        inner_real_factor(a, sm, f, cg_x, cg_g, cg_d, cg_q, U);
+        levels = inner_real_factor(a, sm, f, cg_x, cg_g, cg_d, cg_q, U);
       else
         inner_mixed<true>(a, sm, f, v, cg_x, cg_g, cg_d, cg_q, dyn);
       const float2 *x0 = cg_x, *x1 = cg_x + NE, *x2 = cg_g + NE, *x3 = cg_d + NE;
@@ -166,17 +167,17 @@ __device__ void solve_panel_real(const Args& a, RealSmem& sm, char* ws, char* dy
         float4 vv;
         if (factor) {  // v = the levels' sum, smallest first
           gbff::ff p{0.f, 0.f}, q{0.f, 0.f};
-          if (a.bc_levels > 3) {
+          if (levels > 3) {
             const float2 t = x3[e];
             p.hi = t.x;
             q.hi = t.y;
           }
-          if (a.bc_levels > 2) {
+          if (levels > 2) {
             const float2 t = x2[e];
             p = gbff::two_sum(t.x, p.hi);
             q = gbff::two_sum(t.y, q.hi);
           }
-          if (a.bc_levels > 1) {
+          if (levels > 1) {
             const float2 t = x1[e];
             p = gbff::ff_add(gbff::ff{t.x, 0.f}, p);
             q = gbff::ff_add(gbff::ff{t.y, 0.f}, q);
