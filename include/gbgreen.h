@@ -241,7 +241,9 @@ typedef struct {
   int32_t* inner_iters; /* [nrhs] inner steps of the column's panel summed over
                            the whole solve and all refinement levels: CG
                            iterations, Chebyshev steps, or one per level for
-                           the exact factor solve and the dense inverse      */
+                           the exact factor solve and the dense inverse (a
+                           fourth level that is left out because it cannot
+                           change the sum is counted with them)             */
   int32_t* col_status;  /* [nrhs] bit flags per column: 1 COCG breakdown, 2 S not
                            SPD, 4 a shift missed tol, 8 inner CG hit its cap,
                            16 a bounded wait for a factor tile gave up,

@@ -783,7 +783,10 @@ __device__ __noinline__ int inner_real_factor(const Args& a, Smem& sm, const flo
   }
   if (a.bc_levels <= 3) return a.bc_levels;
   const bool need = m0 != 0.f && !(4.f * m2 * fmaxf(m1 / m0, m2 / m1) <= 0x1p-56f * m0);
-  if (!__syncthreads_or(need)) return 3;
+  if (!__syncthreads_or(need)) {
+    if (threadIdx.x == 0) ++sm.inner_count;  // counted with the levels asked for
+    return 3;
+  }
   real_residual<3>(a, sm, U, g + NE, er, g);
   solve(g, d + NE);
   return 4;
