@@ -6,6 +6,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <memory>
 #include <vector>
 
@@ -2210,6 +2211,48 @@ struct BatchPlan {
   gbk::Args proto;
 };
 
+// A system's estimated time in a batch: its iterations grow like n^0.6 (152 to 912
+// orbitals: 396 to 1130) and the time of each like n, beside the shift polynomials.
+double batch_cost(const gb_matrix* m, const gb_solve_params* p) {
+  const double n = (double)m->n;
+  return std::pow(n, 0.6) * (n + 0.25 * p->nshift);
+}
+
+// The panel width of a mixed batch on wide teams, one per SM, at most C.  A batch of
+// unequal systems waits for its largest, whose panels get faster with fewer columns (24
+// systems: 290, 220, 181 ms with 8, 4, 2), while the small ones can share SMs: so a
+// narrower width is taken where the modelled finishing time of the work queue (largest
+// first) is at least 12 % shorter.  GB300, uneven chains of 8 columns, 8 / 4 / 2 columns a
+// panel: 96 of up to 32 monomers 446 / 354 / 379 ms (taken: 4), 40 398 / 308 / 265 (2), 60
+// of up to 20 240 / 189 / 151 (2), 150 of up to 12 161 / 137 / 234 (4).
+int batch_width(int nsys, const gb_matrix* const* mats, const gb_solve_params* params, const std::vector<int>& order,
+                int nsm, int C) {
+  auto relative = [](int cols) { return cols == 8 ? 1.6 : cols == 4 ? 1.21 : cols == 2 ? 1.0 : 0.3 * cols; };
+  double best = 0.0;
+  int width = C;
+  for (int cand = C; cand >= 2; cand /= 2) {
+    std::vector<double> busy((size_t)nsm, 0.0);  // a heap, the first SM to be free on top
+    long long panels = 0;
+    for (int s = 0; s < nsys; ++s) panels += (params[s].nrhs + cand - 1) / cand;
+    if (panels > 8LL * nsm) break;
+    double end = 0.0;
+    for (int q = 0; q < nsys; ++q) {
+      const int s = order[q];
+      const double t = relative(cand) * batch_cost(mats[s], &params[s]);
+      for (int k = (params[s].nrhs + cand - 1) / cand; k > 0; --k) {
+        std::pop_heap(busy.begin(), busy.end(), std::greater<double>());
+        busy.back() += t;
+        end = std::max(end, busy.back());
+        std::push_heap(busy.begin(), busy.end(), std::greater<double>());
+      }
+    }
+    if (best > 0.0 && end >= 0.88 * best) continue;
+    best = end;
+    width = cand;
+  }
+  return width;
+}
+
 gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_solve_params* params,
                           const gb_outputs* outs, int32_t panel, BatchPlan* bp) {
   if (nsys < 1 || !mats || !params) return fail(GB_EINVAL, "need nsys >= 1, mats and params");
@@ -2254,22 +2297,36 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
       per_sm = 1;
     return per_sm;
   };
+  // largest systems first for load balance
+  bp->order.resize(nsys);
+  for (int s = 0; s < nsys; ++s) bp->order[s] = s;
+  std::stable_sort(bp->order.begin(), bp->order.end(),
+                   [&](int x, int y) { return batch_cost(mats[x], &params[x]) > batch_cost(mats[y], &params[y]); });
   int C = panel;
+  bool wide = false;  // wide teams, one per SM
   if (C <= 0) {  // widest panel that still gives every resident team a work item
     auto panels = [&](int cand) {
       long long np = 0;
       for (int s = 0; s < nsys; ++s) np += (params[s].nrhs + cand - 1) / cand;
       return np;
     };
+    int cap = 2;  // wider panels would stay partly empty in every system
+    for (int s = 0; s < nsys; ++s)
+      while (cap < 32 && cap < params[s].nrhs) cap *= 2;
     C = 1;
-    if (real && prec == GB_MIXED) {  // as in make_plan
+    if (real && prec == GB_MIXED) {
+      // wide teams where one wave holds every panel (as in make_plan), or where no system
+      // has more than 8 columns: 300 chains of 8, wide teams / 512 threads, 8 columns a
+      // panel 303 / 367 ms, 4 columns 382 / 322
       C = 2;
-      while (C < 32 && panels(C) > nsm) C *= 2;
+      while (C < cap && panels(C) > nsm) C *= 2;
+      wide = panels(C) <= nsm || C == 8;
+      if (wide) C = batch_width(nsys, mats, params, bp->order, nsm, C);
     }
-    if (C == 1 || panels(C) > nsm) {
+    if (!wide) {
       C = 1;
       for (int cand : {32, 16, 8, 4, 2})
-        if (4 * panels(cand) >= 3LL * nsm * occupancy(dyn_bytes(width(cand)))) {
+        if (cand <= cap && 4 * panels(cand) >= 3LL * nsm * occupancy(dyn_bytes(width(cand)))) {
           C = cand;
           break;
         }
@@ -2296,14 +2353,9 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   bp->proto.C = C;
   bp->total_panels = 0;
   for (int s = 0; s < nsys; ++s) bp->total_panels += (params[s].nrhs + C - 1) / C;
-  bp->teams = std::min(bp->total_panels, nsm * per_sm);
-  bp->threads = real && prec != GB_FP64 && bp->total_panels <= nsm ? gbk::TPB_WIDE : gbk::TPB;
-  // largest systems first (cost ~ basis size x shifts) for load balance
-  bp->order.resize(nsys);
-  for (int s = 0; s < nsys; ++s) bp->order[s] = s;
-  std::stable_sort(bp->order.begin(), bp->order.end(), [&](int x, int y) {
-    return (double)mats[x]->n * params[x].nshift > (double)mats[y]->n * params[y].nshift;
-  });
+  wide = wide || (real && prec != GB_FP64 && bp->total_panels <= nsm);
+  bp->teams = std::min(bp->total_panels, wide ? nsm : nsm * per_sm);
+  bp->threads = wide ? gbk::TPB_WIDE : gbk::TPB;
   // header: descriptors, panel prefix, counter, then per-system arrays
   size_t hb = align256(sizeof(gbk::Args) * nsys) + align256(sizeof(int) * (nsys + 1)) + 256;
   for (int s = 0; s < nsys; ++s)
