@@ -20,7 +20,7 @@
  * conjugate orthogonal CG (COCG) in the S-bilinear form with that seed.
  * S^{-1} is applied exactly by a block-bidiagonal Cholesky factor of S where
  * S's half-bandwidth is at most 63 (chains); else, in the mixed path, by the
- * dense inverse of an S of at most 1024 orbitals; else by an inner
+ * dense inverse of a well-scaled S of at most 1024 orbitals; else by an inner
  * block-Jacobi-preconditioned iteration (CG, or Chebyshev in the mixed path).
  * The paper defers the method's details to its references; the recurrences
  * used are the standard ones.
@@ -201,8 +201,9 @@ typedef struct {
                             half-bandwidth is <= 63 (FP64: one solve; mixed: two
                             FP32 solves around a float-float residual), else
                             (mixed, the real recurrence) the dense inverse of
-                            an S of at most 1024 orbitals, refined as well, else
-                            an iteration (FP64: CG; mixed: Chebyshev).
+                            an S of at most 1024 orbitals with max |S| max
+                            |S^-1| <= 64, refined as well, else an iteration
+                            (FP64: CG; mixed: Chebyshev).
                             bit 1: keep the inner-iteration vectors of a panel
                             in shared memory when they fit (iterations only;
                             no dense inverse);

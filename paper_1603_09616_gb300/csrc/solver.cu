@@ -542,9 +542,13 @@ cudaError_t form_on_device(const gbk::DevMat& d, size_t nnzb, const FactorTiles&
 constexpr int kDenseMax = 1024;
 bool dense_wanted(int64_t n, bool factor) { return !factor && n <= kDenseMax; }
 
-// Forms d.di; leaves it null where S is not SPD or the scratch cannot be had (the
-// solves then iterate, and report such an S as before).
-cudaError_t form_dense_inverse(gbk::DevMat& d, uint4* frags, cudaStream_t s) {
+// Forms d.di; leaves it null where S is not SPD, the scratch cannot be had, or S is badly
+// scaled or conditioned (the solves then iterate, and report such an S as before).  An FP32
+// solve is accurate to some 1e-6 of the solution's largest entry, so a refinement level
+// shrinks the residual by 1e-6 max |S| max |S^-1| and a few: 64 leaves 1e-4 (bundles: the
+// product is 1.02).  s_max: max |S|.
+constexpr double kDenseCond = 64.0;
+cudaError_t form_dense_inverse(gbk::DevMat& d, uint4* frags, double s_max, cudaStream_t s) {
   const int np = (d.n + gbk::kDiB - 1) / gbk::kDiB * gbk::kDiB, nblk = np / gbk::kDiB, nt = (4 * d.nb + 15) / 16;
   const size_t one = sizeof(double) * (size_t)np * np, piv = sizeof(double) * gbk::kDiB * np;
   char* tmp = nullptr;
@@ -575,7 +579,7 @@ cudaError_t form_dense_inverse(gbk::DevMat& d, uint4* frags, cudaStream_t s) {
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   double mx;
   std::memcpy(&mx, &h.top, sizeof mx);
-  if (e == cudaSuccess && !h.bad && std::isfinite(mx) && mx > 0.0) {
+  if (e == cudaSuccess && !h.bad && std::isfinite(mx) && mx > 0.0 && mx * s_max <= kDenseCond) {
     int ex;
     std::frexp(mx, &ex);
     if (ex > -40 && ex < 40) {  // largest entry in [2^14, 2^15)
@@ -739,7 +743,11 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   e = cudaMemcpyAsync(m->base, host.get(), up, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = form_on_device(d, nnzb, ft, s);
   d.di = nullptr;
-  if (e == cudaSuccess && dense) e = form_dense_inverse(d, reinterpret_cast<uint4*>(b + o_di), s);
+  if (e == cudaSuccess && dense) {
+    double s_max = 0.0;
+    for (double v : hb.s_val) s_max = std::max(s_max, std::fabs(v));
+    e = form_dense_inverse(d, reinterpret_cast<uint4*>(b + o_di), s_max, s);
+  }
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) {
     cudaFree(m->base);
@@ -880,8 +888,11 @@ void set_inner_method(const gb_matrix* m, const gb_solve_params* p, double itol,
     return;
   }
   if (dense_inner(m, p, real)) {
-    a.inner_dense = 1;  // an iteration's inner_tol holds per level, of which there are two
-    a.bc_levels = refinement_levels(p->tol, p->inner_tol * p->inner_tol);
+    // an iteration's inner_tol (1e-7 by default) holds per level, of which there are two:
+    // an application's error stays below its square
+    a.inner_dense = 1;
+    a.bc_levels = p->inner_tol > 0 ? refinement_levels(p->tol, p->inner_tol * p->inner_tol)
+                                   : std::max(3, refinement_levels(p->tol, 0.0));
     return;
   }
   const double lmin = m->dm.s_lam_min * 0.98, lmax = m->dm.s_lam_max * 1.02;

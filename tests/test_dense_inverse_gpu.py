@@ -56,3 +56,15 @@ def test_dense_inverse_solves(n, scale, panel):
     err = np.abs(out["g_proj"].cpu().numpy() - want).max()
     mat.close()
     assert err <= 2 * tol / (eta * np.linalg.eigvalsh(S)[0])
+
+
+def test_badly_scaled_overlap_iterates():
+    # S and H scaled by 10 on every third orbital: max |S| max |S^-1| is above 64
+    system = shuffled(200, 1.0)
+    d = np.where(np.arange(system.n) % 3 == 0, 10.0, 1.0)
+    f = d[np.repeat(np.arange(system.n), np.diff(system.row_ptr))] * d[system.col_idx]
+    system.h_val, system.s_val = system.h_val * f, system.s_val * f
+    mat = gbg.Matrix(system)
+    plan = gbg.solve_plan(mat, shift_grid(-6.0, 6.0, 9, 0.4), np.arange(8), prec="mixed")
+    mat.close()
+    assert plan["inner"] == "chebyshev"
