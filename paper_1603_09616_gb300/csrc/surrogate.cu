@@ -162,16 +162,22 @@ __device__ __forceinline__ float gelu_grad(float x) {
 }
 
 // The network runs in three kernels: all four layers forward, the gradients of the
-// activations backward, and the weight gradients of all layers.  The 0.5 GFLOP of a
-// training step at batch 2048 are 1 us of tensor cores; what counts is launches and
-// latency, so a block takes 16 samples through every layer with the activations in
-// shared memory.
+// activations backward, and the weight gradients of all layers.  The 0.25 G products
+// of a training step at batch 2048 are 7 us of the FP32 pipes; what counts beside them
+// is launches and latency, so a block takes 16 samples through every layer with the
+// activations in shared memory.
 //
-// FP32 accuracy on BF16 MMAs: an activation (or gradient) is the sum of three BF16
-// values, its 24 bits, and the weights are BF16 already, so three exact products
-// with FP32 accumulation take the place of one FP32 product.
+// Every product's sum runs over its index in ascending order in one FP32 accumulator.
+// Adam's first steps divide a gradient by its own magnitude (beside eps = 1e-8), so a
+// bias whose gradient cancels over the batch shows the order of the additions: sums in
+// slices, or in the tensor cores' order, are as exact, but moved such a step by 1e-3 of
+// the learning rate.  GB300, batch 2048: a step takes 80 us, most of it the host's (92 with
+// three-way BF16 splits on the tensor cores and the batch in slices; 610 with a launch of
+// 32 x 32 tiles for each product).
 constexpr int kMlpThreads = 512;
-constexpr int kRows = 16, kPad = GB_MLP_MAXW + 8;  // samples per block; row pitch of a plane (bank-conflict free)
+constexpr int kRows = 16;                  // samples per block
+constexpr int kPad = GB_MLP_MAXW + 8;      // row pitch of a weight plane (16 bytes a row more: no bank conflicts)
+constexpr int kXPad = GB_MLP_MAXW + 4;     // and of the activations
 
 struct Net {
   int dims[GB_MLP_LAYERS + 1];
@@ -182,37 +188,7 @@ struct Net {
 // the gradient G of P, all [batch][width].
 struct Acts {
   float *P[GB_MLP_LAYERS], *A[GB_MLP_LAYERS], *G[GB_MLP_LAYERS];
-  float* part;  // weight-gradient partials
 };
-
-struct Planes {
-  __nv_bfloat16 v[3][kRows][kPad];
-};
-__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"((uint32_t)__cvta_generic_to_shared(p)));
-}
-__device__ __forceinline__ void ldsm2(uint32_t& r0, uint32_t& r1, const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];"
-               : "=r"(r0), "=r"(r1)
-               : "r"((uint32_t)__cvta_generic_to_shared(p)));
-}
-__device__ __forceinline__ void ldsm2_trans(uint32_t& r0, uint32_t& r1, const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];"
-               : "=r"(r0), "=r"(r1)
-               : "r"((uint32_t)__cvta_generic_to_shared(p)));
-}
-__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// A fragment of plane p, columns 16 kk ..: lane l names row l % 16, column half l / 16.
-__device__ __forceinline__ const void* a_row(const Planes& s, int p, int kk, int lane) {
-  return &s.v[p][lane & 15][16 * kk + 8 * (lane >> 4)];
-}
 
 // Weights W [rows][cols] into shared memory, pitch kPad, zero up to multiples of 16;
 // asynchronous (one commit group) where the rows are whole 16-byte pieces.
@@ -248,81 +224,42 @@ __device__ __forceinline__ void wait_w(int left) {
     default: asm volatile("cp.async.wait_group 3;" ::: "memory"); break;
   }
 }
-__device__ __forceinline__ float2 load2(const float* p, bool pair, bool in0, bool in1) {
-  if (pair && in1) return *reinterpret_cast<const float2*>(p);
-  return make_float2(in0 ? p[0] : 0.f, in1 ? p[1] : 0.f);
-}
-__device__ __forceinline__ void store2(float* p, bool pair, bool in0, bool in1, float2 v) {
-  if (pair && in1) {
-    *reinterpret_cast<float2*>(p) = v;
-  } else {
-    if (in0) p[0] = v.x;
-    if (in1) p[1] = v.y;
+// The 16 samples' rows of M [B][width] into shared memory, zero up to a multiple of 16 columns.
+__device__ __forceinline__ void stage_x(const float* __restrict__ M, int row0, int B, int width, float (*s)[kXPad]) {
+  const int cp = (width + 15) & ~15;
+  for (int e = threadIdx.x; e < kRows * cp; e += kMlpThreads) {
+    const int r = e / cp, c = e - r * cp;
+    s[r][c] = row0 + r < B && c < width ? M[(size_t)(row0 + r) * width + c] : 0.f;
   }
 }
-__device__ __forceinline__ bool pairs_ok(const float* p, int width) {
-  return (width & 1) == 0 && (reinterpret_cast<uintptr_t>(p) & 7) == 0;
+// The two BF16 values of a word, as FP32.
+__device__ __forceinline__ float2 bf16_pair(uint32_t v) {
+  return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
 
-// All of a network's weights stay in shared memory (115 KB for the widest one's four
-// layers with the activations: one block per SM, which is all a batch of 2048 gives).
-// w[l]: layer l, rows [dims[l+1]] x kPad, packed one after the other.
+// All of a network's weights stay in shared memory (123 KB for 64-128-128-128-2 and 153 KB
+// for the widest network, with the activations: one block per SM, which is all a batch of
+// 2048 gives).  w: layer l's rows [dims[l+1] up to 16] x kPad, packed one after the other.
 struct MlpSmem {
-  Planes x[2];
+  float x[2][kRows][kXPad];
   __nv_bfloat16 w[1][kPad];
 };
 __host__ __device__ inline int mlp_rows(const Net& n, int l) { return (n.dims[l + 1] + 15) & ~15; }
 size_t mlp_smem(const Net& n) {
   size_t rows = 0;
   for (int l = 0; l < GB_MLP_LAYERS; ++l) rows += mlp_rows(n, l);
-  return sizeof(Planes) * 2 + rows * kPad * sizeof(__nv_bfloat16);
-}
-
-// One thread's 2 x 2 outputs of its warp's 16 x 8 tile: rows g, g + 8, columns u, u + 1.
-// acc: the three planes' sums, the head's in two chains (the tensor cores truncate).
-__device__ __forceinline__ float2 tile_row(const float (&d)[4][4], int h) {
-  return make_float2((d[0][2 * h] + d[3][2 * h]) + (d[1][2 * h] + d[2][2 * h]),
-                     (d[0][2 * h + 1] + d[3][2 * h + 1]) + (d[1][2 * h + 1] + d[2][2 * h + 1]));
-}
-__device__ __forceinline__ void split3x2(Planes& p, int r, int k, float2 x) {
-  const __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y);
-  const float2 fa = __bfloat1622float2(a), y = make_float2(x.x - fa.x, x.y - fa.y);
-  const __nv_bfloat162 b = __floats2bfloat162_rn(y.x, y.y);
-  const float2 fb = __bfloat1622float2(b);
-  *reinterpret_cast<__nv_bfloat162*>(&p.v[0][r][k]) = a;
-  *reinterpret_cast<__nv_bfloat162*>(&p.v[1][r][k]) = b;
-  *reinterpret_cast<__nv_bfloat162*>(&p.v[2][r][k]) = __floats2bfloat162_rn(y.x - fb.x, y.y - fb.y);
-}
-// acc += the 16 samples' planes times the warp's eight columns of B; kk: 16-wide steps.
-// TRANS: B is stored [k][column], else [column][k].
-template <bool TRANS>
-__device__ __forceinline__ void tile_mma(float (&d)[4][4], const Planes& in, const __nv_bfloat16 (*w)[kPad], int steps,
-                                         int col0, int lane) {
-#pragma unroll 2
-  for (int kk = 0; kk < steps; ++kk) {
-    uint32_t a[3][4], b0, b1;
-#pragma unroll
-    for (int p = 0; p < 3; ++p) ldsm4(a[p], a_row(in, p, kk, lane));
-    if (TRANS)
-      ldsm2_trans(b0, b1, &w[16 * kk + (lane & 15)][col0]);
-    else
-      ldsm2(b0, b1, &w[col0 + (lane & 7)][16 * kk + 8 * ((lane >> 3) & 1)]);
-    mma_bf16(kk & 1 ? d[3] : d[0], a[0], b0, b1);
-    mma_bf16(d[1], a[1], b0, b1);
-    mma_bf16(d[2], a[2], b0, b1);
-  }
+  return sizeof(float) * 2 * kRows * kXPad + rows * kPad * sizeof(__nv_bfloat16);
 }
 
 // Every layer of 16 samples: P = A_prev W^T + b, A = gelu(P) (the last layer: Y = P).
-// Warp w forms units 8 w .. 8 w + 7.  Batch 2048: 128 blocks, one wave; bound by the
-// latency of four dependent layers (fetch of the weights, MMAs, GELU, barrier).
-// Four launches of 32 x 32 FP32 tiles took 47 us.
+// Thread: unit tid % 128 of four samples, eight terms a step (one 16-byte read of the
+// unit's weights, the samples' values broadcast to the warp).  Batch 2048: 128 blocks, one
+// wave, 17 us a call (four launches of 32 x 32 tiles 47).
 __global__ void __launch_bounds__(kMlpThreads) mlp_fwd(const Net net, const float* __restrict__ X, int B, Acts ws,
                                                        float* __restrict__ Y) {
   extern __shared__ __align__(16) char mlp_sm[];
   MlpSmem& sm = *reinterpret_cast<MlpSmem*>(mlp_sm);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int row0 = blockIdx.x * kRows, u = 8 * warp + 2 * t;
+  const int u = threadIdx.x % GB_MLP_MAXW, s0 = 4 * (threadIdx.x / GB_MLP_MAXW), row0 = blockIdx.x * kRows;
   {
     int at = 0;
 #pragma unroll
@@ -330,39 +267,48 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_fwd(const Net net, const floa
       stage_w(net.wb[l], net.dims[l + 1], net.dims[l], sm.w + at);
       at += mlp_rows(net, l);
     }
-    const int nin = net.dims[0], kp = (nin + 15) & ~15;
-    const bool pair = pairs_ok(X, nin);
-    for (int e = tid; e < kRows * kp / 2; e += kMlpThreads) {
-      const int r = 2 * e / kp, k = 2 * e - r * kp;
-      const bool in = row0 + r < B;
-      split3x2(sm.x[0], r, k, load2(X + (size_t)(row0 + r) * nin + k, pair, in && k < nin, in && k + 1 < nin));
-    }
+    stage_x(X, row0, B, net.dims[0], sm.x[0]);
   }
   int at = 0;
 #pragma unroll
   for (int l = 0; l < GB_MLP_LAYERS; ++l) {
     const int nin = net.dims[l], nout = net.dims[l + 1], np = (nout + 15) & ~15;
-    const bool last = l == GB_MLP_LAYERS - 1, in0 = u < nout, in1 = u + 1 < nout;
-    const float2 bias = make_float2(in0 ? net.b[l][u] : 0.f, in1 ? net.b[l][u + 1] : 0.f);
+    const bool last = l == GB_MLP_LAYERS - 1, in = u < nout;
+    const float bias = in ? net.b[l][u] : 0.f;
     wait_w(GB_MLP_LAYERS - 1 - l);
     __syncthreads();
-    if (8 * warp < np) {
-      float d[4][4] = {};
-      tile_mma<false>(d, sm.x[l & 1], sm.w + at, (nin + 15) / 16, 8 * warp, lane);
-      float* out = last ? Y : ws.A[l];
-      const bool pp = pairs_ok(ws.P[l], nout), po = pairs_ok(out, nout);
+    if (u < np) {
+      float acc[4] = {};
+      const __nv_bfloat16* w = sm.w[at + u];
+      const float(*x)[kXPad] = sm.x[l & 1];
+#pragma unroll 2
+      for (int k = 0; k < nin; k += 8) {
+        const uint4 wq = *reinterpret_cast<const uint4*>(w + k);
+        const float2 w01 = bf16_pair(wq.x), w23 = bf16_pair(wq.y), w45 = bf16_pair(wq.z), w67 = bf16_pair(wq.w);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int r = g + 8 * h;
-        const size_t o = (size_t)(row0 + r) * nout + u;
-        const bool in = row0 + r < B;
-        float2 p = tile_row(d, h);
-        p.x += bias.x;
-        p.y += bias.y;
-        const float2 y = last ? p : make_float2(in0 ? gelu(p.x) : 0.f, in1 ? gelu(p.y) : 0.f);
-        store2(ws.P[l] + o, pp, in && in0, in && in1, p);
-        store2(out + o, po, in && in0, in && in1, y);
-        if (!last) split3x2(sm.x[(l + 1) & 1], r, u, y);
+        for (int s = 0; s < 4; ++s) {
+          const float4 a = *reinterpret_cast<const float4*>(&x[s0 + s][k]);
+          const float4 b = *reinterpret_cast<const float4*>(&x[s0 + s][k + 4]);
+          acc[s] = fmaf(a.x, w01.x, acc[s]);
+          acc[s] = fmaf(a.y, w01.y, acc[s]);
+          acc[s] = fmaf(a.z, w23.x, acc[s]);
+          acc[s] = fmaf(a.w, w23.y, acc[s]);
+          acc[s] = fmaf(b.x, w45.x, acc[s]);
+          acc[s] = fmaf(b.y, w45.y, acc[s]);
+          acc[s] = fmaf(b.z, w67.x, acc[s]);
+          acc[s] = fmaf(b.w, w67.y, acc[s]);
+        }
+      }
+      float* out = last ? Y : ws.A[l];
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const float p = acc[s] + bias, y = last ? p : gelu(p);
+        if (in && row0 + s0 + s < B) {
+          const size_t o = (size_t)(row0 + s0 + s) * nout + u;
+          ws.P[l][o] = p;
+          out[o] = y;
+        }
+        if (!last) sm.x[(l + 1) & 1][s0 + s][u] = in ? y : 0.f;
       }
     }
     at += mlp_rows(net, l);
@@ -370,12 +316,13 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_fwd(const Net net, const floa
 }
 
 // Gradients of every layer's pre-activations for 16 samples: G of the last layer is
-// dY; G_{l-1} = (G_l W_l) gelu'(P_{l-1}).  Warp w forms columns 8 w .. 8 w + 7.
+// dY; G_{l-1} = (G_l W_l) gelu'(P_{l-1}).  Thread: columns 2 (tid % 64), + 1 of two
+// samples, four terms a step.
 __global__ void __launch_bounds__(kMlpThreads) mlp_bwd_x(const Net net, const float* __restrict__ dY, int B, Acts ws) {
   extern __shared__ __align__(16) char mlp_sm[];
   MlpSmem& sm = *reinterpret_cast<MlpSmem*>(mlp_sm);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
-  const int row0 = blockIdx.x * kRows, u = 8 * warp + 2 * t;
+  const int c = 2 * (threadIdx.x % (GB_MLP_MAXW / 2)), s0 = 2 * (threadIdx.x / (GB_MLP_MAXW / 2));
+  const int row0 = blockIdx.x * kRows;
   {
     int at = 0;
 #pragma unroll
@@ -383,171 +330,150 @@ __global__ void __launch_bounds__(kMlpThreads) mlp_bwd_x(const Net net, const fl
       stage_w(net.wb[l], net.dims[l + 1], net.dims[l], sm.w + at);
       at += mlp_rows(net, l);
     }
-    const int n = net.dims[GB_MLP_LAYERS], kp = (n + 15) & ~15;
-    for (int e = tid; e < kRows * kp / 2; e += kMlpThreads) {
-      const int r = 2 * e / kp, k = 2 * e - r * kp;
-      const bool in = row0 + r < B;
-      split3x2(sm.x[0], r, k, load2(dY + (size_t)(row0 + r) * n + k, false, in && k < n, in && k + 1 < n));
-    }
+    stage_x(dY, row0, B, net.dims[GB_MLP_LAYERS], sm.x[0]);
   }
   int at = 0;
 #pragma unroll
   for (int l = GB_MLP_LAYERS - 1, it = 0; l > 0; --l, ++it) {
     const int nin = net.dims[l], nout = net.dims[l + 1], np = (nin + 15) & ~15;
-    const bool in0 = u < nin, in1 = u + 1 < nin, pp = pairs_ok(ws.P[l - 1], nin), pg = pairs_ok(ws.G[l - 1], nin);
-    float2 pre[2];
+    float pre[2][2];
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const bool in = row0 + g + 8 * h < B;
-      pre[h] = load2(ws.P[l - 1] + (size_t)(row0 + g + 8 * h) * nin + u, pp, in && in0, in && in1);
-    }
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int j = 0; j < 2; ++j)
+        pre[s][j] = row0 + s0 + s < B && c + j < nin ? ws.P[l - 1][(size_t)(row0 + s0 + s) * nin + c + j] : 0.f;
     wait_w(GB_MLP_LAYERS - 2 - it);
     __syncthreads();
-    if (8 * warp < np) {
-      float d[4][4] = {};
-      tile_mma<true>(d, sm.x[it & 1], sm.w + at, (nout + 15) / 16, 8 * warp, lane);
+    if (c < np) {
+      float acc[2][2] = {};
+      const __nv_bfloat16(*w)[kPad] = sm.w + at;
+      const float(*g)[kXPad] = sm.x[it & 1];
+#pragma unroll 4
+      for (int o = 0; o < nout; o += 4) {
+        float2 wq[4];
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int r = g + 8 * h;
-        const bool in = row0 + r < B;
-        float2 v = tile_row(d, h);
-        v.x = in && in0 ? v.x * gelu_grad(pre[h].x) : 0.f;
-        v.y = in && in1 ? v.y * gelu_grad(pre[h].y) : 0.f;
-        store2(ws.G[l - 1] + (size_t)(row0 + r) * nin + u, pg, in && in0, in && in1, v);
-        if (l > 1) split3x2(sm.x[(it + 1) & 1], r, u, v);
+        for (int q = 0; q < 4; ++q) wq[q] = bf16_pair(*reinterpret_cast<const uint32_t*>(&w[o + q][c]));
+#pragma unroll
+        for (int s = 0; s < 2; ++s) {
+          const float4 gv = *reinterpret_cast<const float4*>(&g[s0 + s][o]);
+          const float gq[4] = {gv.x, gv.y, gv.z, gv.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            acc[s][0] = fmaf(gq[q], wq[q].x, acc[s][0]);
+            acc[s][1] = fmaf(gq[q], wq[q].y, acc[s][1]);
+          }
+        }
       }
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int j = 0; j < 2; ++j) {
+          const bool in = row0 + s0 + s < B && c + j < nin;
+          const float v = in ? acc[s][j] * gelu_grad(pre[s][j]) : 0.f;
+          if (in) ws.G[l - 1][(size_t)(row0 + s0 + s) * nin + c + j] = v;
+          if (l > 1) sm.x[(it + 1) & 1][s0 + s][c + j] = v;
+        }
     }
     at += mlp_rows(net, l);
   }
 }
 
-// dW_l = G_l^T A_{l-1} and db_l = column sums of G_l, over one slice of the batch and
-// one 64 x 64 tile of one layer (blockIdx.x: the layers' tiles in order), in FP32 on
-// the FMA pipes: both operands are FP32, and 84 M products are 2.4 us of the chip.
-// Slices give the 12 tiles of the 64-128-128-128-2 network enough blocks; their
-// partials are added in order by mlp_bwd_sum (one slice: written in place).
+// dW_l = G_l^T A_{l-1} and db_l = column sums of G_l over the whole batch, for one 16 x 16
+// tile of one layer (blockIdx.x: the layers' tiles in order).  Two warps of 2 x 2 outputs a
+// thread: a sample is two shared-memory reads and four FMAs, and the 2048 samples of an
+// output are a chain of additions whatever is done, so small tiles (168 for the
+// 64-128-128-128-2 network: one wave) take the least time.  Samples come through a ring of
+// asynchronous copies.
 struct GradOut {
   float *gw[GB_MLP_LAYERS], *gb[GB_MLP_LAYERS];
 };
-__host__ __device__ inline int mlp_slices(int batch) {  // of at least 128 samples, 32 at most
-  return batch <= 128 ? 1 : (batch >= 4096 ? 32 : (batch + 127) / 128);
-}
-__global__ void __launch_bounds__(256) mlp_bwd_w(const Net net, const float* __restrict__ X,
-                                                 const float* __restrict__ dY, int B, Acts ws, GradOut out,
-                                                 size_t stride) {
-  constexpr int KC = 32;  // samples per step, the next step's fetched meanwhile
-  __shared__ __align__(16) float gs[KC][68];
-  __shared__ __align__(16) float xs[KC][68];
+constexpr int kGradThreads = 64, kGradTile = 16, kGradStep = 64, kGradRing = 4;
+__global__ void __launch_bounds__(kGradThreads) mlp_bwd_w(const Net net, const float* __restrict__ X,
+                                                          const float* __restrict__ dY, int B, Acts ws, GradOut out) {
+  __shared__ __align__(16) float gs[kGradRing][kGradStep][kGradTile];
+  __shared__ __align__(16) float xs[kGradRing][kGradStep][kGradTile];
   // the tile's layer (unrolled: the parameters' arrays are not copied to be indexed)
-  int tile = blockIdx.x, nin = 0, nout = 0;
-  size_t at = 0, next = 0;
+  int left = blockIdx.x, tile = 0, nin = 0, nout = 0;
   const float *G = nullptr, *A = nullptr;
   float *dw = nullptr, *db = nullptr;
 #pragma unroll
   for (int l = 0; l < GB_MLP_LAYERS; ++l) {
-    const int ni = net.dims[l], no = net.dims[l + 1], nt = ((ni + 63) / 64) * ((no + 63) / 64);
-    if (tile >= 0 && tile < nt) {
+    const int ni = net.dims[l], no = net.dims[l + 1];
+    const int nt = ((ni + kGradTile - 1) / kGradTile) * ((no + kGradTile - 1) / kGradTile);
+    if (left >= 0 && left < nt) {
+      tile = left;
       nin = ni;
       nout = no;
-      at = next;
       G = l == GB_MLP_LAYERS - 1 ? dY : ws.G[l];
       A = l == 0 ? X : ws.A[l - 1];
       dw = out.gw[l];
       db = out.gb[l];
-      break;
     }
-    tile -= nt;
-    next += (size_t)no * (ni + 1);
+    left -= nt;
   }
-  const int ti = (nin + 63) / 64, o0 = 64 * (tile / ti), i0 = 64 * (tile % ti);
-  const int len = ((B + gridDim.y - 1) / gridDim.y + 31) / 32 * 32;
-  const int s0 = blockIdx.y * len, s1 = min(B, s0 + len);
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-  float acc[4][4] = {}, accb[4] = {};
-  // thread: rows tid / 16 and + 16 of a step, columns 4 (tid % 16) ..
-  const bool gq4 = (nout & 3) == 0 && (reinterpret_cast<uintptr_t>(G) & 15) == 0;
-  const bool xq4 = (nin & 3) == 0 && (reinterpret_cast<uintptr_t>(A) & 15) == 0;
-  auto fetch = [&](const float* M, int width, bool quad, int row, int c) {
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (row < s1) {
-      const float* p = M + (size_t)row * width + c;
-      if (quad) {
-        if (c < width) v = *reinterpret_cast<const float4*>(p);
-      } else {
-        if (c < width) v.x = p[0];
-        if (c + 1 < width) v.y = p[1];
-        if (c + 2 < width) v.z = p[2];
-        if (c + 3 < width) v.w = p[3];
+  const int ti = (nin + kGradTile - 1) / kGradTile, o0 = kGradTile * (tile / ti), i0 = kGradTile * (tile % ti);
+  const int tid = threadIdx.x, tx = tid % 8, ty = tid / 8;
+  const bool bias = i0 == 0;
+  // Rows s .. s + kGradStep - 1 of a matrix's 16 columns; zero beyond the batch and the width.
+  auto fetch = [&](const float* __restrict__ M, int width, int c0, int s, float (*dst)[kGradTile]) {
+    if ((width & 3) == 0 && (reinterpret_cast<uintptr_t>(M) & 15) == 0) {
+#pragma unroll
+      for (int q = 0; q < kGradStep * kGradTile / 4 / kGradThreads; ++q) {
+        const int e = tid + q * kGradThreads, r = e / (kGradTile / 4), c = 4 * (e % (kGradTile / 4));
+        const bool in = s + r < B && c0 + c < width;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(&dst[r][c])),
+                     "l"(in ? M + (size_t)(s + r) * width + c0 + c : M), "r"(in ? 16 : 0)
+                     : "memory");
+      }
+    } else {
+      for (int e = tid; e < kGradStep * kGradTile; e += kGradThreads) {
+        const int r = e / kGradTile, c = e % kGradTile;
+        const bool in = s + r < B && c0 + c < width;
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"((uint32_t)__cvta_generic_to_shared(&dst[r][c])),
+                     "l"(in ? M + (size_t)(s + r) * width + c0 + c : M), "r"(in ? 4 : 0)
+                     : "memory");
       }
     }
-    return v;
   };
-  float4 gn[2], xn[2];
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    gn[q] = fetch(G, nout, gq4, s0 + ty + 16 * q, o0 + 4 * tx);
-    xn[q] = fetch(A, nin, xq4, s0 + ty + 16 * q, i0 + 4 * tx);
-  }
-  for (int s = s0; s < s1; s += KC) {
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      *reinterpret_cast<float4*>(&gs[ty + 16 * q][4 * tx]) = gn[q];
-      *reinterpret_cast<float4*>(&xs[ty + 16 * q][4 * tx]) = xn[q];
+  auto issue = [&](int step) {
+    const int s = step * kGradStep;
+    if (s < B) {
+      fetch(G, nout, o0, s, gs[step % kGradRing]);
+      fetch(A, nin, i0, s, xs[step % kGradRing]);
     }
-    __syncthreads();
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      gn[q] = fetch(G, nout, gq4, s + KC + ty + 16 * q, o0 + 4 * tx);
-      xn[q] = fetch(A, nin, xq4, s + KC + ty + 16 * q, i0 + 4 * tx);
-    }
+  for (int q = 0; q < kGradRing - 1; ++q) issue(q);
+  float acc[2][2] = {}, accb[2] = {};
+  for (int step = 0; step * kGradStep < B; ++step) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(kGradRing - 2) : "memory");
+    __syncthreads();  // step's samples are there; the buffer of step - 1 is free
+    issue(step + kGradRing - 1);
+    const float(*g)[kGradTile] = gs[step % kGradRing];
+    const float(*x)[kGradTile] = xs[step % kGradRing];
 #pragma unroll 8
-    for (int r = 0; r < KC; ++r) {
-      const float4 gv = *reinterpret_cast<const float4*>(&gs[r][4 * ty]);
-      const float4 xv = *reinterpret_cast<const float4*>(&xs[r][4 * tx]);
-      const float gq[4] = {gv.x, gv.y, gv.z, gv.w}, xq[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        accb[i] += gq[i];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(gq[i], xq[j], acc[i][j]);
+    for (int r = 0; r < kGradStep; ++r) {
+      const float2 gv = *reinterpret_cast<const float2*>(&g[r][2 * ty]);
+      const float2 xv = *reinterpret_cast<const float2*>(&x[r][2 * tx]);
+      acc[0][0] = fmaf(gv.x, xv.x, acc[0][0]);
+      acc[0][1] = fmaf(gv.x, xv.y, acc[0][1]);
+      acc[1][0] = fmaf(gv.y, xv.x, acc[1][0]);
+      acc[1][1] = fmaf(gv.y, xv.y, acc[1][1]);
+      if (bias) {
+        accb[0] += gv.x;
+        accb[1] += gv.y;
       }
     }
-    __syncthreads();
-  }
-  if (gridDim.y > 1) {
-    dw = ws.part + blockIdx.y * stride + at;
-    db = dw + (size_t)nout * nin;
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int o = o0 + 4 * ty + i;
+  for (int i = 0; i < 2; ++i) {
+    const int o = o0 + 2 * ty + i;
     if (o >= nout) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j)
-      if (i0 + 4 * tx + j < nin) dw[(size_t)o * nin + i0 + 4 * tx + j] = acc[i][j];
-    if (i0 == 0 && tx == 0) db[o] = accb[i];
-  }
-}
-__global__ void __launch_bounds__(256) mlp_bwd_sum(const Net net, const float* __restrict__ part, int slices,
-                                                   size_t stride, GradOut out) {
-  size_t i = blockIdx.x * 256ull + threadIdx.x;
-  if (i >= stride) return;
-  float s = 0.f;
-#pragma unroll 8
-  for (int q = 0; q < slices; ++q) s += part[q * stride + i];
-#pragma unroll
-  for (int l = 0; l < GB_MLP_LAYERS; ++l) {
-    const size_t nw = (size_t)net.dims[l + 1] * net.dims[l], nb = net.dims[l + 1];
-    if (i < nw) {
-      out.gw[l][i] = s;
-      return;
-    }
-    i -= nw;
-    if (i < nb) {
-      out.gb[l][i] = s;
-      return;
-    }
-    i -= nb;
+    for (int j = 0; j < 2; ++j)
+      if (i0 + 2 * tx + j < nin) dw[(size_t)o * nin + i0 + 2 * tx + j] = acc[i][j];
+    if (bias && tx == 0) db[o] = accb[i];
   }
 }
 
@@ -605,12 +531,7 @@ __global__ void affine_cols(float* __restrict__ X, size_t n, int cols, const flo
 
 int grid_for(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 152 * 16); }
 
-// Parameters of the network, and what the kernels need of it and of a workspace.
-size_t params(const gb_mlp* net) {
-  size_t n = 0;
-  for (int l = 0; l < GB_MLP_LAYERS; ++l) n += (size_t)net->dims[l + 1] * (net->dims[l] + 1);
-  return n;
-}
+// What the kernels need of the network and of a workspace.
 Net net_of(const gb_mlp* net) {
   Net n{};
   for (int l = 0; l <= GB_MLP_LAYERS; ++l) n.dims[l] = net->dims[l];
@@ -629,7 +550,6 @@ Acts acts_of(const gb_mlp* net, int batch, float* ws) {
     a.G[l] = ws + 2 * n;
     ws += 3 * n;
   }
-  a.part = ws;
   return a;
 }
 
@@ -652,11 +572,10 @@ gb_status gb_descriptors(const gb_matrix* m, int32_t n_atoms, const float* pos, 
 
 size_t gb_mlp_workspace_size(const gb_mlp* net, int32_t batch) {
   if (!net || batch < 1) return 0;
-  // per layer: pre-activation, activation and gradient [batch x width]; then the
-  // partial weight gradients of the batch's slices
+  // per layer: pre-activation, activation and gradient [batch x width]
   size_t tot = 0;
   for (int l = 0; l < GB_MLP_LAYERS; ++l) tot += 3 * (size_t)batch * net->dims[l + 1];
-  return (tot + mlp_slices(batch) * params(net)) * sizeof(float);
+  return tot * sizeof(float);
 }
 
 static gb_status check_net(const gb_mlp* net) {
@@ -706,12 +625,9 @@ gb_status gb_mlp_backward(const gb_mlp* net, const float* X, const float* dY, in
   for (int l = 0; l < GB_MLP_LAYERS; ++l) {
     out.gw[l] = net->gw[l];
     out.gb[l] = net->gb[l];
-    tiles += (unsigned)(((net->dims[l] + 63) / 64) * ((net->dims[l + 1] + 63) / 64));
+    tiles += (unsigned)(((net->dims[l] + kGradTile - 1) / kGradTile) * ((net->dims[l + 1] + kGradTile - 1) / kGradTile));
   }
-  const size_t stride = params(net);
-  const int slices = mlp_slices(batch);
-  mlp_bwd_w<<<dim3(tiles, (unsigned)slices), 256, 0, s>>>(n, X, dY, batch, a, out, stride);
-  if (slices > 1) mlp_bwd_sum<<<(unsigned)((stride + 255) / 256), 256, 0, s>>>(n, a.part, slices, stride, out);
+  mlp_bwd_w<<<tiles, kGradThreads, 0, s>>>(n, X, dY, batch, a, out);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return gb::fail(GB_ECUDA, "MLP backward: %s", cudaGetErrorString(e));
   return GB_OK;
