@@ -377,10 +377,34 @@ void block_factor(HostBSR* hb) {
 }
 
 // Scales and growth bounds of the mixed path's factor tiles (the tiles themselves
-// are formed from the FP64 factor on the device).
+// are formed from the FP64 factor on the device), and whether FP16 has the range for them.
+//
+// Tiles and vectors hold FP16 head / tail pairs under one power of two each: 22 bits of an
+// entry, but no finer than 2^-25 in scaled units.  Two kinds of S do not fit, and `ok` sends
+// them to the TF32 tiles, which keep an exponent per entry (the seed recurrence):
+//  - rows of different scale.  The small-scale rows of x are the large ones, so what a
+//    large-scale row loses below their floor comes back times S_ii.  Largest residual of one
+//    solve of unit vectors against TF32's (190 orbitals, every third scaled by c): c = 4 4e-7 /
+//    3e-7, 16 2e-6 / 5e-7, 100 8e-5 / 2e-6, 1000 0.2 / 1e-5.  The line: S_ii within 16 of
+//    each other (c = 4).
+//  - growth bounds far above what the vectors do.  They are products of absolute values, which
+//    grow with the number of blocks where a wide band of mixed signs does not decay block by
+//    block, and the scaled vectors sink to the floor.  lg = 8 leaves full precision to entries
+//    within 2^8 of the largest (lg in units of S's own scale; 1900 orbitals, random bands, residuals as above: lg 8 3e-7 /
+//    2e-7, 17 5e-6 / 4e-7, 33 0.2 / 6e-7, where the condition number is 19; PPV chains: 1).
+constexpr double kTileSpread = 16.0;
+constexpr int kTileGrowth = 8;
+
 FactorTiles factor_tiles(const HostBSR& hb) {
   FactorTiles f;
   if (hb.bf_bw <= 0 || hb.bf.empty()) return f;
+  double dmin = 0.0, dmax = 0.0;  // of S's diagonal
+  for (int64_t i = 0; i < hb.n; ++i) {
+    const auto b = hb.col_idx.begin() + hb.row_ptr[i], e = hb.col_idx.begin() + hb.row_ptr[i + 1];
+    const double d = hb.s_val[std::lower_bound(b, e, (int32_t)i) - hb.col_idx.begin()];
+    dmin = i == 0 ? d : std::min(dmin, d);
+    dmax = std::max(dmax, d);
+  }
   const int64_t nblk = hb.bf_nblk;
   const size_t part = (size_t)nblk * 4096;
   const double* m[4] = {hb.bf.data(), hb.bf.data() + 2 * part, hb.bf.data() + part, hb.bf.data() + 3 * part};
@@ -395,11 +419,12 @@ FactorTiles factor_tiles(const HostBSR& hb) {
       for (int k = 0; k < 64; ++k)
         for (int i = 0; i < rows; ++i) mx = std::max(mx, std::fabs(m[q][(size_t)b * 4096 + k * 64 + i]));
     }
-    std::frexp(mx > 0.0 ? mx : 1.0, &ex[q]);
+    std::frexp(mx > 0.0 && std::isfinite(mx) ? mx : 1.0, &ex[q]);
   }
   // Growth bounds: |y| <= 2^lg1 max|f| and, with y scaled by 2^-lg1, |x| <= 2^lg2 max|f|, from the
   // recursions with absolute values (r_i = |D^-1| 1 + |E| r_{i-1}, then the same backward).
   std::vector<double> r((size_t)nblk * 64), u((size_t)nblk * 64);
+  bool finite = true;
   auto bound = [&](int dir, const std::vector<double>& in, std::vector<double>& out) {
     double top = 0.0;
     for (int64_t s = 0; s < nblk; ++s) {
@@ -416,6 +441,7 @@ FactorTiles factor_tiles(const HostBSR& hb) {
       }
     }
     int lg = 0;
+    finite = finite && std::isfinite(top);
     std::frexp(top > 0.0 && std::isfinite(top) ? top : 1.0, &lg);
     return lg;
   };
@@ -424,6 +450,7 @@ FactorTiles factor_tiles(const HostBSR& hb) {
   for (auto& v : r) v = std::ldexp(v, -lg1);
   const int lg2 = bound(1, r, u);
   f.lg = lg1 + lg2;
+  f.ok = finite && f.lg + std::ilogb(dmax) <= kTileGrowth && dmax <= kTileSpread * dmin;
   f.kd[0] = (float)std::ldexp(1.0, ex[0] - 4 - lg1);  // tile entries are scaled to below 2^4
   f.ke[0] = (float)std::ldexp(1.0, ex[1] - 4);
   f.kd[1] = (float)std::ldexp(1.0, ex[2] - 4 - lg2);

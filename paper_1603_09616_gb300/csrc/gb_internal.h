@@ -44,6 +44,7 @@ void block_factor(HostBSR* hb);
 // and kd / ke undo the scaling (kd: triangular tile of either direction, with the
 // growth bound of the direction; ke: band tile; lg: both bounds' exponent).
 struct FactorTiles {
+  bool ok = false;  // FP16's range holds the tiles and the vectors (false: they are not formed)
   int ne = 0;  // 16-column steps of the band tile (0: no factor)
   int lg = 0;
   int ex[4] = {0, 0, 0, 0};

@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(256) tile_kernel(TileArgs a) {
   const double* D = a.bf + dir * a.part + (size_t)blk * 4096;
   const double* E = a.bf + (2 + dir) * a.part + (size_t)blk * 4096;
   uint32_t* fx = a.fx + (size_t)blockIdx.x * (10 + 4 * a.ne) * 256;
-  for (int e = threadIdx.x; e < (10 + 4 * a.ne) * 128; e += 256) {
+  for (int e = threadIdx.x; a.fx && e < (10 + 4 * a.ne) * 128; e += 256) {
     const int f = e >> 7, l = (e & 127) >> 2, q = e & 3;
     int mi, kk;
     if (f < 10) {
@@ -672,7 +672,7 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   const size_t o_m32 = take(sizeof(float) * nbl * 16), o_hd = take(sizeof(float) * n);
   const size_t o_bfm = take(sizeof(float) * 2 * nblk * gbk::kMmaTileFloatsDev);
   const size_t o_bft = take(sizeof(double) * 2 * nblk * gbk::kTriTile);
-  const size_t o_fx = take(sizeof(uint4) * 2 * nblk * gbk::fx_block_words(ft.ne));
+  const size_t o_fx = take(ft.ok ? sizeof(uint4) * 2 * nblk * gbk::fx_block_words(ft.ne) : 0);
   const bool dense = dense_wanted(n, nbf != 0);
   const size_t dnt = dense ? (4 * nbl + 15) / 16 : 0;
   const size_t o_di = take(sizeof(uint4) * 64 * dnt * dnt);
@@ -732,7 +732,7 @@ gb_status gb_build_bsr(int64_t n, const int64_t* row_ptr, const int32_t* col_idx
   d.bf_nblk = nbf ? (int)hb.bf_nblk : 0;
   d.bf64 = nbf ? reinterpret_cast<const double*>(b + o_bf64) : nullptr;
   d.bft = nbf ? reinterpret_cast<const double*>(b + o_bft) : nullptr;
-  d.fx = nbf ? reinterpret_cast<const uint4*>(b + o_fx) : nullptr;
+  d.fx = ft.ok ? reinterpret_cast<const uint4*>(b + o_fx) : nullptr;
   d.fx_ne = ft.ne;
   d.fx_lg = ft.lg;
   for (int q = 0; q < 2; ++q) {
@@ -916,11 +916,15 @@ void set_inner_method(const gb_matrix* m, const gb_solve_params* p, double itol,
 
 // Which recurrence solves the panels.  The real three-term recurrence
 // (panel_real.cuh) does, except where the caller names a seed shift or asks for
-// panels of one or two columns: those run the seed recurrence (panel.cuh).  The
-// FP64 correction of stagnating columns is built on it (one-column panels,
-// another seed each time), and narrow panels are how callers reproduce what it
-// corrects.
-bool real_recurrence(const gb_solve_params* p, int panel) { return p->seed_shift < 0 && panel != 1 && panel != 2; }
+// panels of one or two columns, and in the mixed path where S's factor does not fit
+// the FP16 tiles (factor_tiles): those run the seed recurrence (panel.cuh), whose
+// TF32 tiles keep an exponent per entry.  The FP64 correction of stagnating columns
+// is built on it (one-column panels, another seed each time).
+bool real_recurrence(const gb_matrix* m, const gb_solve_params* p, int panel) {
+  const bool factor = m->dm.bf_bw > 0 && !(p->flags & (kFlagCG | kFlagCheb));
+  if (p->prec == GB_MIXED && factor && !m->dm.fx) return false;
+  return p->seed_shift < 0 && panel != 1 && panel != 2;
+}
 
 // Team-workspace layout of panels of W pairs (real recurrence) or W complex
 // columns (seed recurrence).
@@ -1028,7 +1032,7 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
   // two staged factor tiles in dynamic shared memory instead
   const bool bchol = !(p->flags & (kFlagCG | kFlagCheb)) && m->dm.bf_bw > 0;
   const bool want_smem = (p->flags & kFlagSmem) != 0 && !bchol;
-  const bool f64 = p->prec == GB_FP64, real = full_hist ? verified_real : real_recurrence(p, p->panel);
+  const bool f64 = p->prec == GB_FP64, real = full_hist ? verified_real : real_recurrence(m, p, p->panel);
   auto width = [&](int cols) { return real ? std::max(1, cols / 2) : cols; };  // stored pairs or complex columns
   auto fits = [&](int w) { return want_smem && 3 * n4 * (size_t)w * cg_esz + gbk::kRedBytes <= smem_budget; };
   auto dyn_bytes = [&](int w) -> size_t {
@@ -1258,7 +1262,9 @@ __global__ void __launch_bounds__(gbk::TPB, 1)
   if (threadIdx.x < gbk::WMAX) sm.act[threadIdx.x] = threadIdx.x < a.W ? 1 : 0;
   if (threadIdx.x == 0) sm.inner_count = 0;
   __syncthreads();
-  if constexpr (sizeof(T) == 4) {
+  if (sizeof(T) == 4 && !a.m.fx) {
+    if constexpr (sizeof(T) == 4) gbk::seed_solve(a, sm, x, y, t1);
+  } else if constexpr (sizeof(T) == 4) {
     float m0 = 0.f, m1 = 0.f;
     for (int e = threadIdx.x; e < 4 * a.m.nb * a.W; e += gbk::TPB) {
       m0 = fmaxf(m0, fabsf(x[e].x));
@@ -1306,7 +1312,7 @@ gb_status gb_apply_sinv(const gb_matrix* m, gb_precision prec, int32_t w, const 
   a.W = w;
   a.inner_bchol = 1;
   a.bc_bw_alloc = m->dm.bf_bw;
-  const size_t dyn = gbk::dyn_layout(f64, w, true, 0, m->dm.bf_bw).bytes;
+  const size_t dyn = gbk::dyn_layout(f64, w, true, 0, m->dm.bf_bw, !m->dm.fx).bytes;
   if (e == cudaSuccess) {
     if (f64) {
       e = cudaFuncSetAttribute(sinv_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dyn);
@@ -1467,7 +1473,7 @@ gb_status ver_layout(const gb_matrix* m, const gb_solve_params* p, int32_t nver,
   q.nrhs = nver;
   q.rhs_cols = cols.data();
   q.panel = W;
-  gb_status st = make_plan(m, &q, true, &L->pl, true, real_recurrence(p, p->panel));
+  gb_status st = make_plan(m, &q, true, &L->pl, true, real_recurrence(m, p, p->panel));
   if (st != GB_OK) return st;
   L->W = W;
   L->pl.teams = L->pl.npanels;  // verification: every panel at once, one team each
@@ -2295,7 +2301,7 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDeviceProperties");
   const int nsm = prop.multiProcessorCount;
   bool real = true;  // one recurrence per launch
-  for (int s = 0; s < nsys; ++s) real = real && real_recurrence(&params[s], panel);
+  for (int s = 0; s < nsys; ++s) real = real && real_recurrence(mats[s], &params[s], panel);
   auto width = [&](int cols) { return real ? std::max(1, cols / 2) : cols; };
   const void* fn = batched_fn(prec == GB_FP64, real);
   // dynamic shared memory: the factor solve's buffers (systems without a
