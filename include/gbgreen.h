@@ -532,7 +532,8 @@ gb_status gb_tune_panel_batched(int32_t nsys, const gb_matrix* const* mats, cons
  *   - Problems whose scratch exceeds the array, or with nrhs > 4096, are
  *     rejected (GB_ENOMEM / GB_EINVAL) with a message naming the limit; the
  *     number of concurrent teams is reduced when that lets the problem fit
- *     (results do not depend on it).
+ *     (results do not depend on it), and with panel <= 0 narrower panels are
+ *     taken for it (of one or two columns by the seed recurrence).
  *   - Every call shares the one array and leaves its contents behind; the call
  *     re-initialises everything it reads (the work counter is cleared from
  *     the host).  Calls whose GPU work overlaps (other streams, other host

@@ -992,9 +992,10 @@ struct Plan {
   gbk::Args a;
 };
 
-// full_hist: the plan of a verification run of a solve by the recurrence `real`
+// full_hist: the plan of a verification run; recurrence: 0 the seed's, 1 the real one, else
+// real_recurrence's choice
 gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, Plan* pl, bool full_hist = false,
-                    bool verified_real = false) {
+                    int recurrence = -1) {
   if (!m) return fail(GB_EINVAL, "matrix is NULL");
   if (!p) return fail(GB_EINVAL, "params is NULL");
   if (p->nshift < 1 || p->nshift > 256) return fail(GB_EINVAL, "nshift must be in [1, 256]");
@@ -1032,7 +1033,7 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
   // two staged factor tiles in dynamic shared memory instead
   const bool bchol = !(p->flags & (kFlagCG | kFlagCheb)) && m->dm.bf_bw > 0;
   const bool want_smem = (p->flags & kFlagSmem) != 0 && !bchol;
-  const bool f64 = p->prec == GB_FP64, real = full_hist ? verified_real : real_recurrence(m, p, p->panel);
+  const bool f64 = p->prec == GB_FP64, real = recurrence < 0 ? real_recurrence(m, p, p->panel) : recurrence != 0;
   auto width = [&](int cols) { return real ? std::max(1, cols / 2) : cols; };  // stored pairs or complex columns
   auto fits = [&](int w) { return want_smem && 3 * n4 * (size_t)w * cg_esz + gbk::kRedBytes <= smem_budget; };
   auto dyn_bytes = [&](int w) -> size_t {
@@ -2118,6 +2119,18 @@ gb_status gb_shifted_solve_static(const gb_matrix* m, const gb_solve_params* p, 
   const bool want_g = out->g_proj != nullptr;
   gb_status st = make_plan(m, p, want_g, &pl);
   if (st != GB_OK) return st;
+  // The library's choice of panels for the real recurrence is made for time: room for two
+  // columns at least, and more up to one wave, and a team's records (16 K (maxit + 1) bytes a
+  // column with g_proj) grow with them.  Where they do not fit, the seed recurrence's choice of
+  // width, which starts at one column, may.
+  if (p->panel <= 0 && pl.real && align256(pl.header_bytes) + pl.team_bytes > kStaticScratchBytes) {
+    Plan alt;
+    if ((st = make_plan(m, p, want_g, &alt, false, 0)) != GB_OK) return st;
+    gb_solve_params narrow = *p;
+    narrow.panel = alt.C;
+    if ((st = make_plan(m, &narrow, want_g, &alt)) != GB_OK) return st;
+    if (alt.team_bytes < pl.team_bytes) pl = alt;
+  }
   int dev = 0;
   GB_CUDA(cudaGetDevice(&dev));
   if (dev != m->device) return fail(GB_EINVAL, "current device %d differs from the matrix's device %d", dev, m->device);
