@@ -464,7 +464,9 @@ size_t gb_wavepacket_workspace_size(const gb_matrix* m, int32_t nwp);
  * per MD step; independent chains of uneven length are this entry point's
  * unit of work).  Each system s solves (z_k S_s - H_s) x = e_j for its own shifts and columns
  * (params[s]) on its own matrix mats[s] and writes its own outputs outs[s];
- * all systems share one precision and one device.  Work items are (system,
+ * all systems share one precision and one device.  A system's own seed_shift and
+ * panel choose its recurrence, as in gb_shifted_solve (so gb_true_residual with
+ * params[s] runs the same one); a batch with both kinds takes two launches.  Work items are (system,
  * panel of `panel` columns) pairs taken from a device counter, largest systems
  * first; converged shifts and columns retire inside their panel.  panel <= 0:
  * library choice.  `workspace`: gb_batched_workspace_size bytes, 256-byte

@@ -920,10 +920,10 @@ void set_inner_method(const gb_matrix* m, const gb_solve_params* p, double itol,
 // the FP16 tiles (factor_tiles): those run the seed recurrence (panel.cuh), whose
 // TF32 tiles keep an exponent per entry.  The FP64 correction of stagnating columns
 // is built on it (one-column panels, another seed each time).
-bool real_recurrence(const gb_matrix* m, const gb_solve_params* p, int panel) {
+bool real_recurrence(const gb_matrix* m, const gb_solve_params* p) {
   const bool factor = m->dm.bf_bw > 0 && !(p->flags & (kFlagCG | kFlagCheb));
   if (p->prec == GB_MIXED && factor && !m->dm.fx) return false;
-  return p->seed_shift < 0 && panel != 1 && panel != 2;
+  return p->seed_shift < 0 && p->panel != 1 && p->panel != 2;
 }
 
 // Team-workspace layout of panels of W pairs (real recurrence) or W complex
@@ -1033,7 +1033,7 @@ gb_status make_plan(const gb_matrix* m, const gb_solve_params* p, bool want_g, P
   // two staged factor tiles in dynamic shared memory instead
   const bool bchol = !(p->flags & (kFlagCG | kFlagCheb)) && m->dm.bf_bw > 0;
   const bool want_smem = (p->flags & kFlagSmem) != 0 && !bchol;
-  const bool f64 = p->prec == GB_FP64, real = recurrence < 0 ? real_recurrence(m, p, p->panel) : recurrence != 0;
+  const bool f64 = p->prec == GB_FP64, real = recurrence < 0 ? real_recurrence(m, p) : recurrence != 0;
   auto width = [&](int cols) { return real ? std::max(1, cols / 2) : cols; };  // stored pairs or complex columns
   auto fits = [&](int w) { return want_smem && 3 * n4 * (size_t)w * cg_esz + gbk::kRedBytes <= smem_budget; };
   auto dyn_bytes = [&](int w) -> size_t {
@@ -1474,7 +1474,7 @@ gb_status ver_layout(const gb_matrix* m, const gb_solve_params* p, int32_t nver,
   q.nrhs = nver;
   q.rhs_cols = cols.data();
   q.panel = W;
-  gb_status st = make_plan(m, &q, true, &L->pl, true, real_recurrence(m, p, p->panel));
+  gb_status st = make_plan(m, &q, true, &L->pl, true, real_recurrence(m, p));
   if (st != GB_OK) return st;
   L->W = W;
   L->pl.teams = L->pl.npanels;  // verification: every panel at once, one team each
@@ -2313,8 +2313,8 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   cudaError_t e = cudaGetDeviceProperties(&prop, dev);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetDeviceProperties");
   const int nsm = prop.multiProcessorCount;
-  bool real = true;  // one recurrence per launch
-  for (int s = 0; s < nsys; ++s) real = real && real_recurrence(mats[s], &params[s], panel);
+  bool real = true;  // one recurrence per launch (batch_parts)
+  for (int s = 0; s < nsys; ++s) real = real && real_recurrence(mats[s], &params[s]);
   auto width = [&](int cols) { return real ? std::max(1, cols / 2) : cols; };
   const void* fn = batched_fn(prec == GB_FP64, real);
   // dynamic shared memory: the factor solve's buffers (systems without a
@@ -2396,41 +2396,52 @@ gb_status make_batch_plan(int32_t nsys, const gb_matrix* const* mats, const gb_s
   return GB_OK;
 }
 
-}  // namespace
-
-extern "C" {
-
-size_t gb_batched_workspace_size(int32_t nsys, const gb_matrix* const* mats, const gb_solve_params* params,
-                                 int32_t panel, int32_t want_g) {
-  clear_error();
-  BatchPlan bp;
-  std::vector<gb_outputs> fake;
-  if (want_g && nsys > 0) {
-    fake.assign(nsys, gb_outputs{});
-    for (auto& f : fake) f.g_proj = reinterpret_cast<double*>(1);
+// The systems of a batch that one launch solves.  A system's own parameters say by which
+// recurrence it is solved, alone, in any batch and when gb_true_residual runs it again; a
+// batch that holds both kinds takes two launches, one after the other in the same workspace.
+struct BatchPart {
+  BatchPlan plan;
+  std::vector<const gb_matrix*> mats;
+  std::vector<gb_solve_params> params;
+  std::vector<gb_outputs> outs;  // empty: a size query without g_proj
+};
+gb_status batch_parts(int32_t nsys, const gb_matrix* const* mats, const gb_solve_params* params,
+                      const gb_outputs* outs, int32_t panel, std::vector<BatchPart>* parts) {
+  BatchPlan whole;  // checks every argument, in the caller's numbering
+  gb_status st = make_batch_plan(nsys, mats, params, outs, panel, &whole);
+  if (st != GB_OK) return st;
+  for (const bool real : {true, false}) {
+    BatchPart part;
+    for (int s = 0; s < nsys; ++s) {
+      if (real_recurrence(mats[s], &params[s]) != real) continue;
+      part.mats.push_back(mats[s]);
+      part.params.push_back(params[s]);
+      if (outs) part.outs.push_back(outs[s]);
+    }
+    const int32_t n = (int32_t)part.mats.size();
+    if (n == 0) continue;
+    if (n == nsys)
+      part.plan = whole;
+    else if ((st = make_batch_plan(n, part.mats.data(), part.params.data(), outs ? part.outs.data() : nullptr, panel,
+                                   &part.plan)) != GB_OK)
+      return st;
+    parts->push_back(std::move(part));
   }
-  if (make_batch_plan(nsys, mats, params, want_g ? fake.data() : nullptr, panel, &bp) != GB_OK) return 0;
-  return bp.total;
+  return GB_OK;
+}
+size_t parts_total(const std::vector<BatchPart>& parts) {
+  size_t total = 0;
+  for (const BatchPart& p : parts) total = std::max(total, p.plan.total);
+  return total;
 }
 
-gb_status gb_shifted_solve_batched(int32_t nsys, const gb_matrix* const* mats, const gb_solve_params* params,
-                                   const gb_outputs* outs, int32_t panel, void* workspace, size_t workspace_bytes,
-                                   void* stream) {
-  clear_error();
-  if (!outs) return fail(GB_EINVAL, "outputs is NULL");
-  for (int i = 0; i < nsys; ++i)
-    if (check_outputs(&outs[i]) != GB_OK) return GB_EINVAL;
-  BatchPlan bp;
-  gb_status st = make_batch_plan(nsys, mats, params, outs, panel, &bp);
-  if (st != GB_OK) return st;
-  if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
-    return fail(GB_EINVAL, "workspace must be a 256-byte aligned device pointer");
-  if (workspace_bytes < bp.total) return fail(GB_ENOMEM, "workspace too small: %zu < %zu bytes", workspace_bytes, bp.total);
-  int dev = 0;
-  GB_CUDA(cudaGetDevice(&dev));
-  if (dev != mats[0]->device) return fail(GB_EINVAL, "current device differs from the matrices' device");
-  cudaStream_t s = static_cast<cudaStream_t>(stream);
-  char* wsb = static_cast<char*>(workspace);
+// One part's launch; its columns' status bits are added to *any.  Synchronous.
+gb_status run_part(const BatchPart& part, char* wsb, cudaStream_t s, int* any) {
+  const BatchPlan& bp = part.plan;
+  int nsys = (int)part.mats.size();
+  const gb_matrix* const* mats = part.mats.data();
+  const gb_solve_params* params = part.params.data();
+  const gb_outputs* outs = part.outs.data();
   std::vector<char> hdr(bp.header_bytes, 0);
   gbk::Args* desc = reinterpret_cast<gbk::Args*>(hdr.data());
   size_t off = align256(sizeof(gbk::Args) * nsys);
@@ -2539,16 +2550,56 @@ gb_status gb_shifted_solve_batched(int32_t nsys, const gb_matrix* const* mats, c
   {
     const void* fn = batched_fn(!bp.mixed, bp.real);
     GB_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bp.dyn_smem));
-    void* args[] = {&d_desc, &d_prefix, &nsys, &d_counter, &team_ws, &bp.team_bytes};
+    size_t team_bytes = bp.team_bytes;
+    void* args[] = {&d_desc, &d_prefix, &nsys, &d_counter, &team_ws, &team_bytes};
     GB_CUDA(cudaLaunchKernel(fn, dim3(bp.teams), dim3(bp.threads), args, bp.dyn_smem, s));
   }
   GB_CUDA(cudaMemcpyAsync(hdr.data(), wsb, bp.header_bytes, cudaMemcpyDeviceToHost, s));
   GB_CUDA(cudaStreamSynchronize(s));
-  int any = 0;
   for (int q = 0; q < nsys; ++q) {
     const int* hs = reinterpret_cast<const int*>(hdr.data() + o_status[q]);
-    for (int i = 0; i < params[q].nrhs; ++i) any |= hs[i];
+    for (int i = 0; i < params[q].nrhs; ++i) *any |= hs[i];
   }
+  return GB_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
+size_t gb_batched_workspace_size(int32_t nsys, const gb_matrix* const* mats, const gb_solve_params* params,
+                                 int32_t panel, int32_t want_g) {
+  clear_error();
+  std::vector<BatchPart> parts;
+  std::vector<gb_outputs> fake;
+  if (want_g && nsys > 0) {
+    fake.assign(nsys, gb_outputs{});
+    for (auto& f : fake) f.g_proj = reinterpret_cast<double*>(1);
+  }
+  if (batch_parts(nsys, mats, params, want_g ? fake.data() : nullptr, panel, &parts) != GB_OK) return 0;
+  return parts_total(parts);
+}
+
+gb_status gb_shifted_solve_batched(int32_t nsys, const gb_matrix* const* mats, const gb_solve_params* params,
+                                   const gb_outputs* outs, int32_t panel, void* workspace, size_t workspace_bytes,
+                                   void* stream) {
+  clear_error();
+  if (!outs) return fail(GB_EINVAL, "outputs is NULL");
+  for (int i = 0; i < nsys; ++i)
+    if (check_outputs(&outs[i]) != GB_OK) return GB_EINVAL;
+  std::vector<BatchPart> parts;
+  gb_status st = batch_parts(nsys, mats, params, outs, panel, &parts);
+  if (st != GB_OK) return st;
+  if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255) != 0)
+    return fail(GB_EINVAL, "workspace must be a 256-byte aligned device pointer");
+  const size_t need = parts_total(parts);
+  if (workspace_bytes < need) return fail(GB_ENOMEM, "workspace too small: %zu < %zu bytes", workspace_bytes, need);
+  int dev = 0;
+  GB_CUDA(cudaGetDevice(&dev));
+  if (dev != mats[0]->device) return fail(GB_EINVAL, "current device differs from the matrices' device");
+  int any = 0;
+  for (const BatchPart& part : parts)
+    if ((st = run_part(part, static_cast<char*>(workspace), static_cast<cudaStream_t>(stream), &any)) != GB_OK) return st;
   if (any & gbk::kStTimeout) return fail(GB_ETIMEOUT, "a bounded wait for a staged factor tile gave up");
   if (any & gbk::kStNotSPD) return fail(GB_ENOTSPD, "inner CG found S not positive definite");
   if (any & gbk::kStBreakdown) return fail(GB_EBREAKDOWN, "COCG breakdown in at least one column");
@@ -2577,8 +2628,8 @@ gb_status gb_tune_panel_batched(int32_t nsys, const gb_matrix* const* mats, cons
   *best_panel = 0;
   for (int i = 0; i < 3; ++i) {
     if (times_ms) times_ms[i] = -1.f;
-    BatchPlan bp;
-    if (make_batch_plan(nsys, mats, probe.data(), outs, cands[i], &bp) != GB_OK || bp.total > workspace_bytes)
+    std::vector<BatchPart> parts;
+    if (batch_parts(nsys, mats, probe.data(), outs, cands[i], &parts) != GB_OK || parts_total(parts) > workspace_bytes)
       continue;
     cudaEventRecord(e0, s);
     const gb_status st = gb_shifted_solve_batched(nsys, mats, probe.data(), outs, cands[i], workspace,
