@@ -36,13 +36,13 @@ constexpr int kTileBufs = 3;  // band tiles staged: two in flight ahead of the o
 constexpr unsigned kRedBytes = TPB_WIDE / 32 * NVMAX * 32 * 8;  // block_reduce's partials
 
 // Dynamic shared memory of a team (host and device agree through this):
-//   FP32 factor passes: the tensor-core layout below (mma_layout);
+//   FP32 factor passes: the tensor-core layouts below (pass_layout, mma_layout);
 //   FP64 factor chain: [partials: block_reduce's, or the chain's nks x 64 x
-//   (W+1) sums]  [y block: 64 x W];
+//   (W+1) sums]  [y block: 64 x W], in nchunk chunks of up to two columns;
 //   iterative inner solve with its vectors in shared memory: [partials] [g, d, q]
 struct DynLayout {
-  int cw, nchunk, nks, G;
-  unsigned o_red, o_ysm, o_ebuf, o_cg, bytes;
+  int nchunk, nks, G;
+  unsigned o_red, o_ysm, o_cg, bytes;
 };
 // The seed recurrence's passes (seed_passes.cuh): [S staged factor tiles][input block x 2][output
 // block x 2], blocks of 64 rows x P floats (2 W real columns, padded so that
@@ -97,44 +97,25 @@ __host__ __device__ inline PassLayout pass_layout(int W, int ne) {
 
 __host__ __device__ inline DynLayout dyn_layout(bool fp64, int W, bool bchol, unsigned cg_bytes, int bw = 63,
                                                 bool seed = false) {
-  DynLayout L;
+  DynLayout L{};
   if (bchol && !fp64) {
-    const unsigned bytes = seed ? mma_layout(W, bw).bytes : pass_layout(W, (bw + 15) / 16).bytes;
-    L.cw = L.nchunk = L.nks = L.G = 0;
-    L.o_red = L.o_ysm = 0;
-    L.o_ebuf = 0;
-    L.o_cg = bytes;
-    L.bytes = bytes;
+    L.o_cg = L.bytes = seed ? mma_layout(W, bw).bytes : pass_layout(W, (bw + 15) / 16).bytes;
     return L;
   }
-  const int RPT = fp64 ? 1 : 2, CW = fp64 ? 2 : 4;
-  const unsigned esz = fp64 ? 16u : 8u;
-  L.G = TPB / (64 / RPT);
-  L.cw = W < CW ? W : CW;
-  L.nchunk = W / L.cw;
-  // FP64 chain: slices of k.  Two give four warps even for one column, one per scheduler,
-  // which keep its FP64 pipe busy; more only add partial sums (eight: 1024 more additions
-  // a block against 1920 FMAs at a half-bandwidth of 15).
-  L.nks = L.nchunk >= L.G ? 1 : (fp64 ? 2 : L.G / L.nchunk);
-  unsigned red = kRedBytes;
-  if (bchol) {
-    const unsigned part = (unsigned)(L.nks * 64 * (W + 1)) * esz, xin = 64u * (unsigned)W * esz;
+  unsigned red = kRedBytes, y = 0;
+  if (bchol) {  // FP64 chain
+    L.G = TPB / 64;
+    L.nchunk = W / (W < 2 ? 1 : 2);
+    // Slices of k.  Two give four warps even for one column, one per scheduler, which
+    // keep its FP64 pipe busy; more only add partial sums (eight: 1024 more additions a
+    // block against 1920 FMAs at a half-bandwidth of 15).
+    L.nks = L.nchunk >= L.G ? 1 : 2;
+    y = 64u * (unsigned)W * 16u;
+    const unsigned part = (unsigned)(L.nks * 64 * (W + 1)) * 16u;
     red = red > part ? red : part;
-    red = red > xin ? red : xin;
   }
-  unsigned off = 0;
-  L.o_red = off;
-  off = (off + red + 127u) & ~127u;
-  L.o_ysm = off;
-  L.o_cg = off;
-  if (bchol) {  // FP64 chain: the y block
-    off = (off + 64u * (unsigned)W * esz + 127u) & ~127u;
-    L.o_ebuf = off;
-  } else {
-    L.o_ebuf = off;
-    off += cg_bytes;
-  }
-  L.bytes = (off + 127u) & ~127u;
+  L.o_ysm = L.o_cg = (red + 127u) & ~127u;
+  L.bytes = (L.o_cg + (bchol ? y : cg_bytes) + 127u) & ~127u;
   return L;
 }
 
@@ -192,28 +173,11 @@ __device__ __forceinline__ float2 bc_in(const float4* p, size_t e) {  // hi part
   return make_float2(v.x, v.z);
 }
 __device__ __forceinline__ double2 bc_in(const double2* p, size_t e) { return p[e]; }
-__device__ __forceinline__ void cfma(float2& acc, float m, float2 v) {
-  acc.x = fmaf(m, v.x, acc.x);
-  acc.y = fmaf(m, v.y, acc.y);
-}
 __device__ __forceinline__ void cfma(double2& acc, double m, double2 v) {
   acc.x = fma(m, v.x, acc.x);
   acc.y = fma(m, v.y, acc.y);
 }
-template <typename C>
-__device__ __forceinline__ C czero();
-template <>
-__device__ __forceinline__ float2 czero<float2>() {
-  return make_float2(0.f, 0.f);
-}
-template <>
-__device__ __forceinline__ double2 czero<double2>() {
-  return make_double2(0.0, 0.0);
-}
-__device__ __forceinline__ float2 csub_(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ double2 csub_(double2 a, double2 b) { return make_double2(a.x - b.x, a.y - b.y); }
-__device__ __forceinline__ float2 cadd_(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 cadd_(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 czero() { return make_double2(0.0, 0.0); }
 
 // ------------------------------------------------------------ triangular pass, FP64
 // The triangles of D_i^-1 and D_i^-T for a warp that owns row pairs: lane l takes the
@@ -246,7 +210,7 @@ __device__ __noinline__ void bc_tri_f64(const Args& a, const Smem& sm, const InT
     const int kmax = N4 - base;  // rows of the vector from the block on
     double2 acc[CWV], res[CWV];
 #pragma unroll
-    for (int c = 0; c < CWV; ++c) acc[c] = res[c] = czero<double2>();
+    for (int c = 0; c < CWV; ++c) acc[c] = res[c] = czero();
     int k = s0.k;
 #pragma unroll (CWV == 1 ? 4 : 2)
     for (int j = 0; j < 65; ++j, ++k) {
@@ -255,13 +219,13 @@ __device__ __noinline__ void bc_tri_f64(const Args& a, const Smem& sm, const InT
 #pragma unroll
         for (int c = 0; c < CWV; ++c) {
           res[c] = acc[c];
-          acc[c] = czero<double2>();
+          acc[c] = czero();
         }
       }
       const double m = __ldg(M + j * 32);
 #pragma unroll
       for (int c = 0; c < CWV; ++c)
-        cfma(acc[c], m, k < kmax ? bc_in(in, (size_t)(base + k) * W + c0 + c) : czero<double2>());
+        cfma(acc[c], m, k < kmax ? bc_in(in, (size_t)(base + k) * W + c0 + c) : czero());
     }
 #pragma unroll
     for (int c = 0; c < CWV; ++c) {
@@ -295,7 +259,7 @@ __device__ __noinline__ void bc_chain64(const Args& a, Smem& sm, const double* _
     const int i0 = blk_of(0);
     for (int o = tid; o < 64 * W; o += TPB) {
       const int r = o / W, c = o - r * W, row = 64 * i0 + r;
-      const C v = row < N4 ? tin[(size_t)64 * i0 * W + o] : czero<C>();
+      const C v = row < N4 ? tin[(size_t)64 * i0 * W + o] : czero();
       ysm[o] = v;
       if (row < N4 && sm.act[c]) yout[(size_t)64 * i0 * W + o] = v;
     }
@@ -311,7 +275,7 @@ __device__ __noinline__ void bc_chain64(const Args& a, Smem& sm, const double* _
     for (int m = 0; m < PF; ++m) {
       const int o = tid + m * TPB;
       const int row = 64 * i + o / W;
-      tnext[m] = (s <= nsteps && o < 64 * W && row < N4) ? tin[(size_t)64 * i * W + o] : czero<C>();
+      tnext[m] = (s <= nsteps && o < 64 * W && row < N4) ? tin[(size_t)64 * i * W + o] : czero();
     }
   };
   load_t(1);
@@ -328,7 +292,7 @@ __device__ __noinline__ void bc_chain64(const Args& a, Smem& sm, const double* _
       const int kb = kbase + ks * len, ke = min(kb + len, kbase + bw);
       C acc[CWV];
 #pragma unroll
-      for (int j = 0; j < CWV; ++j) acc[j] = czero<C>();
+      for (int j = 0; j < CWV; ++j) acc[j] = czero();
 #pragma unroll 2
       for (int k = kb; k < ke; ++k) {
         const double mv = __ldg(Mt + k * 64 + r0);
@@ -344,9 +308,9 @@ __device__ __noinline__ void bc_chain64(const Args& a, Smem& sm, const double* _
       const int o = tid + m * TPB;
       if (o >= 64 * W) break;
       const int r = o / W, c = o - r * W, row = 64 * i + r;
-      C sacc = czero<C>();
-      for (int ks = 0; ks < nks; ++ks) sacc = cadd_(sacc, red[((size_t)ks * 64 + r) * (W + 1) + c]);
-      const C y = row < N4 ? csub_(tcur[m], sacc) : czero<C>();
+      C sacc = czero();
+      for (int ks = 0; ks < nks; ++ks) sacc = cadd(sacc, red[((size_t)ks * 64 + r) * (W + 1) + c]);
+      const C y = row < N4 ? csub(tcur[m], sacc) : czero();
       ysm[o] = y;
       if (row < N4 && sm.act[c]) yout[(size_t)64 * i * W + o] = y;
     }

@@ -31,9 +31,6 @@ constexpr int NWARP = TPB / 32;
 #ifndef GB_MIN_TEAMS
 #define GB_MIN_TEAMS ((1024 / GB_TPB) > 0 ? (1024 / GB_TPB) : 1)
 #endif
-#ifndef GB_WARP_SPMM
-#define GB_WARP_SPMM 0
-#endif
 constexpr int MIN_TEAMS_PER_SM = GB_MIN_TEAMS;
 // The real recurrence's mixed teams run 512 threads, two per SM, or 1024 (the same
 // 64 registers a thread) where a launch has no more panels than SMs: its products
@@ -158,7 +155,13 @@ __device__ __forceinline__ void block_reduce_tree(double (&v)[NV], int W, RedSme
 // lanes of a warp meet in FP32 pairs and FP64 starts with one lane per warp and
 // column.  A warp's FP64 instruction holds its scheduler for 64 cycles on GB300, so
 // converting and adding in every lane cost 6000 cycles a reduction.
-__device__ __forceinline__ void acc_xor_combine(gbff::acc& a, int off);
+__device__ __forceinline__ void acc_xor_combine(gbff::acc& a, int off) {
+  const float oh = __shfl_xor_sync(0xffffffffu, a.hi, off);
+  const float oe = __shfl_xor_sync(0xffffffffu, a.err, off);
+  const gbff::ff sm = gbff::two_sum(a.hi, oh);
+  a.hi = sm.hi;
+  a.err = __fadd_rn(__fadd_rn(a.err, oe), sm.lo);
+}
 __device__ __forceinline__ void block_reduce_acc(gbff::acc d0, gbff::acc d1, int W, RedSmem& rs) {
   extern __shared__ __align__(16) double br_dyn[];
   float2* part = reinterpret_cast<float2*>(br_dyn);
@@ -447,220 +450,6 @@ __device__ __forceinline__ double2 row_d(const DevMat& m, const double* __restri
     acc.y = fma(a23.y, x3.y, acc.y);
   }
   return acc;
-}
-
-// ------------------------------------------------------------ warp-cooperative block rows
-// The 32 lanes of a warp share one block row I: lane = slot * Wp + c with Wp a
-// power of two >= W (Wp <= 32), column c = lane % Wp, and slot s = lane / Wp
-// takes the stored blocks b = b0 + s, b0 + s + S, ... (S = 32 / Wp).  Each lane
-// accumulates its share; xor shuffles over the slot bits then give every lane
-// the full row sums of its column.  Lanes with `active` false (column beyond
-// W, or a finished column) skip the loads but still take part in the shuffles.
-__device__ __forceinline__ void wbsr_row_d(const DevMat& m, const double* __restrict__ A,
-                                           const double2* __restrict__ x, int W, int Wp, int lane, int I,
-                                           bool active, double2 (&acc)[4]) {
-#pragma unroll
-  for (int r = 0; r < 4; ++r) acc[r] = make_double2(0.0, 0.0);
-  const int S = 32 / Wp, s = lane / Wp, c = lane - s * Wp;
-  if (active) {
-    const int b1 = m.blk_ptr[I + 1];
-    for (int b = m.blk_ptr[I] + s; b < b1; b += S) {
-      const int J = m.blk_col[b];
-      const double2* xr = x + (size_t)(4 * J) * W + c;
-      double2 xv[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) xv[t] = xr[(size_t)t * W];
-      const double2* ab = reinterpret_cast<const double2*>(A + (size_t)b * 16);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const double2 a01 = __ldg(ab + 2 * r), a23 = __ldg(ab + 2 * r + 1);
-        acc[r].x = fma(a01.x, xv[0].x, acc[r].x);
-        acc[r].y = fma(a01.x, xv[0].y, acc[r].y);
-        acc[r].x = fma(a01.y, xv[1].x, acc[r].x);
-        acc[r].y = fma(a01.y, xv[1].y, acc[r].y);
-        acc[r].x = fma(a23.x, xv[2].x, acc[r].x);
-        acc[r].y = fma(a23.x, xv[2].y, acc[r].y);
-        acc[r].x = fma(a23.y, xv[3].x, acc[r].x);
-        acc[r].y = fma(a23.y, xv[3].y, acc[r].y);
-      }
-    }
-  }
-  for (int off = Wp; off < 32; off <<= 1) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, off);
-      acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, off);
-    }
-  }
-}
-
-__device__ __forceinline__ void wbsr_row_f(const DevMat& m, const float* __restrict__ A,
-                                           const float2* __restrict__ x, int W, int Wp, int lane, int I,
-                                           bool active, float2 (&acc)[4]) {
-#pragma unroll
-  for (int r = 0; r < 4; ++r) acc[r] = make_float2(0.f, 0.f);
-  const int S = 32 / Wp, s = lane / Wp, c = lane - s * Wp;
-  if (active) {
-    const int b1 = m.blk_ptr[I + 1];
-    int b = m.blk_ptr[I] + s;
-    // groups of four blocks per lane: all block columns first, then every
-    // matrix and x load of the group, then the FMAs (four times the loads in
-    // flight of a block-at-a-time loop)
-    for (; b + 3 * S < b1; b += 4 * S) {
-      int J[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) J[u] = __ldg(m.blk_col + b + u * S);
-      float4 a[4][4];
-      float2 xv[4][4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float4* ab = reinterpret_cast<const float4*>(A + (size_t)(b + u * S) * 16);
-#pragma unroll
-        for (int r = 0; r < 4; ++r) a[u][r] = __ldg(ab + r);
-        const float2* xr = x + (size_t)(4 * J[u]) * W + c;
-#pragma unroll
-        for (int t = 0; t < 4; ++t) xv[u][t] = xr[(size_t)t * W];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          acc[r].x = fmaf(a[u][r].x, xv[u][0].x, acc[r].x);
-          acc[r].y = fmaf(a[u][r].x, xv[u][0].y, acc[r].y);
-          acc[r].x = fmaf(a[u][r].y, xv[u][1].x, acc[r].x);
-          acc[r].y = fmaf(a[u][r].y, xv[u][1].y, acc[r].y);
-          acc[r].x = fmaf(a[u][r].z, xv[u][2].x, acc[r].x);
-          acc[r].y = fmaf(a[u][r].z, xv[u][2].y, acc[r].y);
-          acc[r].x = fmaf(a[u][r].w, xv[u][3].x, acc[r].x);
-          acc[r].y = fmaf(a[u][r].w, xv[u][3].y, acc[r].y);
-        }
-    }
-    for (; b < b1; b += S) {
-      const int J = m.blk_col[b];
-      const float2* xr = x + (size_t)(4 * J) * W + c;
-      float2 xv[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) xv[t] = xr[(size_t)t * W];
-      const float4* ab = reinterpret_cast<const float4*>(A + (size_t)b * 16);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float4 a = __ldg(ab + r);
-        acc[r].x = fmaf(a.x, xv[0].x, acc[r].x);
-        acc[r].y = fmaf(a.x, xv[0].y, acc[r].y);
-        acc[r].x = fmaf(a.y, xv[1].x, acc[r].x);
-        acc[r].y = fmaf(a.y, xv[1].y, acc[r].y);
-        acc[r].x = fmaf(a.z, xv[2].x, acc[r].x);
-        acc[r].y = fmaf(a.z, xv[2].y, acc[r].y);
-        acc[r].x = fmaf(a.w, xv[3].x, acc[r].x);
-        acc[r].y = fmaf(a.w, xv[3].y, acc[r].y);
-      }
-    }
-  }
-  for (int off = Wp; off < 32; off <<= 1) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      acc[r].x += __shfl_xor_sync(0xffffffffu, acc[r].x, off);
-      acc[r].y += __shfl_xor_sync(0xffffffffu, acc[r].y, off);
-    }
-  }
-}
-
-// compensated sum of two accumulators held by lanes `lane` and `lane ^ off`
-__device__ __forceinline__ void acc_xor_combine(gbff::acc& a, int off) {
-  const float oh = __shfl_xor_sync(0xffffffffu, a.hi, off);
-  const float oe = __shfl_xor_sync(0xffffffffu, a.err, off);
-  const gbff::ff sm = gbff::two_sum(a.hi, oh);
-  a.hi = sm.hi;
-  a.err = __fadd_rn(__fadd_rn(a.err, oe), sm.lo);
-}
-
-// float-float matrix (hi + lo) times float-float complex vector (float4 {re.hi,
-// re.lo, im.hi, im.lo}), compensated accumulation and compensated combine.
-__device__ __forceinline__ void wbsr_row_ff(const DevMat& m, const float* __restrict__ Ahi,
-                                            const float* __restrict__ Alo, const float4* __restrict__ x, int W,
-                                            int Wp, int lane, int I, bool active, gbff::acc (&are)[4],
-                                            gbff::acc (&aim)[4]) {
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    gbff::acc_init(are[r]);
-    gbff::acc_init(aim[r]);
-  }
-  const int S = 32 / Wp, s = lane / Wp, c = lane - s * Wp;
-  if (active) {
-    const int b1 = m.blk_ptr[I + 1];
-    for (int b = m.blk_ptr[I] + s; b < b1; b += S) {
-      const int J = m.blk_col[b];
-      const float4* xr = x + (size_t)(4 * J) * W + c;
-      float4 xv[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) xv[t] = xr[(size_t)t * W];
-      const float4* ah = reinterpret_cast<const float4*>(Ahi + (size_t)b * 16);
-      const float4* al = reinterpret_cast<const float4*>(Alo + (size_t)b * 16);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float4 h = __ldg(ah + r), l = __ldg(al + r);
-        const float hv[4] = {h.x, h.y, h.z, h.w};
-        const float lv[4] = {l.x, l.y, l.z, l.w};
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const gbff::ff a = {hv[t], lv[t]};
-          gbff::acc_mul_add(are[r], a, gbff::ff{xv[t].x, xv[t].y});
-          gbff::acc_mul_add(aim[r], a, gbff::ff{xv[t].z, xv[t].w});
-        }
-      }
-    }
-  }
-  for (int off = Wp; off < 32; off <<= 1) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      acc_xor_combine(are[r], off);
-      acc_xor_combine(aim[r], off);
-    }
-  }
-}
-
-// float-float matrix times FP32 complex vector (exact in float), compensated.
-__device__ __forceinline__ void wbsr_row_ffx(const DevMat& m, const float* __restrict__ Ahi,
-                                             const float* __restrict__ Alo, const float2* __restrict__ x, int W,
-                                             int Wp, int lane, int I, bool active, gbff::acc (&are)[4],
-                                             gbff::acc (&aim)[4]) {
-#pragma unroll
-  for (int r = 0; r < 4; ++r) {
-    gbff::acc_init(are[r]);
-    gbff::acc_init(aim[r]);
-  }
-  const int S = 32 / Wp, s = lane / Wp, c = lane - s * Wp;
-  if (active) {
-    const int b1 = m.blk_ptr[I + 1];
-    for (int b = m.blk_ptr[I] + s; b < b1; b += S) {
-      const int J = m.blk_col[b];
-      const float2* xr = x + (size_t)(4 * J) * W + c;
-      float2 xv[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) xv[t] = xr[(size_t)t * W];
-      const float4* ah = reinterpret_cast<const float4*>(Ahi + (size_t)b * 16);
-      const float4* al = reinterpret_cast<const float4*>(Alo + (size_t)b * 16);
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const float4 h = __ldg(ah + r), l = __ldg(al + r);
-        const float hv[4] = {h.x, h.y, h.z, h.w};
-        const float lv[4] = {l.x, l.y, l.z, l.w};
-#pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const gbff::ff a = {hv[t], lv[t]};
-          gbff::acc_mul_add(are[r], a, xv[t].x);
-          gbff::acc_mul_add(aim[r], a, xv[t].y);
-        }
-      }
-    }
-  }
-  for (int off = Wp; off < 32; off <<= 1) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      acc_xor_combine(are[r], off);
-      acc_xor_combine(aim[r], off);
-    }
-  }
 }
 
 }  // namespace gbk

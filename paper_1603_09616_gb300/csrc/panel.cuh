@@ -190,21 +190,11 @@ __device__ void solve_panel(const Args& a, SeedSmem& sm, PanelSmemExtra& sx, cha
       gbff::acc_init(d1);
       gbff::acc_init(d2);
       gbff::acc_init(d3);
-#if GB_WARP_SPMM
-      const int lane = tid & 31;
-      const bool act = sm.act[c] != 0;
-      for (int I = tid >> 5; I < nb; I += NWARP) {
-#else
       for (int it = tid; it < nb * W; it += TPB) {
         if (!sm.act[c]) continue;
         const int I = it / W;
-#endif
         if constexpr (MIX) {
           gbff::acc are[4], aim[4];
-#if GB_WARP_SPMM
-          wbsr_row_ff(a.m, a.m.hb_hi, a.m.hb_lo, p, W, W, lane, I, act, are, aim);
-          if (lane >= W || !act) continue;
-#else
           if (a.hp_fp32) {  // unrefined FP32 product: U = H hi(p), accumulated in FP32
             float2 acc[4];
             bsr_row_fhi(a.m, a.m.hb_hi, p, W, c, I, acc);
@@ -216,7 +206,6 @@ __device__ void solve_panel(const Args& a, SeedSmem& sm, PanelSmemExtra& sx, cha
           } else {
             bsr_row_ff(a.m, a.m.hb_hi, a.m.hb_lo, p, W, c, I, are, aim);
           }
-#endif
 #pragma unroll
           for (int rr = 0; rr < 4; ++rr) {
             const size_t e = (size_t)(4 * I + rr) * W + c;
@@ -235,12 +224,7 @@ __device__ void solve_panel(const Args& a, SeedSmem& sm, PanelSmemExtra& sx, cha
           }
         } else {
           double2 acc[4];
-#if GB_WARP_SPMM
-          wbsr_row_d(a.m, a.m.hb, p, W, W, lane, I, act, acc);
-          if (lane >= W || !act) continue;
-#else
           bsr_row_d(a.m, a.m.hb, p, W, c, I, acc);
-#endif
 #pragma unroll
           for (int rr = 0; rr < 4; ++rr) {
             const size_t e = (size_t)(4 * I + rr) * W + c;
