@@ -31,10 +31,10 @@ NOMINAL_MAX_SM_MHZ = 2070.0
 # captured again.  spmm_quad_kernel<1> (FP32, one column) on the block-aligned
 # bundle Hamiltonian:
 SPMM_F32_W1_DRAM_BYTES = 271.619584e6
-# team_kernel<mixed> with the exact factor inner solve on the 1900-orbital
-# chain, bytes per column-iteration of a 60-iteration capture (84.54 GB over
-# 114,000 column-iterations), scaled to a launch by its column-iterations:
-TEAM_MIXED_DRAM_BYTES_PER_COL_ITER = 741.6e3
+# team_kernel<mixed, real recurrence> with the exact factor inner solve on the
+# 1900-orbital chain, bytes per column-iteration of a 60-iteration capture (24.25 GB
+# over 114,000 column-iterations), scaled to a launch by its column-iterations:
+TEAM_MIXED_DRAM_BYTES_PER_COL_ITER = 212.7e3
 
 
 def spmm_alg_bytes(info, v, W):
@@ -43,30 +43,40 @@ def spmm_alg_bytes(info, v, W):
     return v * info["nnz"] + 4 * info["nnzb"] + 4 * (info["nb"] + 1) + 2 * (2 * v) * info["n"] * W
 
 
-def team_alg_bytes_per_col_iter(info, W, K, mean_row, inner_per_outer, method, v=4):
-    """Algorithmic bytes the shifted COCG must move per column-iteration.
+def team_alg_bytes_per_col_iter(info, C, K, mean_row, inner_per_outer, inner, mixed):
+    """Bytes that the real recurrence reads and writes per column-iteration.
 
-    Per outer iteration of a W-column panel: the H p product; the inner solve
-    (iterative: n_in x (S product + 5 vector passes); exact factor: per level
-    the triangular blocks D^-1, D^-T and the band blocks E, F plus 8 vector
-    passes (read f, write / read t, y, u, write x), and one S product for the
-    float-float residual between the two mixed levels); the seed update (10
-    vector passes); the per-shift projected state 4 x 16 B x |R_j| x K read and
-    written plus the 16 B x |R_j| gather of r.  Divided by W.
+    A panel holds C real columns as C / 2 pairs; a pair vector takes 16 bytes a row
+    (two float-floats or two doubles), its FP32 form 8.  Per iteration of a panel:
+    the H v product (8-byte values, float-float or FP64); the update of s from three
+    vectors; the inner solve (factor: per level the tiles, FP16 pairs or FP64, and
+    eight passes over a vector, and between levels one float-float S product with
+    the residual; dense inverse: 4 bytes an element of S^-1 and four passes; iteration: an FP32 S product and
+    seven passes a step); the sum of the levels with its dot product; the shift
+    polynomials, read and written; and v on the pattern rows, written and read again
+    by the contraction.  Divided by C.
     """
     N = info["n"]
-    vec = 2 * v * N * W  # one pass over a complex panel vector
-    b = spmm_alg_bytes(info, v, W)
-    if method == "factor":
-        nblk, bw = info["factor_nblk"], info["factor_bw"]
-        factor = v * (2 * nblk * 2080 + 2 * nblk * 64 * bw)
+    W = max(1, C // 2)
+    pair, v32 = 16 * N * W, 8 * N * W
+    product = 8 * info["nnz"] + 4 * info["nnzb"] + 4 * (info["nb"] + 1)
+    b = product + 2 * pair  # U = H v
+    b += 4 * pair  # s_{n+1}
+    if inner == "factor":
+        nblk, bw, levels = info["factor_nblk"], info["factor_bw"], inner_per_outer
+        if mixed:
+            tiles = 2 * nblk * (10 + 4 * ((bw + 15) // 16)) * 16 * 16 * 4
+            b += levels * (tiles + 8 * v32) + (levels - 1) * (product + v32 + 2 * pair)
+        else:
+            b += 8 * nblk * 2 * (2080 + 64 * bw) + 8 * pair
+    elif inner == "inverse":
         levels = inner_per_outer
-        b += levels * (factor + 8 * vec) + (levels - 1) * spmm_alg_bytes(info, v, W)
+        b += levels * (4 * N * N + 4 * v32) + (levels - 1) * (product + v32 + 2 * pair)
     else:
-        b += inner_per_outer * (spmm_alg_bytes(info, v, W) + 5 * vec)
-    b += 10 * vec
-    b += W * (4 * 16 * mean_row * K + 16 * mean_row)
-    return b / W
+        b += inner_per_outer * (spmm_alg_bytes(info, 4 if mixed else 8, W) + 5 * (v32 if mixed else pair))
+    b += 2 * pair + (inner_per_outer * v32 if mixed and inner in ("factor", "inverse") else 0)
+    b += C * (K * 64 + 16 * mean_row)
+    return b / C
 
 
 def dense_peaks(torch):
@@ -271,10 +281,8 @@ def run_ours(args):
     npan = (nrhs + W - 1) // W
     it_p = np.array([iters[p * W : (p + 1) * W].max() for p in range(npan)])
     inner_per_outer = float(inner[::W].sum() / max((it_p + 1).sum(), 1))
-    method = "factor" if plan["inner"] == "factor" else "iterative"
     mean_row = float(np.mean(np.diff(system.row_ptr)[cols]))
-    bpc = team_alg_bytes_per_col_iter(info, W, K, mean_row, round(inner_per_outer) if method == "factor"
-                                      else inner_per_outer, method, v=4 if wl["prec"] == "mixed" else 8)
+    bpc = team_alg_bytes_per_col_iter(info, W, K, mean_row, inner_per_outer, plan["inner"], wl["prec"] == "mixed")
     col_iters = float(iters.sum())
     alg_bytes = bpc * col_iters  # per launch = per step
     achieved_gbs = alg_bytes / (ms_per_step / 1e3) / 1e9
@@ -314,13 +322,14 @@ def run_ours(args):
             "frac": achieved_gbs / hbm_peak,
             "traffic": TEAM_MIXED_DRAM_BYTES_PER_COL_ITER * col_iters
             if (TEAM_MIXED_DRAM_BYTES_PER_COL_ITER and wl["prec"] == "mixed" and args.workload == "ppv1900"
-                and method == "factor") else None,
+                and plan["inner"] == "factor") else None,
             "peak_source": f"{peak_src}: MEASURED_PEAKS hbm_gbs" if peak_src == "measured" else "fallback 6.8 TB/s",
             "alg_bytes_per_col_iter": bpc,
             "col_iters_per_launch": col_iters,
-            "model": "algorithmic bytes per column-iteration (H p product, inner solve, seed update, per-shift "
-                     "projected state; v = 4 B mixed / 8 B FP64, true nonzeros) x column-iterations / step time; "
-                     "the panel vectors partly hit L2, so this HBM fraction is L2-assisted",
+            "model": "bytes read and written per column-iteration of the real recurrence (H v product, update, inner "
+                     "solve, shift polynomials, pattern rows of v; true nonzeros) x column-iterations / step time; "
+                     "about two thirds of them hit a cache (traffic: DRAM), and the launch is bound by issue and the "
+                     "latency of its phases, so this is no fraction of a limit",
         },
         "clocks": clk,
     }
@@ -447,7 +456,8 @@ def measure_spmm(gbg, torch, widths=(1, 2, 4, 8, 16, 32, 64), reps=10):
     Algorithmic bytes per launch: v*nnz (values) + 4*nnzb (block columns)
     + 4*(nb+1) (block row pointers) + 2*(2v)*N*W (read X, write Y), v = 4
     (FP32) or 8 (FP64) -- true nonzeros only, so the 4x4 padding of the
-    block format counts against the kernel.  X and Y exceed L2 at these sizes
+    block format counts against the FP32 kernels; the FP64 kernel walks the
+    pattern's entries (12 bytes each, no padding).  X and Y exceed L2 at these sizes
     only together with the matrix (>= 300 MB per launch), so every launch
     streams from HBM.
     """
@@ -482,29 +492,32 @@ def measure_spmm(gbg, torch, widths=(1, 2, 4, 8, 16, 32, 64), reps=10):
             torch.cuda.synchronize()
             ms = e0.elapsed_time(e1) / reps
             alg = v * nnz + 4 * nnzb + 4 * (nb + 1) + 2 * (2 * v) * n * w
-            stored = v * 16 * nnzb + 4 * nnzb + 4 * (nb + 1) + 2 * (2 * v) * n * w
+            matrix = v * 16 * nnzb + 4 * nnzb + 4 * (nb + 1) if prec == "fp32" else 12 * nnz + 4 * (n + 1)
+            stored = matrix + 2 * (2 * v) * n * w
             flops = 4.0 * nnz * w
-            flops_padded = 4.0 * 16 * nnzb * w  # executed: every stored 4x4 entry, 2 FMA per complex column
+            # executed, 2 FMA per entry and complex column: every stored 4x4 entry (FP32), the pattern's (FP64)
+            executed = 4.0 * 16 * nnzb * w if prec == "fp32" else flops
             hbm_ms = alg / (peak * 1e9) * 1e3
-            alu_ms = flops_padded / (alu[prec] * 1e12) * 1e3
+            alu_ms = executed / (alu[prec] * 1e12) * 1e3
             bound = "hbm" if hbm_ms >= alu_ms else "alu"
             rows.append({"prec": prec, "w": w, "ms": ms, "algorithmic_bytes": int(alg), "stored_bytes": int(stored),
                          "achieved_gbs": alg / (ms / 1e3) / 1e9, "stored_gbs": stored / (ms / 1e3) / 1e9,
-                         "useful_tflops": flops / (ms / 1e3) / 1e12, "executed_tflops": flops_padded / (ms / 1e3) / 1e12,
+                         "useful_tflops": flops / (ms / 1e3) / 1e12, "executed_tflops": executed / (ms / 1e3) / 1e12,
                          "hbm_floor_ms": hbm_ms, "alu_floor_ms": alu_ms, "binding_roof": bound,
                          "frac_of_binding_roof": max(hbm_ms, alu_ms) / ms})
             del x, y
     mat.close()
     best = max((r for r in rows if r["prec"] == "fp32"), key=lambda r: r["achieved_gbs"])
     return {
-        "kernel": "spmm_kernel (gb_spmm, Y = H X)",
+        "kernel": "spmm kernels (gb_spmm, Y = H X)",
         "workload": f"bundle169 H: N={n}, nnz={nnz}, 4x4 blocks nnzb={nnzb} (fill {nnz / (16 * nnzb):.3f})",
         "bound": "hbm",
         "achieved": best["achieved_gbs"], "peak": peak, "unit": "GB/s", "frac": best["achieved_gbs"] / peak,
         "peak_source": src, "best": {"prec": best["prec"], "w": best["w"]}, "sweep": rows,
         "alu_peaks_tflops": alu,
         "alu_note": "FP64 / FP32 roofs: cuBLAS DGEMM / SGEMM (no TF32) measured in this run; the FP64 product is "
-                    "ALU-bound on GB300 (its FMA floor exceeds the HBM floor)",
+                    "ALU-bound on GB300 (its FMA floor exceeds the HBM floor); cuBLAS stays some percent below the "
+                    "FP64 pipe's rate, so its fraction can pass 1",
         "traffic": SPMM_F32_W1_DRAM_BYTES if (best["prec"], best["w"]) == ("fp32", 1) else None,
     }
 
