@@ -17,7 +17,9 @@
  * three-term recurrence in the S inner product; each shift's solution is the
  * Galerkin one, its residual a polynomial in the shift.  Calls that name a seed
  * shift or ask for panels of one or two columns build the same space by a
- * conjugate orthogonal CG (COCG) in the S-bilinear form with that seed.
+ * conjugate orthogonal CG (COCG) in the S-bilinear form with that seed, and so do
+ * mixed solves of an S whose factor does not fit the FP16 tiles of the real
+ * recurrence's inner solve (badly scaled rows, or growth bounds above 2^8).
  * S^{-1} is applied exactly by a block-bidiagonal Cholesky factor of S where
  * S's half-bandwidth is at most 63 (chains); else, in the mixed path, by the
  * dense inverse of a well-scaled S of at most 1024 orbitals; else by an inner
@@ -170,8 +172,11 @@ gb_status gb_spmm(const gb_matrix* m, int32_t which, gb_precision prec, int32_t 
  * equations, Introduction).  On its own here, for tests and timing.  X and Y:
  * device arrays of n rows x w complex columns, layout as in gb_spmm;
  * prec = GB_FP64: double, one FP64 factor solve (exact to rounding);
- * GB_MIXED: float, one FP32 factor solve on TF32 tensor cores with a
- * three-term split (no refinement: ~2e-6 relative).
+ * GB_MIXED: float, one FP32-accurate factor solve on tensor cores with a
+ * three-term split of both operands, without refinement: ~4e-7 of the solution's
+ * largest entry in the column where S is well conditioned.  FP16 pairs under one
+ * power of two per column where S_ii stay within a factor of 16 and the factor's
+ * growth bounds within 2^8; TF32 pairs, an exponent per entry, for any other S.
  * w in {1, 2, 4, 8, 16, 32}.  GB_EINVAL if the matrix has no factor (S's
  * half-bandwidth above 63).  Allocates its scratch on `stream` (stream-ordered
  * allocator) and frees it; synchronous.
@@ -193,13 +198,17 @@ typedef struct {
   gb_precision prec;     /* GB_FP64 or GB_MIXED                                  */
   double inner_tol;      /* iterative inner solve's relative residual; <= 0:
                             library default (FP64: 1e-14; mixed: 1e-7 per FP32
-                            refinement level); unused by the exact factor solve */
+                            refinement level).  Mixed factor solve: the error
+                            bound of an application, reached by its levels
+                            (dense inverse: per level of two, as an iteration);
+                            unused by the FP64 factor solve */
   int32_t panel;         /* RHS columns per panel (1..32); <= 0: auto; 1 and 2:
                             the seed recurrence                             */
   int32_t flags;         /* Inner solve S w = u.  Default: the exact
                             block-bidiagonal Cholesky solve where S's
-                            half-bandwidth is <= 63 (FP64: one solve; mixed: two
-                            FP32 solves around a float-float residual), else
+                            half-bandwidth is <= 63 (FP64: one solve; mixed: FP32
+                            solves around float-float residuals, two levels for
+                            tol >= 1e-6, three down to 1e-9, four below), else
                             (mixed, the real recurrence) the dense inverse of
                             an S of at most 1024 orbitals with max |S| max
                             |S^-1| <= 64, refined as well, else an iteration
@@ -221,8 +230,9 @@ typedef struct {
                             the correction solves, which set it themselves);
                             other bits are ignored                           */
   int32_t seed_shift;    /* index of the seed shift of the seed recurrence; < 0:
-                            the real recurrence, which has none (with panel 1
-                            or 2: the middle of the grid)                    */
+                            the real recurrence, which has none (where the seed
+                            recurrence runs all the same: the middle of the
+                            grid)                                            */
   int32_t reserved;
 } gb_solve_params;
 

@@ -1,8 +1,8 @@
 // The factor solve of the seed recurrence's mixed path (panel.cuh): FWD and BWD
-// passes with both products of a block in one step, on TF32 MMAs.  Everything
-// else runs the passes of factor_passes.cuh, which are 3 to 4 times faster; the
-// seed recurrence keeps these because where it stagnates, and so which columns
-// its correction solves again, hangs on the rounding of its inner solve.
+// passes with both products of a block in one step, on TF32 MMAs, whose operands keep
+// an exponent per entry: they take every factor, also those outside FP16's range
+// (factor_tiles), which gb_apply_sinv brings here too.  The others run the faster
+// passes of factor_passes.cuh (its header has both times).
 #pragma once
 
 namespace gbk {
