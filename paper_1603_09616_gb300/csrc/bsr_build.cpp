@@ -389,9 +389,10 @@ void block_factor(HostBSR* hb) {
 //    each other (c = 4).
 //  - growth bounds far above what the vectors do.  They are products of absolute values, which
 //    grow with the number of blocks where a wide band of mixed signs does not decay block by
-//    block, and the scaled vectors sink to the floor.  lg = 8 leaves full precision to entries
-//    within 2^8 of the largest (lg in units of S's own scale; 1900 orbitals, random bands, residuals as above: lg 8 3e-7 /
-//    2e-7, 17 5e-6 / 4e-7, 33 0.2 / 6e-7, where the condition number is 19; PPV chains: 1).
+//    block, and the scaled vectors sink to the floor.  lg = 8 (in units of S's own scale)
+//    leaves full precision to entries within 2^8 of the largest.  1900 orbitals, random bands,
+//    residuals as above: lg 8 5e-7 / 3e-7, 17 5e-6 / 4e-7, 33 0.2 / 6e-7, where the condition
+//    number is 19; PPV chains have 1.
 constexpr double kTileSpread = 16.0;
 constexpr int kTileGrowth = 8;
 
